@@ -270,20 +270,19 @@ kadabra_status kadabra_graph_info(const kadabra_graph* g, int32_t* n, int64_t* m
  * a batch or serving launch shared by several graphs runs that tier first if
  * any of them has the flag (and ignores their other flags).  It has no effect
  * together with one of the three flags above.  KADABRA_FLAG_ASYNC_SCAN makes
- * the level scans of the 4096-slot shared-memory table read every stretch of
- * at least 131 arcs inside one row with 16-byte loads (128 arcs per warp
- * load).  The library does this by itself for graphs whose CSR (forward plus
- * reverse) exceeds the device's L2, where each load waits on HBM; the flag
- * asks for it on any graph, and a shared launch takes it from any of its
- * graphs.
+ * the touch test of a level search its long rows for the other frontier's
+ * nodes instead of scanning them.  The library does this by itself for graphs
+ * whose CSR (forward plus reverse) exceeds the device's L2, where each load
+ * waits on HBM; the flag asks for it on any graph, and a shared launch takes
+ * it from any of its graphs.
  * KADABRA_FLAG_FRONTIER_SEGMENTS makes the shared-memory tables scan every
  * frontier in segments of 64 nodes, as they do for frontiers beyond their
  * frontier array (1024 nodes, 512 in the compact tier-S layout), and
  * to take at most two searched long rows per segment; it exists to test
  * those paths and only slows sampling.  KADABRA_FLAG_COMPACT_TABLES runs tier
  * S in the compact layout (the autotuner's 5-CTA setup: lists of 2048 nodes,
- * 38 levels per side) whatever the tuned setup, except with the 16-byte
- * scans, which have no compact variant.  No flag changes a result.  Returns
+ * 38 levels per side) whatever the tuned setup, except with the row
+ * searches, which have no compact variant.  No flag changes a result.  Returns
  * KADABRA_ERR_ARG for unknown bits. */
 enum {
   KADABRA_FLAG_GLOBAL_TABLES = 1,

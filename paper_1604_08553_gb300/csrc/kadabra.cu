@@ -37,12 +37,16 @@
 //     atomically).
 //   * The two backtracking walks (v -> s, w -> t) take disjoint Philox
 //     blocks, so two warps walk them at the same time.
-//   * Each warp scans a contiguous slice of the level's flattened arc range,
-//     one window of 32 arcs in flight (the next one's loads issued before
-//     the current one is processed) or, for graphs beyond the L2, with
-//     16-byte loads along long row stretches.
+//   * Each warp scans a contiguous slice of the level's flattened arc range:
+//     pass 1 with 32 * TOUCH_DEPTH arcs in flight, pass 2 in windows of 32
+//     arcs, the next one's loads issued before the current one is processed.
+//     For graphs beyond the L2, pass 1 searches long rows instead.
 //     Candidate edges are chosen in (x, y) order without a sort (quadratic
 //     ranking or a weighted radix selection).
+//   * The kernel is short of issue slots and instruction cache, not of
+//     bandwidth: loops of the sampler are not unrolled unless it says so
+//     (130 KB of code against 72 KB; 128 KB of instruction cache per SM), and
+//     what one thread does while the others wait is kept short.
 //   * A sample that outgrows its table moves on to bigger tables (tier B in
 //     shared memory, then global-memory tiers M and L) with identical
 //     results.
@@ -125,6 +129,11 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int F_CAP = 1;       // a capacity bound was hit
 constexpr int F_SIGMA = 2;     // sigma overflowed uint64
 constexpr int F_INTERNAL = 4;  // an invariant failed
+// a level's failures, kept apart from the sample's flags until the level is
+// known not to touch
+constexpr int LF_SIGMA = 1;        // a sigma overflowed uint64
+constexpr int LF_CAP = 2;          // the lists, the table or a packed sigma ran out of room
+constexpr int LF_TOUCH_SIGMA = 4;  // a candidate edge's weight overflowed uint64
 
 // ============================================================== Philox
 // Philox4x32-10, Salmon, Moraes, Dror, Shaw (SC'11): ten rounds of two
@@ -147,6 +156,12 @@ __device__ __forceinline__ uint4 philox(uint32_t k0, uint32_t k1, uint4 x) {
 __device__ __forceinline__ uint4 draw(uint64_t seed, uint32_t domain, uint64_t idx, uint32_t j) {
   return philox((uint32_t)seed, (uint32_t)(seed >> 32),
                 make_uint4((uint32_t)idx, (uint32_t)(idx >> 32), j, domain));
+}
+
+// the blocks beyond a sample's first 32 (long paths only): not inlined, the
+// sampler's code is long for the instruction caches
+__device__ __noinline__ uint4 draw_late(uint64_t seed, uint32_t domain, uint64_t idx, uint32_t j) {
+  return draw(seed, domain, idx, j);
 }
 
 // floor(U * S / 2^128) for the 128-bit block U (x least significant)
@@ -180,7 +195,7 @@ __device__ __forceinline__ int64_t kchk(int64_t i, int64_t bound, int site) {
 #endif
 
 // ============================================================== tables
-struct PiEntry {
+struct alignas(16) PiEntry {
   int32_t x, y;          // x on the expanding side, y the scanned neighbour
   unsigned long long w;  // sigma_x * sigma_y (exact; overflow flagged)
 };
@@ -202,6 +217,7 @@ struct Tables {
   int frcap;                // frontier nodes per scan segment (the frontier array's capacity)
   uint32_t* bits;           // filter of the other side's frontier (shared-memory tiers), else null
   int fwords, fshift;       //   its 32-bit words and 32 - log2(its bits)
+  struct LongRows* lr;      // long rows of the segment (shared memory; null in the compact layout)
   int* lvl;                 // [side][lo|hi][maxd+2]
   int maxd;
   PiEntry* pi;              // 2*NW segments of pcap entries (the second half is scratch)
@@ -302,6 +318,7 @@ __device__ __forceinline__ bool filter_has(const uint32_t* bits, int32_t v, int 
 // position of v's entry (its word in *wout), or -1
 __device__ __forceinline__ int tab_probe(const Tables& T, int32_t v, unsigned long long* wout) {
   uint32_t pos = hash_pos(v, T.hlog);
+#pragma unroll 1
   for (uint32_t k = 0; k <= T.hmask; ++k) {
     const unsigned long long w = T.hkv[pos];
     if (w == EMPTY) return -1;
@@ -317,6 +334,7 @@ __device__ __forceinline__ int tab_probe(const Tables& T, int32_t v, unsigned lo
 // position of v's entry, or -1
 __device__ __forceinline__ int tab_find_pos(const Tables& T, int32_t v) {
   uint32_t pos = hash_pos(v, T.hlog);
+#pragma unroll 1
   for (uint32_t k = 0; k <= T.hmask; ++k) {
     const unsigned long long w = T.hkv[pos];
     if (w == EMPTY) return -1;
@@ -329,6 +347,7 @@ __device__ __forceinline__ int tab_find_pos(const Tables& T, int32_t v) {
 // 1 = inserted at *pos_out, 0 = already present at *pos_out, -1 = table full
 __device__ __forceinline__ int tab_insert(const Tables& T, int32_t v, unsigned long long want, uint32_t* pos_out) {
   uint32_t pos = hash_pos(v, T.hlog);
+#pragma unroll 1
   for (uint32_t k = 0; k <= T.hmask; ++k) {
     unsigned long long w = T.hkv[pos];
     if (w == EMPTY) {
@@ -430,56 +449,58 @@ constexpr int LONG_CAP = KD_LONG_CAP;
 #ifndef KD_FUSE_MAX
 #define KD_FUSE_MAX 256
 #endif
-#ifndef KD_FU_RG
-#define KD_FU_RG 1  // the fused pass in tier S's beyond-L2 scan variant
+#ifndef KD_FU_CMP
+#define KD_FU_CMP 0  // the fused pass in the compact layout
 #endif
+#ifndef KD_TD
+#define KD_TD 4
+#endif
+// Pass 1: arcs per lane in flight.  Batches of 65,536 samples on the Chung-Lu
+// graph of 10^6 nodes and R-MAT scale 22 with 2, 3, 4, 6 (and 8): 4.16, 3.99,
+// 3.91, 3.88 ms and 2.45, 2.36, 2.32, 2.27 ms; the small ER graph's runs lose
+// 2 % from 4 to 6 to the longer code.
+constexpr int TOUCH_DEPTH = KD_TD;
 constexpr int FUSE_MAX = KD_FUSE_MAX;  // levels of at most this many arcs insert and test for touches in one pass
-#ifndef KD_PREFIX_WARP
-#define KD_PREFIX_WARP 1  // frontiers of at most 32 nodes: the degree prefix by one warp
-#endif
 __device__ __forceinline__ bool row_is_long(int deg, int k) {
   if (KD_MEMB_W <= 0 || k <= 0 || deg < KD_LONG_MIN) return false;
   const int lg = 32 - __clz(deg);  // bits of deg: the search steps
   return (long long)deg * 16 > (long long)k * lg * KD_MEMB_W;
 }
 
+struct LongRows {
+  int start[LONG_CAP], deg[LONG_CAP];  // row start and degree
+  uint16_t pos[LONG_CAP];              // position in the frontier segment
+};
+
 struct Ctl {
   Job job;        // the job of the current sample
-  int job_id;
   int tot_job;    // the job that tot accumulates for (-1: none)
-  long long cost[2];
-  long long stat[KADABRA_NSTAT];
+  long long stat[KADABRA_NSTAT];  // per sample; but for BT_SCANNED, adds go to the low words (32 bits hold them)
   long long tot[KADABRA_NSTAT];
   unsigned long long wsum[NW];
   unsigned long long wsum_hi[NW];
   unsigned long long u64tmp[NW];
   unsigned long long r;
-  unsigned long long sel_off;
-  int depth[2];
-  int npi[NW];
-  int scan_tmp[NW];
-  long long scan_tmp3[NW][3];
+  unsigned cost[2];   // frontier degree sums of the two roots
+  unsigned acc[2];    // degree sum of the nodes a level inserts, by level parity
+  unsigned hacc[2];   //   and its repeat discoveries
+  int scan_tmp[2][NW];
   int s, t;
   int nlist;
+  int npi;            // candidate (touch) edges found
   int flags;
-  int side;
+  int lvl_flags;      // failures of the level that is being inserted (LF_*)
+  int2 fr[2][32];     // row bounds {start, arcs} of each side's frontier, if it has at most 32 nodes
   int fside, fdepth;  // the frontier the filter in T.bits was built for (fside -1: none)
-  int nlong;           // frontier rows of the current segment searched instead of scanned
-  long long ldeg_sum;  //   and their arcs (for the work counter)
-  uint16_t lrow[LONG_CAP];  //   segment position, row start and degree of each
-  int lrs[LONG_CAP];
-  int ldeg[LONG_CAP];
-  int ecount;
-  int done;       // 0 = continue, 1 = touch, 2 = disconnected
+  int nlong;          // frontier rows of the current segment searched instead of scanned (T.lr)
+  int ecount;     // backtracking: candidates found in the previous level
   int bt_flag;    // backtracking: an invariant failed at this step
   uint4 draws[32];  // the sample's Philox blocks j = 0..31, drawn by warp 0 at its start
-  int sel_warp;
-  int pick, pick_pos;
+  int pick;
   int mode;       // backtracking: 0 = scan the row of x, 1 = scan the previous level
   int bt_x[2], bt_dx[2];     // backtracking walkers (0: v -> s, 1: w -> t): node, depth
   uint32_t bt_j[2];          //   and the next Philox block of each
-  int cv, cw;     // chosen candidate edge (v on the s side, w on the t side)
-  unsigned long long cur;
+  unsigned long long cur, k;  // the launch's running index, the sample's work index
   unsigned long long ntotal;
   // weighted radix selection (block_pick_radix; its histogram lives in the
   // frontier array, which is free while a candidate edge is chosen)
@@ -488,11 +509,17 @@ struct Ctl {
   unsigned rsel_cnt;
 };
 
+// adds to a per-sample counter (no thread waits for the sum)
+__device__ __forceinline__ void stat_add(Ctl& c, int q, unsigned x) {
+  atomicAdd(reinterpret_cast<unsigned*>(&c.stat[q]), x);
+}
+
 // ============================================================== block helpers
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 
-// exclusive scan of one int per thread; *total gets the block sum
+// exclusive scan of one int per thread; *total gets the block sum.  One
+// barrier: calls that follow each other alternate between two tmp arrays.
 __device__ __forceinline__ int block_exscan(int x, int* tmp, int* total) {
   const int lane = lane_id(), w = warp_id();
   int v = x;
@@ -510,7 +537,6 @@ __device__ __forceinline__ int block_exscan(int x, int* tmp, int* total) {
     if (i < w) wpre += t;
     tot += t;
   }
-  __syncthreads();
   *total = tot;
   return wpre + v - x;
 }
@@ -539,35 +565,10 @@ __device__ __forceinline__ unsigned long long block_inscan_u64(unsigned long lon
   return wpre + v;
 }
 
-// three block sums in one round (one pair of barriers)
-__device__ __forceinline__ void block_sum3(long long& a, long long& b, long long& d, long long (*tmp)[3]) {
-  const int lane = lane_id(), w = warp_id();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(FULL, a, o);
-    b += __shfl_xor_sync(FULL, b, o);
-    d += __shfl_xor_sync(FULL, d, o);
-  }
-  if (lane == 0) {
-    tmp[w][0] = a;
-    tmp[w][1] = b;
-    tmp[w][2] = d;
-  }
-  __syncthreads();
-  a = b = d = 0;
-#pragma unroll
-  for (int i = 0; i < NW; ++i) {
-    a += tmp[i][0];
-    b += tmp[i][1];
-    d += tmp[i][2];
-  }
-  __syncthreads();
-}
-
-
 // largest p in [0, cnt) with pr[p].x <= e (prefixes non-decreasing, pr[0].x = 0)
 __device__ __forceinline__ int frontier_pos(const int2* pr, int cnt, int e) {
   int lo = 0, hi = cnt;
+#pragma unroll 1
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (pr[mid].x <= e)
@@ -587,6 +588,7 @@ __device__ __forceinline__ int frontier_next(const int2* pr, int a, int cnt, int
     a = b;
     b = cnt;
   }
+#pragma unroll 1
   while (b - a > 1) {
     const int mid = (a + b) >> 1;
     if (pr[mid].x <= e)
@@ -599,6 +601,7 @@ __device__ __forceinline__ int frontier_next(const int2* pr, int a, int cnt, int
 
 // first position of y in the sorted row col[a, b) (b if absent)
 __device__ __forceinline__ int lower_bound_row(const int32_t* col, int a, int b, int32_t y) {
+#pragma unroll 1
   while (a < b) {
     const int mid = (a + b) >> 1;
     if (__ldg(&col[mid]) < y)
@@ -632,6 +635,7 @@ __device__ __forceinline__ void lb4_update(int& a, int& b, int s, int32_t v1, in
 // instead of fourteen dependent loads per search.
 __device__ __forceinline__ void lower_bound_rows2(const int32_t* col, int& a0, int b0, int32_t y0, int& a1, int b1,
                                                   int32_t y1) {
+#pragma unroll 1
   for (;;) {
     const bool w0 = b0 - a0 > 3, w1 = b1 - a1 > 3;
     if (!w0 && !w1) break;
@@ -650,6 +654,7 @@ __device__ __forceinline__ void lower_bound_rows2(const int32_t* col, int& a0, i
     if (w0) lb4_update(a0, b0, s0, u1, u2, u3, y0);
     if (w1) lb4_update(a1, b1, s1, v1, v2, v3, y1);
   }
+#pragma unroll 1
   while (a0 < b0 || a1 < b1) {  // at most two more rounds
     const int m0 = (a0 + b0) >> 1, m1 = (a1 + b1) >> 1;
     const bool w0 = a0 < b0, w1 = a1 < b1;
@@ -674,6 +679,7 @@ __device__ __forceinline__ void lower_bound_rows2(const int32_t* col, int& a0, i
 // fourteen dependent ones.  All lanes get the result.
 __device__ __forceinline__ int warp_lower_bound(const int32_t* col, int a, int b, int32_t y) {
   const int lane = lane_id();
+#pragma unroll 1
   while (b - a > 32) {
     const long long span = b - a;
     const int piv = a + (int)((span * lane) / 32);
@@ -703,6 +709,7 @@ __device__ __forceinline__ int block_pick(int N, unsigned long long r, Ctl& c, W
   if (tid == 0) c.pick = -1;
   __syncthreads();
   unsigned long long carry = 0;
+#pragma unroll 1
   for (int base = 0; base < N; base += NT * U) {
     unsigned long long w[U];
     unsigned long long tsum = 0;
@@ -731,22 +738,133 @@ __device__ __forceinline__ int block_pick(int N, unsigned long long r, Ctl& c, W
 }
 
 // ============================================================== one sample
-// The level scan for graphs whose CSR stays in L2: each warp takes a
-// contiguous slice of the flattened arc range and walks it in windows of 32
-// arcs, software-pipelined: the loads of the next window are issued before the
-// current window is processed, so their L2 latency overlaps its probes
-// (deeper pipelining through shared memory costs more per window than the
-// shorter L2 latency gains).  For every window position it calls f(k, ok, p, y): ok =
-// the lane holds an arc, p = frontier position of its tail, y = its head.
-// All lanes of the warp call f together, in increasing arc order (so f may
-// use warp collectives).  The warp keeps the frontier row of its current
-// window in registers; only lanes whose arc lies in a later row search the
-// frontier prefix.
-template <class F>
-__device__ __forceinline__ void scan_level_regs(const Tables& T, int fcount, int E, const int32_t* cols, int64_t ncols,
-                                                F f) {
+// Arcs per warp of a level of E arcs: whole windows of 32, so that a small
+// level issues few full windows instead of one per warp with a few lanes each.
+__device__ __forceinline__ int warp_slice(int E) {
+  return max(1, (int)(((unsigned)E + 32u * NW - 1u) / (32u * NW))) * 32;
+}
+
+// Frontier positions p[k] of the tails of arcs wb + 32 k + lane (k < D; those
+// below c1 matter), given row pcur with its start <= wb < the next row's
+// start.  Each lane takes one of the next 32 rows and sets a bit where it
+// starts; a lane's row is pcur plus the bits up to its arc.  That is one
+// shared load and a few warp reductions instead of a binary search per lane.
+// Rows without arcs share a start, and more than 32 rows may start in the
+// step: then the lanes search.
+template <int D>
+__device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcount, int wb, int c1, int (&p)[D]) {
+  const int lane = lane_id();
+  const int q = pcur + 1 + lane;
+  const int st = T.pr[KIDX(min(q, fcount), T.frcap + 1, 7)].x - wb;  // at least 1
+  const bool in = q < fcount && st < 32 * D;
+  const unsigned who = __ballot_sync(FULL, in);
+  unsigned w[D];
+  int rows = 0;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    w[k] = __reduce_or_sync(FULL, in && (st >> 5) == k ? 1u << (st & 31) : 0u);
+    rows += __popc(w[k]);
+  }
+  if (rows == __popc(who) && !(who >> 31)) {
+    int at = pcur;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      p[k] = at + __popc(w[k] & (FULL >> (31 - lane)));
+      at += __popc(w[k]);
+    }
+  } else {
+#pragma unroll 1
+    for (int k = 0; k < D; ++k) {
+      const int e = wb + 32 * k + lane;
+      const int f = e < c1 ? frontier_next(T.pr, pcur, fcount, e) : pcur;
+#pragma unroll
+      for (int j = 0; j < D; ++j)
+        if (j == k) p[j] = f;
+    }
+  }
+}
+
+// Pass 1 of a level: looks for touch arcs among its E arcs.  Each warp takes
+// a contiguous slice of the flattened arc range and walks it 32 D arcs at a
+// time, every lane with D independent loads in flight (coalesced within rows,
+// of any alignment), whether the step lies in one row or in many.  Hardly any
+// arc touches, and in the shared-memory tiers one filter load rejects most
+// heads, so a step tests its heads against the filter only; the lanes that
+// pass then probe the table together.  Calls emit(touch, x's frontier
+// position, y, y's table position and word) with all lanes of the warp, in
+// no particular order.  Bound by instruction issue (about 130 per step) and
+// by the slowest warp at the barrier after it: windows of 32 arcs with a
+// probe each, and short rows one window at a time, took 23.2 k of 74 k cycles
+// per sample on the Chung-Lu graph of 10^6 nodes, this takes 16.6 k.
+template <bool PK, int D, class EM>
+__device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount, int E, const int32_t* cols,
+                                           int64_t ncols, EM emit) {
   const int lane = lane_id(), wid = warp_id();
-  const int per = (E + NW - 1) / NW;
+  const int per = warp_slice(E);
+  const int c0 = min(E, wid * per), c1 = min(E, c0 + per);
+  if (c0 >= c1) return;
+  int pcur = frontier_pos(T.pr, fcount, c0);  // warp-uniform
+  int2 cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];  // {first arc index, row start}
+  int nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;  // first arc index of the next row
+#pragma unroll 1
+  for (int wb = c0; wb < c1; wb += 32 * D) {
+    if (nxt <= wb) {  // the next arc lies in a later row
+      pcur = frontier_next(T.pr, pcur + 1, fcount, wb);
+      cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];
+      nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;
+    }
+    int a[D];  // the arcs' places in the column array
+    if (nxt >= min(c1, wb + 32 * D)) {  // one row
+#pragma unroll
+      for (int k = 0; k < D; ++k) a[k] = cur.y + (wb - cur.x) + lane + 32 * k;
+    } else {
+      int p[D];
+      rows_of_step<D>(T, pcur, fcount, wb, c1, p);
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const int2 q = T.pr[KIDX(p[k], T.frcap + 1, 7)];
+        a[k] = q.y + (wb + 32 * k + lane - q.x);
+      }
+    }
+    int y[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      y[k] = wb + 32 * k + lane < c1 ? __ldg(&cols[KIDX((int64_t)a[k], ncols, 8)]) : 0;
+    unsigned hit = 0;  // bit k: head y[k] may touch
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      if (wb + 32 * k + lane < c1 && (!PK || filter_has(T.bits, y[k], T.fshift))) hit |= 1u << k;
+#pragma unroll 1
+    while (__any_sync(FULL, hit != 0)) {
+      bool touch = false;
+      int yy = 0, pos = -1, p = 0;
+      unsigned long long hy = 0;
+      if (hit) {
+        const int k = __ffs(hit) - 1;
+        hit &= hit - 1;
+        yy = y[0];
+#pragma unroll
+        for (int j = 1; j < D; ++j)
+          if (k == j) yy = y[j];
+        pos = tab_probe(T, yy, &hy);
+        touch = pos >= 0 && val_side(ent_val<PK>(hy)) != side;
+        if (touch) p = frontier_pos(T.pr, fcount, wb + 32 * k + lane);
+      }
+      emit(touch, p, yy, pos, hy);
+    }
+  }
+}
+
+// The level scan of pass 2: each warp walks its slice in windows of 32 arcs,
+// software-pipelined (the loads of the next window are issued before the
+// current one is processed, so their latency overlaps its probes).  For every
+// window it calls f(ok, p, y): ok = the lane holds an arc, p = frontier
+// position of its tail, y = its head.  All lanes of the warp call f together.
+template <class F>
+__device__ __forceinline__ void scan_level(const Tables& T, int fcount, int E, const int32_t* cols, int64_t ncols,
+                                           F f) {
+  const int lane = lane_id(), wid = warp_id();
+  const int per = warp_slice(E);
   const int c0 = min(E, wid * per), c1 = min(E, c0 + per);
   if (c0 >= c1) return;
   int pcur = frontier_pos(T.pr, fcount, c0);  // warp-uniform
@@ -762,135 +880,43 @@ __device__ __forceinline__ void scan_level_regs(const Tables& T, int fcount, int
       cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];
       nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;
     }
-    const int e = wb + lane;
-    if (e < c1) {
-      int2 q = cur;
-      p = pcur;
-      if (e >= nxt) {
-        p = frontier_next(T.pr, pcur + 1, fcount, e);
-        q = T.pr[KIDX(p, T.frcap + 1, 7)];
-      }
-      y = __ldg(&cols[KIDX((int64_t)q.y + (e - q.x), ncols, 8)]);
-      ok = true;
+    int2 q = cur;
+    p = pcur;
+    if (nxt < min(c1, wb + 32)) {
+      int pk[1];
+      rows_of_step<1>(T, pcur, fcount, wb, c1, pk);
+      p = pk[0];
+      q = T.pr[KIDX(p, T.frcap + 1, 7)];
     }
+    const int e = wb + lane;
+    ok = e < c1;
+    if (ok) y = __ldg(&cols[KIDX((int64_t)q.y + (e - q.x), ncols, 8)]);
   };
-  bool ok0, ok1;
-  int p0, p1, y0, y1;
-  fetch(c0, ok0, p0, y0);
-  for (int wb = c0; wb < c1; wb += 32) {
+  bool ok0 = false, ok1;
+  int p0 = 0, p1, y0 = 0, y1;
+#pragma unroll 1
+  for (int wb = c0 - 32; wb < c1; wb += 32) {  // the first round only fetches
     fetch(wb + 32, ok1, p1, y1);
-    f(0, ok0, p0, y0);
+    if (wb >= c0) f(ok0, p0, y0);
     ok0 = ok1;
     p0 = p1;
     y0 = y1;
   }
 }
 
-// The level scan for graphs whose CSR does not fit in L2 (its loads wait on
-// HBM): each warp takes a contiguous slice of the flattened arc range.  A
-// stretch of at least 131 arcs inside one row (hub rows hold most arcs of a
-// power-law graph's touching level) is read with 16-byte loads, up to
-// VEC_DEPTH of them per lane at once (128 arcs per warp load), so a hub row
-// takes a sixteenth of the dependent round trips; no lane has to find its
-// row there.  Elsewhere the warp takes windows of 32 arcs, keeping
-// the current frontier row in registers; only lanes whose arc lies in a
-// later row search the frontier prefix.  For every arc it calls f(k, ok, p,
-// y): ok = the lane holds an arc, p = frontier position of its tail, y = its
-// head.  All lanes of the warp call f together (so f may use warp
-// collectives); the arcs come in no particular order.
-#ifndef KD_VEC_DEPTH
-#define KD_VEC_DEPTH 4
-#endif
-constexpr int VEC_DEPTH = KD_VEC_DEPTH;  // 16-byte loads in flight per lane in the beyond-L2 scan
-template <class F>
-__device__ __forceinline__ void scan_level_vec(const Tables& T, int fcount, int E, const int32_t* cols, int64_t ncols,
-                                                F f) {
-  const int lane = lane_id(), wid = warp_id();
-  const int per = (E + NW - 1) / NW;
-  const int c0 = min(E, wid * per), c1 = min(E, c0 + per);
-  if (c0 >= c1) return;
-  int pcur = frontier_pos(T.pr, fcount, c0);  // warp-uniform
-  int2 cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];  // {first arc index, row start}
-  int nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;  // first arc index of the next row
-  // Each step yields a group of one to four arcs per lane (v, with ok and p
-  // for all of them); the callback is called for each in one place, so its
-  // code is inlined once.
-  int wb = c0;
-  while (wb < c1) {
-    if (nxt <= wb) {  // the next arc lies in a later row
-      pcur = frontier_next(T.pr, pcur + 1, fcount, wb);
-      cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];
-      nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;
-    }
-    const int room = min(nxt, c1) - wb;                // arcs of this row left in the slice
-    const int64_t a0 = (int64_t)cur.y + (wb - cur.x);  // address of arc wb
-    const int mis = (int)(((uintptr_t)(cols + a0) >> 2) & 3);  // 4-byte steps past a 16-byte boundary
-    int4 v[VEC_DEPTH];
-#pragma unroll
-    for (int d = 0; d < VEC_DEPTH; ++d) v[d] = make_int4(0, 0, 0, 0);
-    int nk = 1, p = pcur;
-    bool ok = false;
-    if (room >= 131 && mis == 0) {  // 128 arcs of one row (or more): 16-byte loads
-      const int nd = min(VEC_DEPTH, room >> 7);
-      const int4* src = reinterpret_cast<const int4*>(cols + KIDX(a0, ncols - 127, 8)) + lane;
-#pragma unroll
-      for (int d = 0; d < VEC_DEPTH; ++d)
-        if (d < nd) v[d] = __ldg(src + 32 * d);
-      ok = true;
-      nk = 4 * nd;
-      wb += 128 * nd;
-    } else if (room >= 131) {  // up to 3 arcs to the next 16-byte boundary
-      ok = lane < 4 - mis;
-      if (ok) v[0].x = __ldg(&cols[KIDX(a0 + lane, ncols, 8)]);
-      wb += 4 - mis;
-    } else {  // a window of 32 arcs, perhaps across rows
-      const int e = wb + lane;
-      if (e < c1) {
-        int2 q = cur;
-        if (e >= nxt) {
-          p = frontier_next(T.pr, pcur + 1, fcount, e);
-          q = T.pr[KIDX(p, T.frcap + 1, 7)];
-        }
-        v[0].x = __ldg(&cols[KIDX((int64_t)q.y + (e - q.x), ncols, 8)]);
-        ok = true;
-      }
-      wb += 32;
-    }
-#pragma unroll 1
-    for (int k = 0; k < nk; ++k) {
-      int y = 0;
-#pragma unroll
-      for (int d = 0; d < VEC_DEPTH; ++d) {
-        const int4 w = v[d];
-        if ((k >> 2) == d) y = (k & 3) == 0 ? w.x : (k & 3) == 1 ? w.y : (k & 3) == 2 ? w.z : w.w;
-      }
-      f(k & 3, ok, p, y);
-    }
-  }
-}
-
-template <bool RG, class F>
-__device__ __forceinline__ void scan_level(const Tables& T, Ctl& c, int fcount, int E, const int32_t* cols,
-                                           int64_t ncols, F f) {
-  if constexpr (RG)
-    scan_level_vec(T, fcount, E, cols, ncols, f);
-  else
-    scan_level_regs(T, fcount, E, cols, ncols, f);
-}
-
 // Weighted choice among n items held in any order, in the order of their
 // 64-bit keys (distinct): the item whose key-order prefix interval contains r.
-// Quadratic in n: each thread ranks its items against all others.
+// Quadratic in n: each thread ranks its items against all others.  c.pick
+// must be -1 before a barrier that precedes the call.
 template <class KF, class WF>
 __device__ __forceinline__ int block_pick_by_key(int n, unsigned long long r, Ctl& c, KF key, WF w) {
-  const int tid = threadIdx.x;
-  if (tid == 0) c.pick = -1;
-  __syncthreads();
-  for (int i = tid; i < n; i += NT) {
+#pragma unroll 1
+  for (int i = threadIdx.x; i < n; i += NT) {
     const unsigned long long ki = key(i);
     const unsigned long long wi = w(i);
     if (wi == 0) continue;
     unsigned long long below = 0;
+#pragma unroll 1
     for (int j = 0; j < n; ++j)
       if (key(j) < ki) below += w(j);
     if (below <= r && r - below < wi) c.pick = i;
@@ -916,7 +942,9 @@ __device__ __noinline__ int block_pick_radix(const PiEntry* buf, int n, unsigned
   const int chunk = (n + NT - 1) / NT;
   const int a = min(n, tid * chunk), b = min(n, a + chunk);
   unsigned long long fixed = 0;  // the key bytes above `shift` chosen so far
+#pragma unroll 1
   for (int shift = 56; shift >= 0; shift -= 8) {
+#pragma unroll 1
     for (int i = tid; i < 256; i += NT) {
       rhist[i] = 0ull;
       rcnt[i] = 0u;
@@ -925,6 +953,7 @@ __device__ __noinline__ int block_pick_radix(const PiEntry* buf, int n, unsigned
     int cur = -1;
     unsigned long long acc = 0;
     unsigned cnt = 0;
+#pragma unroll 1
     for (int i = a; i < b; ++i) {
       const unsigned long long k = key(i);
       if (shift < 56 && (k >> (shift + 8)) != fixed) continue;
@@ -961,6 +990,7 @@ __device__ __noinline__ int block_pick_radix(const PiEntry* buf, int n, unsigned
       const unsigned long long excl = incl - s8;
       if (excl <= r && r < incl) {
         unsigned long long below = excl;
+#pragma unroll 1
         for (int q = 0; q < 8; ++q) {
           const unsigned long long h = rhist[8 * lane + q];
           if (r < below + h) {
@@ -980,6 +1010,7 @@ __device__ __noinline__ int block_pick_radix(const PiEntry* buf, int n, unsigned
     r = c.rsel_r;
     fixed = (fixed << 8) | (unsigned long long)d;
     if (c.rsel_cnt == 1u || shift == 0) {
+#pragma unroll 1
       for (int i = tid; i < n; i += NT)
         if ((key(i) >> shift) == fixed) c.pick = i;
       __syncthreads();
@@ -1008,7 +1039,7 @@ __device__ __forceinline__ void bt_record(const SampleParams& P, const Job& J, C
 #ifndef KD_WARP_BT_ROW
 #define KD_WARP_BT_ROW 256
 #endif
-constexpr int WARP_BT_ROW = KD_WARP_BT_ROW;  // rows up to this length: the step stays with warp 0
+constexpr int WARP_BT_ROW = KD_WARP_BT_ROW;  // rows up to this length: the step stays with its warp
 
 // One warp's backtracking steps for walker `half` (0: from v towards s over
 // predecessors, 1: from w towards t over successors), from its state in
@@ -1016,63 +1047,82 @@ constexpr int WARP_BT_ROW = KD_WARP_BT_ROW;  // rows up to this length: the step
 // a warp takes comes up (left in c.bt_*[half] for the block).  The draw, the
 // candidate order and the pick are those of the block's steps: the first
 // neighbour one level closer, in row order, whose cumulative sigma exceeds r.
+// A row is read four windows of 32 at a time.
 template <bool PK>
 __device__ void bt_warp_steps(const SampleParams& P, const Job& J, const Tables& T, Ctl& c, uint64_t idx,
                               int64_t out_i, int dv, int dw, bool want_path, int half) {
   const int lane = lane_id();
   const GraphDev& G = J.g;
   int x = c.bt_x[half], dx = c.bt_dx[half];
+  if (dx <= 0) return;
   uint32_t j = c.bt_j[half];
   const int32_t* brow = half == 0 ? G.rrp : G.rp;
   const int32_t* bcol = half == 0 ? G.rci : G.ci;
+  unsigned long long sx = 0;  // sigma of x
+  {
+    const int px = tab_find_pos(T, x);
+    const unsigned long long hx = px >= 0 ? T.hkv[px] : 0ull;
+    if (px < 0 || ent_val<PK>(hx) != pack_val(half, dx)) {
+      if (lane == 0) c.bt_flag = 1;
+      return;
+    }
+    sx = ent_sig<PK>(T, hx, (uint32_t)px);
+  }
+#pragma unroll 1
   while (dx > 0) {
     const int plo = lvl_lo(T, half, dx - 1), phi = lvl_hi(T, half, dx - 1);
     const int r0 = __ldg(&brow[x]), deg = __ldg(&brow[x + 1]) - r0;
     const bool single = phi - plo == 1;
     if (!single && deg > WARP_BT_ROW) break;  // the block takes this step
-    const int px = tab_find_pos(T, x);
-    if (px < 0) {
-      if (lane == 0) c.bt_flag = 1;
-      return;
-    }
-    const unsigned long long r = below128(j < 32 ? c.draws[j] : draw(J.seed, J.domain, idx, j),
-                                          ent_sig<PK>(T, T.hkv[px], (uint32_t)px));
-    ++j;
     int y = -1, pos = -1;
     if (single) {
       // a single node one level closer: it is x's only predecessor
       y = list_node<PK>(T, plo);
+      const uint32_t q = lpos_get<PK>(T, plo);
+      sx = ent_sig<PK>(T, T.hkv[q], q);
       pos = warp_lower_bound(bcol, r0, r0 + deg, y) - r0;
     } else {
+      const unsigned long long r = below128(j < 32 ? c.draws[j] : draw_late(J.seed, J.domain, idx, j), sx);
       const uint32_t want = pack_val(half, dx - 1);
       unsigned long long carry = 0;
-      for (int base = 0; base < deg; base += 32) {
-        const int i = base + lane;
-        unsigned long long w = 0;
-        if (i < deg) {
-          const int yy = __ldg(&bcol[KIDX((int64_t)r0 + i, G.m, 12)]);
-          const int q = tab_find_pos(T, yy);
-          if (q >= 0) {
-            const unsigned long long hw = T.hkv[q];
-            if (ent_val<PK>(hw) == want) w = ent_sig<PK>(T, hw, (uint32_t)q);
-          }
-        }
-        unsigned long long inc = w;  // inclusive scan (partial sums stay below sigma(x))
+#pragma unroll 1
+      for (int base = 0; base < deg && y < 0; base += 128) {
+        int ys[4];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned long long v = __shfl_up_sync(FULL, inc, o);
-          if (lane >= o) inc += v;
+        for (int k = 0; k < 4; ++k) {
+          const int i = base + 32 * k + lane;
+          ys[k] = i < deg ? __ldg(&bcol[KIDX((int64_t)r0 + i, G.m, 12)]) : -1;
         }
-        const bool hit = w != 0 && carry + inc - w <= r && r < carry + inc;
-        const unsigned m = __ballot_sync(FULL, hit);
-        if (m) {
-          pos = base + __ffs(m) - 1;
-          break;
+#pragma unroll 1
+        for (int k = 0; k < 4 && base + 32 * k < deg; ++k) {
+          const int yy = k == 0 ? ys[0] : k == 1 ? ys[1] : k == 2 ? ys[2] : ys[3];
+          unsigned long long w = 0;
+          if (yy >= 0) {
+            unsigned long long hw = 0;
+            const int q = tab_probe(T, yy, &hw);
+            if (q >= 0 && ent_val<PK>(hw) == want) w = ent_sig<PK>(T, hw, (uint32_t)q);
+          }
+          if (!__any_sync(FULL, w != 0)) continue;
+          unsigned long long inc = w;  // inclusive scan (partial sums stay below sigma(x))
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long v = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += v;
+          }
+          const bool hit = w != 0 && carry + inc - w <= r && r < carry + inc;
+          const unsigned m = __ballot_sync(FULL, hit);
+          if (m) {
+            const int from = __ffs(m) - 1;
+            pos = base + 32 * k + from;
+            y = __shfl_sync(FULL, yy, from);
+            sx = __shfl_sync(FULL, w, from);
+            break;
+          }
+          carry += __shfl_sync(FULL, inc, 31);
         }
-        carry += __shfl_sync(FULL, inc, 31);
       }
-      if (pos >= 0) y = __ldg(&bcol[KIDX((int64_t)r0 + pos, G.m, 12)]);
     }
+    ++j;
     if (y < 0) {
       if (lane == 0) c.bt_flag = 1;
       return;
@@ -1088,33 +1138,21 @@ __device__ void bt_warp_steps(const SampleParams& P, const Job& J, const Tables&
   }
 }
 
-// The touch arcs of the long rows of a frontier segment (c.lrow.., nl of
+// The touch arcs of the long rows of a frontier segment (T.lr, nl of
 // them): item q = (row q / kother, node q % kother of the other frontier,
 // list entries [ob, ob + kother)); a thread searches two items at a time.
-// Appends them to the warp's candidate segment like the scan does (npi,
-// sigma_of as there).  All lanes of every warp call it.
+// Calls emit as touch_pass does.  All lanes of every warp call it.
 #ifdef KD_MEMB_NOINLINE
 #define KD_MEMB_ATTR __device__ __noinline__
 #else
 #define KD_MEMB_ATTR __device__ __forceinline__
 #endif
-template <bool PK>
-KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl& c, const int32_t* cols, int64_t m, int fb, int ob,
-                                   int kother, int nl, PiEntry* seg, int& npi, bool& sigma_of) {
+template <bool PK, class EM>
+KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl& c, const int32_t* cols, int64_t m, int ob,
+                                   int kother, int nl, EM emit) {
   const int lane = lane_id(), wid = warp_id();
   const long long items = (long long)nl * kother;
-  auto emit = [&](bool touch, int32_t xnode, int32_t y, unsigned long long wgt) {
-    const unsigned msk = __ballot_sync(FULL, touch);
-    if (touch) {
-      const int at = npi + __popc(msk & ((1u << lane) - 1u));
-      if (at < T.pcap) {
-        seg[at].x = xnode;
-        seg[at].y = y;
-        seg[at].w = wgt;
-      }
-    }
-    npi += __popc(msk);
-  };
+#pragma unroll 1
   for (long long qb = (long long)wid * 32; qb < items; qb += 2 * NT) {
     int r[2], a[2], e[2];
     uint32_t py[2];
@@ -1134,153 +1172,114 @@ KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl& c, const int32_t*
         py[h] = lpos_get<PK>(T, ob + yi);
         hy[h] = T.hkv[KIDX(py[h], T.hmask + 1u, 14)];
         y[h] = (int32_t)(hy[h] >> 32);
-        a[h] = c.lrs[r[h]];
-        e[h] = a[h] + c.ldeg[r[h]];
+        a[h] = T.lr->start[r[h]];
+        e[h] = a[h] + T.lr->deg[r[h]];
       }
     }
     int b0 = e[0], b1 = e[1];
     lower_bound_rows2(cols, a[0], b0, y[0], a[1], b1, y[1]);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      bool touch = false;
-      unsigned long long wgt = 0;
-      int32_t xnode = 0;
-      if (r[h] >= 0 && a[h] < e[h] && __ldg(&cols[KIDX((int64_t)a[h], m, 8)]) == y[h]) {
-        touch = true;
-        const uint32_t px = lpos_get<PK>(T, fb + c.lrow[r[h]]);
-        const unsigned long long hx = T.hkv[px];
-        const unsigned long long sx = ent_sig<PK>(T, hx, px);
-        const unsigned long long sy = ent_sig<PK>(T, hy[h], py[h]);
-        wgt = sx * sy;
-        if (__umul64hi(sx, sy) != 0ull) sigma_of = true;
-        xnode = (int32_t)(hx >> 32);
-      }
-      emit(touch, xnode, y[h], wgt);
+      const bool touch = r[h] >= 0 && a[h] < e[h] && __ldg(&cols[KIDX((int64_t)a[h], m, 8)]) == y[h];
+      emit(touch, touch ? (int)T.lr->pos[r[h]] : 0, y[h], (int)py[h], hy[h]);
     }
   }
 }
 
-// FU: small levels take the fused pass (off in the compact tier-S layout,
-// whose 48 registers it would spill)
+// One sample, from the state begin_sample and insert_roots left (warp 0's
+// insertions need no barrier: the first level's frontier is read by warp 0,
+// and the other warps read the table only after that level's first barrier).
+// FU: small levels take the fused pass.  The caller puts a barrier after it.
+//
+// What a level costs beside its arcs is barriers and the latency of the steps
+// one thread or warp takes while the others wait, so a level has as few of
+// both as its data flow allows: the search's scalars live in every thread's
+// registers (equal in all of them), counters are added without waiting for
+// the sum, and a level has one barrier after its degree prefix, one after the
+// filter if it is rebuilt, one after pass 1 and one after pass 2.  Candidate
+// edges stay in shared memory, and so do the row bounds of small frontiers.
+// With the scans above and the shorter code, batches of 65,536 samples went
+// 4.41 -> 3.37 ms on the Chung-Lu graph of 10^6 nodes (2.49 -> 1.85 G warp
+// instructions) and 2.70 -> 2.21 ms on R-MAT scale 22; a 3.4 M-node ER graph's
+// run 18.3 -> 15.4 ms.
 template <bool PK, bool RG = false, bool FU = true>
 __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, const Tables& T, Ctl& c, uint64_t idx,
                                            int64_t out_i) {
   const int tid = threadIdx.x, lane = lane_id(), wid = warp_id();
   const GraphDev& G = J.g;
 
-  // the first 32 Philox blocks of the sample ((s,t), candidate edge,
-  // backtracking steps), one per lane of warp 0, so the serial steps below
-  // only read them
-  if (wid == 0) c.draws[lane] = draw(J.seed, J.domain, idx, (uint32_t)lane);
-  __syncwarp();
-  if (tid == 0) {
-    const uint4 b0 = c.draws[0];
-    const uint64_t u = (uint64_t)b0.x | ((uint64_t)b0.y << 32);
-    const uint64_t u2 = (uint64_t)b0.z | ((uint64_t)b0.w << 32);
-    const int s = (int)__umul64hi(u, (uint64_t)G.n);
-    const int tp = (int)__umul64hi(u2, (uint64_t)(G.n - 1));
-    const int t = tp + (tp >= s ? 1 : 0);
-    c.s = s;
-    c.t = t;
-    for (int k = 0; k < KADABRA_NSTAT; ++k) c.stat[k] = 0;
-    c.stat[KADABRA_STAT_DIST] = -1;
-    c.flags = 0;
-    c.done = 0;
-    c.bt_flag = 0;
-    uint32_t ps, pt;
-    if (tab_insert(T, s, ent_word<PK>(s, pack_val(0, 0), 1ull), &ps) != 1) c.flags |= F_INTERNAL;
-    if (tab_insert(T, t, ent_word<PK>(t, pack_val(1, 0), 1ull), &pt) != 1) c.flags |= F_INTERNAL;
-    if (!PK) {
-      T.hsig[ps] = 1ull;
-      T.hsig[pt] = 1ull;
-    }
-    if (!PK) {
-      T.lnode[0] = s;
-      T.lnode[1] = t;
-    }
-    lpos_set<PK>(T, 0, ps);
-    lpos_set<PK>(T, 1, pt);
-    c.nlist = 2;
-    lvl_lo(T, 0, 0) = 0;
-    lvl_hi(T, 0, 0) = 1;
-    lvl_lo(T, 1, 0) = 1;
-    lvl_hi(T, 1, 0) = 2;
-    c.depth[0] = 0;
-    c.depth[1] = 0;
-    c.fside = -1;
-    c.nlong = 0;
-    c.ldeg_sum = 0;
-    c.cost[0] = G.rp[s + 1] - G.rp[s];
-    c.cost[1] = G.rrp[t + 1] - G.rrp[t];
-  }
-  __syncthreads();
-  if (c.flags) return;
-
   // ------------------------------------------------ bb-BFS (Sec. 4)
+  int cost0 = (int)c.cost[0], cost1 = (int)c.cost[1];  // frontier degree sums
+  int depth0 = 0, depth1 = 0;
+  int last = -1;  // the side expanded by the previous level, whose bounds end at the lists' end
+  bool touched = false;
+  int side = 0;  // the side a level expands (after the search: the side that touched)
+  int cand_at = 0, cand_cap = 0;  // where the level's candidate edges start in T.pr, and how many fit there
+  const int pi_cap = NW * T.pcap;  // candidate edges a sample may have
+#pragma unroll 1
   for (int iter = 0; iter <= 2 * T.maxd + 2; ++iter) {
-    // every thread derives the frontier from the shared state left by the
-    // previous level (stable since its closing barrier)
-    const int side = c.cost[0] <= c.cost[1] ? 0 : 1;
-    const int f0 = lvl_lo(T, side, c.depth[side]);
-    const int fcount = lvl_hi(T, side, c.depth[side]) - f0;
+    const int par = iter & 1;
+    side = cost0 <= cost1 ? 0 : 1;
+    const int E = side == 0 ? cost0 : cost1;  // the level's arcs
+    const int dcur = side == 0 ? depth0 : depth1, od = side == 0 ? depth1 : depth0;
     const int list_before = c.nlist;
-    if (tid == 0) {
-      c.side = side;
-      c.stat[KADABRA_STAT_LEVELS] += 1;
-      c.stat[KADABRA_STAT_EXPANDED] += fcount;
+    const int f0 = lvl_lo(T, side, dcur);
+    const int fcount = (side == last ? list_before : lvl_hi(T, side, dcur)) - f0;
+    // the other side's current frontier: the only nodes a touch arc reaches
+    const int ob = lvl_lo(T, 1 - side, od);
+    const int kother = (1 - side == last ? list_before : lvl_hi(T, 1 - side, od)) - ob;
+    if (tid == NT - 32) {  // a warp that waits for the first one's prefix
+      stat_add(c, KADABRA_STAT_LEVELS, 1u);
+      stat_add(c, KADABRA_STAT_EXPANDED, (unsigned)fcount);
+      stat_add(c, KADABRA_STAT_EDGES, (unsigned)E);
     }
+    if (E == 0) return;  // no arc leaves this side: s and t are not connected
+    const int dnew = dcur + 1;
     const int32_t* rowp = side == 0 ? G.rp : G.rrp;
     const int32_t* cols = side == 0 ? G.ci : G.rci;
-    // the filter of the other side's frontier for pass 1, unless it is
-    // still current (all threads)
-    auto ensure_filter = [&]() {
-      if constexpr (PK) {
-        const int os = 1 - side, od = c.depth[os];
-        if (c.fside != os || c.fdepth != od) {
-          for (int i = tid; i < T.fwords; i += NT) T.bits[i] = 0u;
-          __syncthreads();
-          for (int i = lvl_lo(T, os, od) + tid; i < lvl_hi(T, os, od); i += NT) {
-            const uint32_t h = filter_slot(list_node<PK>(T, i), T.fshift);
-            atomicOr(&T.bits[h >> 5], 1u << (h & 31));
-          }
-          __syncthreads();
-          if (tid == 0) {
-            c.fside = os;
-            c.fdepth = od;
-          }
-        }
-      }
-    };
+    const int nseg = (fcount + T.frcap - 1) / T.frcap;
+    // A level of at most FUSE_MAX arcs that cannot fill the lists skips pass
+    // 1: pass 2 then tests for touches while it inserts, and undoes its
+    // insertions if it finds one.
+    const bool fused = FU && E <= FUSE_MAX && nseg == 1 && list_before + E <= T.lcap;
+    // pass 1 uses a filter of the other side's frontier, kept while that
+    // frontier stays the same
+    const bool new_filter = PK && !fused && (c.fside != 1 - side || c.fdepth != od);
+    // Candidate edges go behind the frontier prefix in T.pr while they fit
+    // (shared-memory tiers, one segment), then to T.pi, at their running index.
+    cand_at = (fcount + 2) & ~1;
+    cand_cap = PK && nseg == 1 ? max(0, T.frcap + 1 - cand_at) / 2 : 0;
+    PiEntry* const cand = reinterpret_cast<PiEntry*>(T.pr + cand_at);
 
     // Degree prefix and row starts over frontier nodes [fb, fb + cnt) into
-    // T.pr; returns their arc count (all threads).  A frontier of more than
-    // T.frcap nodes (tier B) is scanned in segments of T.frcap: the touch
-    // test and the insertion treat a level's arcs as a set, so segments give
-    // the same result.
-    // With kother > 0 (pass 1), rows that row_is_long picks for searches of
-    // the other frontier's kother nodes go to c.lrow.. (long_cap at most:
-    // one per 32 nodes of a segment, up to LONG_CAP; c.nlong must be 0) and
-    // count 0 arcs in the prefix.
+    // T.pr.  A frontier of more than T.frcap nodes is scanned in segments of
+    // T.frcap: the touch test and the insertion treat a level's arcs as a
+    // set, so segments give the same result.
+    // With kl > 0 (pass 1), rows that row_is_long picks for searches of the
+    // other frontier's kl nodes go to T.lr (long_cap at most: one per 32
+    // nodes of a segment, up to LONG_CAP; c.nlong must be 0) and count 0
+    // arcs in the prefix.
     const int long_cap = min(LONG_CAP, max(1, T.frcap >> 5));
-    auto build_prefix = [&](int fb, int cnt, bool count_edges, int kother) {
-#if KD_PREFIX_WARP
-      if (cnt <= 32) {  // one warp: shuffles only, one barrier
+    auto take_long = [&](int deg, int kl, int seg_pos, int rs) {
+      if (RG && row_is_long(deg, kl)) {
+        const int q = atomicAdd(&c.nlong, 1);
+        if (q < long_cap) {
+          T.lr->pos[q] = (uint16_t)seg_pos;
+          T.lr->start[q] = rs;
+          T.lr->deg[q] = deg;
+          deg = 0;
+        }
+      }
+      return deg;
+    };
+    auto build_prefix = [&](int fb, int cnt, int kl, bool clear_filter) {
+      if (fcount <= 32) {  // one warp: shuffles only; the others clear the filter
         if (wid == 0) {
           int deg = 0, rs = 0;
           if (lane < cnt) {
-            const int x = KIDX(list_node<PK>(T, fb + lane), G.n, 9);
-            rs = __ldg(&rowp[x]);
-            deg = __ldg(&rowp[x + 1]) - rs;
-            if (row_is_long(deg, kother)) {
-              const int q = atomicAdd(&c.nlong, 1);
-              if (q < long_cap) {
-                c.lrow[q] = (uint16_t)lane;
-                c.lrs[q] = rs;
-                c.ldeg[q] = deg;
-                atomicAdd(reinterpret_cast<unsigned long long*>(&c.ldeg_sum), (unsigned long long)deg);
-                deg = 0;
-              }
-            }
+            const int2 b = c.fr[side][lane];  // the rows' bounds, kept when the nodes were inserted
+            rs = b.x;
+            deg = take_long(b.y, kl, lane, rs);
           }
           int v = deg;
 #pragma unroll
@@ -1289,419 +1288,392 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
             if (lane >= o) v += u;
           }
           if (lane < cnt) T.pr[KIDX(lane, T.frcap + 1, 10)] = make_int2(v - deg, rs);
-          const int tot = __shfl_sync(FULL, v, 31);
-          __syncwarp();
-          if (lane == 0) {
-            T.pr[KIDX(cnt, T.frcap + 1, 10)] = make_int2(tot, 0);
-            c.ecount = tot;
-            if (count_edges) c.stat[KADABRA_STAT_EDGES] += tot + c.ldeg_sum;
-          }
+          if (lane == cnt - 1) T.pr[KIDX(cnt, T.frcap + 1, 10)] = make_int2(v, 0);
+        } else if (PK && clear_filter) {
+          int4* b = reinterpret_cast<int4*>(T.bits);
+#pragma unroll 1
+          for (int i = tid - 32; i < T.fwords / 4; i += NT - 32) b[i] = make_int4(0, 0, 0, 0);
         }
-        __syncthreads();
-        return c.ecount;
-      }
-#endif
-      int carry = 0;
-      for (int base = 0; base < cnt; base += NT) {
-        const int i = base + tid;
-        int deg = 0, rs = 0;
-        if (i < cnt) {
-          const int x = KIDX(list_node<PK>(T, fb + i), G.n, 9);
-          rs = __ldg(&rowp[x]);
-          deg = __ldg(&rowp[x + 1]) - rs;
-          if (row_is_long(deg, kother)) {
-            const int q = atomicAdd(&c.nlong, 1);
-            if (q < long_cap) {
-              c.lrow[q] = (uint16_t)i;
-              c.lrs[q] = rs;
-              c.ldeg[q] = deg;
-              atomicAdd(reinterpret_cast<unsigned long long*>(&c.ldeg_sum), (unsigned long long)deg);
-              deg = 0;
-            }
-          }
+      } else {
+        if (PK && clear_filter) {
+          int4* b = reinterpret_cast<int4*>(T.bits);
+#pragma unroll 1
+          for (int i = tid; i < T.fwords / 4; i += NT) b[i] = make_int4(0, 0, 0, 0);
         }
-        int tot;
-        const int ex = block_exscan(deg, c.scan_tmp, &tot);
-        if (i < cnt) T.pr[KIDX(i, T.frcap + 1, 10)] = make_int2(carry + ex, rs);
-        carry += tot;
-      }
-      if (tid == 0) {
-        T.pr[KIDX(cnt, T.frcap + 1, 10)] = make_int2(carry, 0);
-        c.ecount = carry;
-        if (count_edges) c.stat[KADABRA_STAT_EDGES] += carry + c.ldeg_sum;
+        int carry = 0;
+#pragma unroll 1
+        for (int base = 0, h = 0; base < cnt; base += NT, h ^= 1) {
+          const int i = base + tid;
+          int deg = 0, rs = 0;
+          if (i < cnt) {
+            const int x = KIDX(list_node<PK>(T, fb + i), G.n, 9);
+            rs = __ldg(&rowp[x]);
+            deg = take_long(__ldg(&rowp[x + 1]) - rs, kl, i, rs);
+          }
+          int tot;
+          const int ex = block_exscan(deg, c.scan_tmp[h], &tot);
+          if (i < cnt) T.pr[KIDX(i, T.frcap + 1, 10)] = make_int2(carry + ex, rs);
+          carry += tot;
+        }
+        if (tid == 0) T.pr[KIDX(cnt, T.frcap + 1, 10)] = make_int2(carry, 0);
       }
       __syncthreads();
-      return c.ecount;
     };
-    const int nseg = (fcount + T.frcap - 1) / T.frcap;
-    int E = 0;  // arc count of the last segment built
 
-    // pass 1: touch test against the other search.  A level of at most
-    // FUSE_MAX arcs that cannot fill the lists skips it: pass 2 then tests
-    // for touches while it inserts, and undoes its insertions if it finds one.
-    int pass1_bad = 0;
-    bool had_long = false;  // pass 1 searched rows that pass 2 must scan
-    bool fused = false;
-    {
-      int npi = 0;
-      bool sigma_of = false;
-      PiEntry* seg = T.pi + (size_t)wid * T.pcap;
-      // appends the warp's touch arcs (x, y) of weight sigma_x * sigma_y
-      auto emit = [&](bool touch, int32_t xnode, int32_t y, unsigned long long wgt) {
-        const unsigned m = __ballot_sync(FULL, touch);
-        if (touch) {
-          const int at = npi + __popc(m & ((1u << lane) - 1u));
-          if (at < T.pcap) {
-            seg[at].x = xnode;
-            seg[at].y = y;
-            seg[at].w = wgt;
-          }
-        }
-        npi += __popc(m);
-      };
-      // the other side's current frontier: the only nodes a touch arc reaches
-      const int ob = lvl_lo(T, 1 - side, c.depth[1 - side]);
-      const int kother = lvl_hi(T, 1 - side, c.depth[1 - side]) - ob;
-      for (int sg = 0; sg < nseg; ++sg) {
-      const int fb = f0 + sg * T.frcap, cnt = min(T.frcap, fcount - sg * T.frcap);
-      E = build_prefix(fb, cnt, true, RG ? kother : 0);
-      if (FU && nseg == 1 && c.nlong == 0 && E <= FUSE_MAX && c.nlist + E <= T.lcap) {
-        fused = true;
-        break;
-      }
-      ensure_filter();
-      scan_level<RG>(T, c, cnt, E, cols, G.m, [&](int, bool ok, int p, int y) {
-        bool touch = false;
-        unsigned long long wgt = 0;
-        int32_t xnode = 0;
-        if (ok && (!PK || filter_has(T.bits, y, T.fshift))) {
-          unsigned long long hy = 0;
-          const int pos = tab_probe(T, y, &hy);
-          if (pos >= 0 && val_side(ent_val<PK>(hy)) != side) {
-            touch = true;
-            const uint32_t px = lpos_get<PK>(T, fb + p);
-            const unsigned long long hx = T.hkv[px];
-            const unsigned long long sx = ent_sig<PK>(T, hx, px);
-            const unsigned long long sy = ent_sig<PK>(T, hy, (uint32_t)pos);
-            wgt = sx * sy;
-            if (__umul64hi(sx, sy) != 0ull) sigma_of = true;
-            xnode = (int32_t)(hx >> 32);
-          }
-        }
-        emit(touch, xnode, y, wgt);
-      });
-      // the long rows: one search per (row, other-frontier node)
-      if constexpr (RG) {
-        const int nl = min(c.nlong, long_cap);
-        if (nl > 0) {
-          had_long = true;
-          search_long_rows<PK>(T, c, cols, G.m, fb, ob, kother, nl, seg, npi, sigma_of);
-        }
-      }
-      if (sg + 1 < nseg) {
-        __syncthreads();  // the next segment's prefix overwrites T.pr and the long rows
-        if (tid == 0) {
-          c.nlong = 0;
-          c.ldeg_sum = 0;
-        }
-        __syncthreads();
-      }
-      }
-      if (!fused) {
-        int bad = 0;
-        if (__any_sync(FULL, sigma_of) && lane == 0) {
-          atomicOr(&c.flags, F_SIGMA);
-          bad = 1;
-        }
-        if (lane == 0) {
-          c.npi[wid] = npi;
-          if (npi > T.pcap) {
-            atomicOr(&c.flags, F_CAP);
-            bad = 1;
-          }
-        }
-        // Decide from the barrier's own reduction, not by reading c.flags
-        // after it: a warp that has already moved on may set flags (the depth
-        // limit below, or pass 2) before a slower warp would have read them,
-        // and the two would then leave at different barriers.
-        pass1_bad = __syncthreads_or(bad);
-      }
-    }
-    if (!fused) {
-      if (tid == 0) {
-        int tot = 0;
-        for (int w = 0; w < NW; ++w) tot += c.npi[w];
-        if (tot > 0) {
-          c.done = 1;
-          c.stat[KADABRA_STAT_PI] = tot;
-        }
-      }
-      __syncthreads();
-      if (tid == 0) {  // every thread has passed its last read of the long rows
-        c.nlong = 0;
-        c.ldeg_sum = 0;
-      }
-      if (pass1_bad) return;
-      if (c.done) break;
-    }
-
-    // pass 2: the next level.  The first discoverer of an unvisited head y
-    // publishes (y, side, dist) with one CAS and appends y to the level
-    // list; every discoverer adds sigma_x to the sigma field of y's hash
-    // entry (zero until then), so the order of discoveries does not matter.
-    const int dnew = c.depth[side] + 1;
-    if (dnew > T.maxd) {
-      if (tid == 0) c.flags |= F_CAP;
-      __syncthreads();
-      return;
-    }
-    long long hits = 0, fresh = 0, cost = 0;
-    {
-      bool of = false, cap = false;
-      const uint32_t want_val = pack_val(side, dnew);
-      const volatile int* nlist_now = &c.nlist;
-      int ftouch = 0;  // fused level: 1 = a touch arc seen, 2 = its weight overflowed
-      PiEntry* fseg = T.pi + (size_t)wid * T.pcap;
-      if (fused) {
-        if (lane == 0) c.npi[wid] = 0;
-        __syncwarp();
-      }
-      for (int sg = 0; sg < nseg; ++sg) {
-      const int fb = f0 + sg * T.frcap, cnt = min(T.frcap, fcount - sg * T.frcap);
-      // one segment without long rows: pass 1's prefix is still there
-      if (nseg > 1 || had_long) E = build_prefix(fb, cnt, false, 0);
-      scan_level<RG>(T, c, cnt, E, cols, G.m, [&](int, bool ok, int p, int y) {
-        if (!ok || (cap && !fused)) return;
-        // the head's row bounds (its degree joins the new frontier's cost if
-        // it is new), loaded before the probe so the load overlaps it
-        const int ylo = __ldg(&rowp[KIDX(y, G.n, 13)]), yhi = __ldg(&rowp[KIDX(y, G.n, 13) + 1]);
+    // appends a warp's touch arcs (frontier position p, head y at table
+    // position pos with word hy) with weight sigma_x * sigma_y
+    bool sigma_of = false;
+    auto emit = [&](int fb, bool touch, int p, int y, int pos, unsigned long long hy) {
+      const unsigned m = __ballot_sync(FULL, touch);
+      if (m == 0) return;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&c.npi, __popc(m));
+      at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (touch) {
         const uint32_t px = lpos_get<PK>(T, fb + p);
-        const unsigned long long add = ent_sig<PK>(T, T.hkv[px], px);
-        uint32_t pos = hash_pos(y, T.hlog);
-        for (uint32_t k = 0; k <= T.hmask; ++k) {
-          unsigned long long w = T.hkv[pos];
-          if (w == EMPTY) {
-            // stop inserting once the lists are full, so the table never
-            // fills beyond lcap + NT keys and probes stay short
-            if (*nlist_now >= T.lcap) {
-              cap = true;
-              return;
-            }
-            const unsigned long long want = ent_word<PK>(y, want_val, PK ? add : 0ull);
-            const unsigned long long old = atomicCAS(&T.hkv[pos], EMPTY, want);
-            if (old == EMPTY) {
-              const int slot = atomicAdd(&c.nlist, 1);
-              if (slot >= T.lcap) {
-                cap = true;
-                return;
-              }
-              if (!PK) T.lnode[slot] = y;
-              lpos_set<PK>(T, slot, pos);
-              ++fresh;
-              cost += yhi - ylo;
-              if (!PK && !ent_add<PK>(T, pos, add)) of = true;
-              return;
-            }
-            w = old;
-          }
-          if ((int32_t)(w >> 32) == y) {
-            const uint32_t v = ent_val<PK>(w);
-            if (v == want_val) {  // also discovered at this level
-              ++hits;
-              if (!ent_add<PK>(T, pos, add)) {
-                if (PK)
-                  cap = true;  // sigma outgrew the packed field
-                else
-                  of = true;
-              }
-            } else if (fused && val_side(v) != side) {  // a touch arc (x, y)
-              const unsigned long long sy = ent_sig<PK>(T, w, pos);
-              if (__umul64hi(add, sy) != 0ull) ftouch |= 2;
-              const int at = atomicAdd(&c.npi[wid], 1);
-              if (at < T.pcap) {
-                fseg[at].x = (int32_t)(T.hkv[px] >> 32);
-                fseg[at].y = y;
-                fseg[at].w = add * sy;
-              }
-              ftouch |= 1;
-            }
-            return;
-          }
-          pos = (pos + 1) & T.hmask;
-        }
-        cap = true;  // table full
-      });
-      if (sg + 1 < nseg) __syncthreads();
+        const unsigned long long hx = T.hkv[px];
+        const unsigned long long sx = ent_sig<PK>(T, hx, px), sy = ent_sig<PK>(T, hy, (uint32_t)pos);
+        if (!PK && __umul64hi(sx, sy) != 0ull) sigma_of = true;
+        PiEntry e;
+        e.x = (int32_t)(hx >> 32);
+        e.y = y;
+        e.w = sx * sy;
+        if (at < cand_cap)
+          cand[at] = e;
+        else if (at < pi_cap)
+          T.pi[at] = e;
       }
-      if (fused && __syncthreads_or(ftouch & 1)) {
+    };
+
+    // Pass 1 is the touch test against the other search.  Pass 2 makes the
+    // next level: the first discoverer of an unvisited head y publishes (y,
+    // side, dist) with one CAS and appends y to the level list; every
+    // discoverer adds sigma_x to the sigma field of y's hash entry (zero
+    // until then), so the order of discoveries does not matter.  (One loop
+    // over both, so that the prefix is built at one place in the code: the
+    // kernel is long for the instruction caches.)
+    bool had_long = false;  // pass 1 searched rows that pass 2 must scan
+    int Eseg = E;           // arcs of the segment in T.pr
+    unsigned hits = 0, cost = 0;
+    bool of = false, cap = false;
+    const uint32_t want_val = pack_val(side, dnew);
+    const volatile int* nlist_now = &c.nlist;
+#pragma unroll 1
+    for (int pass = fused ? 2 : 1; pass <= 2; ++pass) {
+      if (pass == 2 && dnew > T.maxd) {
+        if (tid == 0) c.flags |= F_CAP;
+        return;
+      }
+#pragma unroll 1
+      for (int sg = 0; sg < nseg; ++sg) {
+        const int fb = f0 + sg * T.frcap, cnt = min(T.frcap, fcount - sg * T.frcap);
+        // pass 2, one segment without long rows: pass 1's prefix is still there
+        if (pass == 1 || fused || nseg > 1 || had_long) {
+          const bool nf = new_filter && pass == 1 && sg == 0;
+          build_prefix(fb, cnt, RG && pass == 1 ? kother : 0, nf);
+          if (PK && nf) {
+#pragma unroll 1
+            for (int i = ob + tid; i < ob + kother; i += NT) {
+              const uint32_t h = filter_slot(list_node<PK>(T, i), T.fshift);
+              atomicOr(&T.bits[h >> 5], 1u << (h & 31));
+            }
+            if (tid == 0) {
+              c.fside = 1 - side;
+              c.fdepth = od;
+            }
+            __syncthreads();
+          }
+          Eseg = T.pr[cnt].x;
+        }
+        if (pass == 1) {
+          touch_pass<PK, TOUCH_DEPTH>(
+              T, side, cnt, Eseg, cols, G.m,
+              [&](bool touch, int p, int y, int pos, unsigned long long hy) { emit(fb, touch, p, y, pos, hy); });
+          // the long rows: one search per (row, other-frontier node)
+          if constexpr (RG) {
+            const int nl = min(c.nlong, long_cap);
+            if (nl > 0) {
+              had_long = true;
+              search_long_rows<PK>(
+                  T, c, cols, G.m, ob, kother, nl,
+                  [&](bool touch, int p, int y, int pos, unsigned long long hy) { emit(fb, touch, p, y, pos, hy); });
+            }
+          }
+        } else {
+          scan_level(T, cnt, Eseg, cols, G.m, [&](bool ok, int p, int y) {
+            int res = 0;  // 1 = inserted, 2 = a touch arc (fused)
+            int ydeg = 0, ylo = 0;
+            uint32_t pos = 0;
+            unsigned long long add = 0, w = 0;
+            if (ok && (fused || !cap)) {
+              // the head's row bounds (its degree joins the new frontier's cost
+              // if it is new), loaded before the probe so the load overlaps it
+              ylo = __ldg(&rowp[KIDX(y, G.n, 13)]);
+              const int yhi = __ldg(&rowp[KIDX(y, G.n, 13) + 1]);
+              const uint32_t px = lpos_get<PK>(T, fb + p);
+              add = ent_sig<PK>(T, T.hkv[px], px);
+              pos = hash_pos(y, T.hlog);
+              uint32_t k = 0;
+#pragma unroll 1
+              for (; k <= T.hmask; ++k) {
+                w = T.hkv[pos];
+                if (w == EMPTY) {
+                  // stop inserting once the lists are full, so the table never
+                  // fills beyond lcap + NT keys and probes stay short
+                  if (*nlist_now >= T.lcap) {
+                    cap = true;
+                    break;
+                  }
+                  w = atomicCAS(&T.hkv[pos], EMPTY, ent_word<PK>(y, want_val, PK ? add : 0ull));
+                  if (w == EMPTY) {
+                    res = 1;
+                    ydeg = yhi - ylo;
+                    break;
+                  }
+                }
+                if ((int32_t)(w >> 32) == y) {
+                  const uint32_t v = ent_val<PK>(w);
+                  if (v == want_val) {  // also discovered at this level
+                    ++hits;
+                    if (!ent_add<PK>(T, pos, add)) {
+                      if (PK)
+                        cap = true;  // sigma outgrew the packed field
+                      else
+                        of = true;
+                    }
+                  } else if (FU && fused && val_side(v) != side) {
+                    res = 2;
+                  }
+                  break;
+                }
+                pos = (pos + 1) & T.hmask;
+              }
+              if (k > T.hmask) cap = true;  // table full
+            }
+            const unsigned ins = __ballot_sync(FULL, res == 1);
+            if (ins) {
+              int at = 0;
+              if (lane == 0) at = atomicAdd(&c.nlist, __popc(ins));
+              at = __shfl_sync(FULL, at, 0) + __popc(ins & ((1u << lane) - 1u));
+              if (res == 1) {
+                if (at >= T.lcap) {
+                  cap = true;
+                } else {
+                  if (!PK) T.lnode[at] = y;
+                  lpos_set<PK>(T, at, pos);
+                  cost += (unsigned)ydeg;
+                  if (at - list_before < 32) c.fr[side][at - list_before] = make_int2(ylo, ydeg);
+                  if (!PK && !ent_add<PK>(T, pos, add)) of = true;
+                }
+              }
+            }
+            if (FU && fused) emit(fb, res == 2, p, y, (int)pos, w);
+          });
+        }
+        if (sg + 1 < nseg) {
+          __syncthreads();  // the next segment's prefix overwrites T.pr and the long rows
+          if (RG && pass == 1) {
+            if (tid == 0) c.nlong = 0;
+            __syncthreads();
+          }
+        }
+      }
+      if (pass == 1) {
+        if (!PK && __any_sync(FULL, sigma_of) && lane == 0) atomicOr(&c.lvl_flags, LF_TOUCH_SIGMA);
+        __syncthreads();
+        if (RG && tid == 0) c.nlong = 0;  // every thread has passed its last read of the long rows
+        touched = c.npi > 0;
+        if (touched) break;
+      }
+    }
+    if (!touched) {
+      if (tid == NT - 32) {
+        if (last >= 0) lvl_hi(T, last, last == 0 ? depth0 : depth1) = list_before;
+        lvl_lo(T, side, dnew) = list_before;
+        c.acc[par ^ 1] = 0;  // the next level's
+        c.hacc[par ^ 1] = 0;
+      }
+      cost = __reduce_add_sync(FULL, cost);
+      hits = __reduce_add_sync(FULL, hits);
+      if (lane == 0) {
+        if (cost) atomicAdd(&c.acc[par], cost);
+        if (hits) atomicAdd(&c.hacc[par], hits);
+      }
+      const int lf = (of ? LF_SIGMA : 0) | (cap ? LF_CAP : 0) | (sigma_of ? LF_TOUCH_SIGMA : 0);
+      if (lf) atomicOr(&c.lvl_flags, lf);
+      __syncthreads();
+      if (FU && fused && c.npi > 0) {
         // the level touches: undo its insertions (slots that were empty
         // before it) and choose among its touch arcs, as after pass 1
-        const int sig_of = __syncthreads_or(ftouch & 2);
+#pragma unroll 1
         for (int i = list_before + tid; i < c.nlist; i += NT) {
           const uint32_t q = lpos_get<PK>(T, i);
           T.hkv[q] = EMPTY;
           if (!PK) T.hsig[q] = 0ull;
         }
         __syncthreads();
-        if (tid == 0) {
-          c.nlist = list_before;
-          int tot = 0;
-          for (int w = 0; w < NW; ++w) {
-            tot += c.npi[w];
-            if (c.npi[w] > T.pcap) c.flags |= F_CAP;
-          }
-          if (sig_of) c.flags |= F_SIGMA;
-          c.done = 1;
-          c.stat[KADABRA_STAT_PI] = tot;
-        }
-        __syncthreads();
-        if (c.flags) return;
-        break;
+        if (tid == 0) c.nlist = list_before;
+        touched = true;
       }
-      if (of) atomicOr(&c.flags, F_SIGMA);
-      if (cap) atomicOr(&c.flags, F_CAP);
     }
-    block_sum3(hits, fresh, cost, c.scan_tmp3);
-    if (c.flags) return;
-    if (fresh == 0) {  // frontier exhausted: s and t are not connected
-      if (tid == 0) c.done = 2;
-      __syncthreads();
+    if (touched) {
+      if (tid == 0 && last >= 0) lvl_hi(T, last, last == 0 ? depth0 : depth1) = list_before;
       break;
     }
-    if (tid == 0) {
-      lvl_lo(T, side, dnew) = list_before;
-      lvl_hi(T, side, dnew) = c.nlist;
-      c.depth[side] = dnew;
-      c.cost[side] = cost;
-      c.stat[KADABRA_STAT_NEW] += fresh;
-      c.stat[KADABRA_STAT_SIGMA_ADDS] += hits;
+    const int lf = c.lvl_flags, nl = c.nlist;
+    if (lf) {
+      if (tid == 0) c.flags |= ((lf & LF_SIGMA) ? F_SIGMA : 0) | ((lf & LF_CAP) ? F_CAP : 0);
+      return;
     }
-    __syncthreads();
+    if (nl == list_before) return;  // frontier exhausted: s and t are not connected
+    if (tid == NT - 32) {
+      stat_add(c, KADABRA_STAT_NEW, (unsigned)(nl - list_before));
+      stat_add(c, KADABRA_STAT_SIGMA_ADDS, c.hacc[par]);
+    }
+    if (side == 0) {
+      depth0 = dnew;
+      cost0 = (int)c.acc[par];
+    } else {
+      depth1 = dnew;
+      cost1 = (int)c.acc[par];
+    }
+    last = side;
   }
-  if (c.done == 0) {  // loop bound reached (cannot happen within maxd levels)
+  if (!touched) {  // loop bound reached (cannot happen within maxd levels)
     if (tid == 0) c.flags |= F_CAP;
-    __syncthreads();
     return;
   }
-  if (c.done == 2) return;  // disconnected: no hits
 
   // ------------------------------------------------ candidate-edge choice
   // Candidates are ordered by (x, y), x on the expanding side.
-  {
-    unsigned long long lo = 0, hi = 0;
-    const int npi = c.npi[wid];
-    const PiEntry* seg = T.pi + (size_t)wid * T.pcap;
-    for (int i = lane; i < npi; i += 32) {
-      const unsigned long long w = seg[i].w;
-      lo += w;
-      if (lo < w) ++hi;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long lo2 = __shfl_xor_sync(FULL, lo, o);
-      const unsigned long long hi2 = __shfl_xor_sync(FULL, hi, o);
-      const unsigned long long s = lo + lo2;
-      hi = hi + hi2 + (s < lo ? 1ull : 0ull);
-      lo = s;
-    }
-    if (lane == 0) {
-      c.wsum[wid] = lo;
-      c.wsum_hi[wid] = hi;
-    }
+  const int total = c.npi;
+  if (total > pi_cap || (!PK && (c.lvl_flags & LF_TOUCH_SIGMA))) {
+    if (tid == 0) c.flags |= (total > pi_cap ? F_CAP : 0) | ((c.lvl_flags & LF_TOUCH_SIGMA) ? F_SIGMA : 0);
+    return;
   }
-  __syncthreads();
-  if (tid == 0) {
-    unsigned long long lo = 0, hi = 0;
-    for (int w = 0; w < NW; ++w) {
-      const unsigned long long s = lo + c.wsum[w];
-      hi += c.wsum_hi[w] + (s < lo ? 1ull : 0ull);
-      lo = s;
-    }
-    if (hi != 0) {
-      c.flags |= F_SIGMA;
-    } else {
-      c.stat[KADABRA_STAT_SIGMA_LO] = (long long)(lo & 0xFFFFFFFFull);
-      c.stat[KADABRA_STAT_SIGMA_HI] = (long long)(lo >> 32);
-      c.r = below128(c.draws[1], lo);
-    }
-    int acc = 0;  // segment starts of the flat candidate index
-    for (int w = 0; w < NW; ++w) {
-      const int n_w = c.npi[w];
-      c.npi[w] = acc;
-      acc += n_w;
-    }
-    c.ecount = acc;
-  }
-  __syncthreads();
-  if (c.flags) return;
+  const int dv = depth0, dw = depth1;
   {
-    const int total = c.ecount;
-    // gather the candidates into the scratch half of this CTA's buffer
-    PiEntry* buf = T.pi + (size_t)NW * T.pcap;
-    for (int w = 0; w < NW; ++w) {
-      const int a = c.npi[w], b = (w + 1 < NW) ? c.npi[w + 1] : total;
-      for (int i = a + tid; i < b; i += NT) buf[i] = T.pi[(size_t)w * T.pcap + (i - a)];
-    }
-    __syncthreads();
-    int pick;
-    // the frontier prefix array is free now: small candidate sets are copied
-    // there as (key, weight) pairs and ranked quadratically; larger ones go
-    // through the radix selection
-    unsigned long long* kw = reinterpret_cast<unsigned long long*>(T.pr);
-    if (total <= min(T.frcap / 2, PK ? T.frcap / 2 : QUAD_PICK_MAX)) {  // (key, weight) pairs fit in pr
-      for (int i = tid; i < total; i += NT) {
-        kw[2 * i] = ((unsigned long long)(uint32_t)buf[i].x << 32) | (uint32_t)buf[i].y;
-        kw[2 * i + 1] = buf[i].w;
-      }
-      __syncthreads();
-      pick = block_pick_by_key(
-          total, c.r, c, [&](int i) { return kw[2 * i]; }, [&](int i) { return kw[2 * i + 1]; });
-    } else {
-      // histogram: 256 u64 weights then 256 counts in the frontier array
-      pick = block_pick_radix(buf, total, c.r, c, kw, reinterpret_cast<unsigned*>(kw + 256));
-    }
-    if (pick < 0) {
-      if (tid == 0) c.flags |= F_INTERNAL;
-      __syncthreads();
-      return;
-    }
+    PiEntry* const sh = reinterpret_cast<PiEntry*>(T.pr + cand_at);
+    const int in_sh = PK ? min(total, cand_cap) : 0;  // the first of them are in shared memory
     if (tid == 0) {
-      const PiEntry pe = buf[pick];
-      if (c.side == 0) {
-        c.cv = pe.x;
-        c.cw = pe.y;
+      c.bt_dx[0] = dv;
+      c.bt_dx[1] = dw;
+      c.bt_j[0] = 2;
+      c.bt_j[1] = 2 + (uint32_t)dv;
+      stat_add(c, KADABRA_STAT_PI, (unsigned)total);
+    }
+    if (PK && total <= min(in_sh, NT)) {
+      // Ranked quadratically in shared memory, all pairs spread over the
+      // block: 2^sl neighbouring lanes share a candidate and each adds up
+      // every 2^sl-th weight, both the total and that of the smaller keys, so
+      // the draw's range needs no pass (and no barrier) of its own.  A packed
+      // sigma has 24 bits: the sums fit 64.
+      const int sl = total <= NT / 8 ? 3 : total <= NT / 4 ? 2 : total <= NT / 2 ? 1 : 0;
+      const int i = tid >> sl;
+      if (wid * 32 < total << sl) {
+        const int4 me = reinterpret_cast<const int4*>(sh)[min(i, total - 1)];
+        const unsigned long long key = ((unsigned long long)(uint32_t)me.x << 32) | (uint32_t)me.y;
+        const unsigned long long mw = ((unsigned long long)(uint32_t)me.w << 32) | (uint32_t)me.z;
+        unsigned long long all = 0, below = 0;
+#pragma unroll 2
+        for (int j = tid & ((1 << sl) - 1); j < total; j += 1 << sl) {
+          const int4 e = reinterpret_cast<const int4*>(sh)[j];
+          const unsigned long long w = ((unsigned long long)(uint32_t)e.w << 32) | (uint32_t)e.z;
+          all += w;
+          if ((((unsigned long long)(uint32_t)e.x << 32) | (uint32_t)e.y) < key) below += w;
+        }
+#pragma unroll 1
+        for (int o = 1; o < 1 << sl; o <<= 1) {
+          all += __shfl_xor_sync(FULL, all, o);
+          below += __shfl_xor_sync(FULL, below, o);
+        }
+        const unsigned long long r = below128(c.draws[1], all);
+        if (i < total && (tid & ((1 << sl) - 1)) == 0 && below <= r && r - below < mw) {
+          c.pick = i;
+          c.bt_x[0] = side == 0 ? me.x : me.y;
+          c.bt_x[1] = side == 0 ? me.y : me.x;
+          c.stat[KADABRA_STAT_SIGMA_LO] = (long long)(all & 0xFFFFFFFFull);
+          c.stat[KADABRA_STAT_SIGMA_HI] = (long long)(all >> 32);
+        }
+      }
+    } else {
+      // the weights' 128-bit sum
+#pragma unroll 1
+      for (int i = tid; i < in_sh; i += NT) T.pi[i] = sh[i];
+      unsigned long long lo = 0, hi = 0;
+#pragma unroll 1
+      for (int i = tid; i < total; i += NT) {
+        const unsigned long long w = i < in_sh ? sh[i].w : T.pi[KIDX(i, pi_cap, 15)].w;
+        lo += w;
+        if (lo < w) ++hi;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long lo2 = __shfl_xor_sync(FULL, lo, o);
+        hi += __shfl_xor_sync(FULL, hi, o);
+        lo += lo2;
+        if (lo < lo2) ++hi;
+      }
+      if (lane == 0) {
+        c.wsum[wid] = lo;
+        c.wsum_hi[wid] = hi;
+      }
+      __syncthreads();
+      lo = hi = 0;
+#pragma unroll 1
+      for (int w = 0; w < NW; ++w) {
+        lo += c.wsum[w];
+        hi += c.wsum_hi[w] + (lo < c.wsum[w] ? 1ull : 0ull);
+      }
+      if (hi != 0) {
+        if (tid == 0) c.flags |= F_SIGMA;
+        return;
+      }
+      const unsigned long long r = below128(c.draws[1], lo);
+      int pick;
+      if (!PK && total <= QUAD_PICK_MAX) {
+        pick = block_pick_by_key(
+            total, r, c, [&](int i) { return ((unsigned long long)(uint32_t)T.pi[i].x << 32) | (uint32_t)T.pi[i].y; },
+            [&](int i) { return T.pi[i].w; });
       } else {
-        c.cv = pe.y;
-        c.cw = pe.x;
+        // its histogram (256 u64 weights, then 256 counts) takes the frontier array
+        unsigned long long* kw = reinterpret_cast<unsigned long long*>(T.pr);
+        pick = block_pick_radix(T.pi, total, r, c, kw, reinterpret_cast<unsigned*>(kw + 256));
+      }
+      if (tid == 0) {
+        c.stat[KADABRA_STAT_SIGMA_LO] = (long long)(lo & 0xFFFFFFFFull);
+        c.stat[KADABRA_STAT_SIGMA_HI] = (long long)(lo >> 32);
+        c.pick = pick;
+        if (pick >= 0) {
+          const PiEntry e = T.pi[pick];
+          c.bt_x[0] = side == 0 ? e.x : e.y;
+          c.bt_x[1] = side == 0 ? e.y : e.x;
+        }
       }
     }
-    __syncthreads();
+  }
+  __syncthreads();
+  if (c.pick < 0) {
+    if (tid == 0) c.flags |= F_INTERNAL;
+    return;
   }
 
   // ------------------------------------------------ backtracking
-  // The candidate edge joins the two current frontiers, so v is at depth[0]
-  // on the s side and w at depth[1] on the t side.
-  const int dv = c.depth[0], dw = c.depth[1];
-  if (tid == 0) {
-    const int a = tab_find_pos(T, c.cv), b = tab_find_pos(T, c.cw);
-    const bool ok_a = a >= 0 && ent_val<PK>(T.hkv[a]) == pack_val(0, dv);
-    const bool ok_b = b >= 0 && ent_val<PK>(T.hkv[b]) == pack_val(1, dw);
-    if (!ok_a || !ok_b) c.flags |= F_INTERNAL;
-  }
-  __syncthreads();
-  if (c.flags) return;
+  // The candidate edge joins the two current frontiers, so v is at depth0
+  // on the s side and w at depth1 on the t side.
   const bool want_path = P.paths != nullptr && out_i >= 0;
-  if (tid == 0) {
+  if (tid == NT - 1) {  // a warp that does not walk
+    const int cv = c.bt_x[0], cw = c.bt_x[1];
     c.stat[KADABRA_STAT_DIST] = dv + 1 + dw;
     c.stat[KADABRA_STAT_PATH_NODES] = dv + dw + 2;
     if (want_path) {
       int32_t* row = P.paths + out_i * (int64_t)P.max_len;
-      if (dv < P.max_len) row[dv] = c.cv;
-      if (dv + 1 < P.max_len) row[dv + 1] = c.cw;
+      if (dv < P.max_len) row[dv] = cv;
+      if (dv + 1 < P.max_len) row[dv + 1] = cw;
     }
     if (J.counts) {
-      if (dv > 0) atomicAdd(&J.counts[KIDX(c.cv, J.g.n, 11)], 1u);
-      if (dw > 0) atomicAdd(&J.counts[KIDX(c.cw, J.g.n, 11)], 1u);
+      if (dv > 0) atomicAdd(&J.counts[KIDX(cv, J.g.n, 11)], 1u);
+      if (dw > 0) atomicAdd(&J.counts[KIDX(cw, J.g.n, 11)], 1u);
     }
   }
   // Steps go one node at a time, v -> s over predecessors (walker 0, weights
@@ -1713,15 +1685,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
   // A longer step goes to the whole block.  Both choose the same node with
   // the same draw.  The state between them (node, depth, next draw) lives in
   // c.bt_*[walker].
-  if (tid == 0) {
-    c.bt_x[0] = c.cv;
-    c.bt_dx[0] = dv;
-    c.bt_j[0] = 2;
-    c.bt_x[1] = c.cw;
-    c.bt_dx[1] = dw;
-    c.bt_j[1] = 2 + (uint32_t)dv;
-  }
-  __syncthreads();
+#pragma unroll 1
   for (;;) {
     if (wid < 2) bt_warp_steps<PK>(P, J, T, c, idx, out_i, dv, dw, want_path, wid);
     __syncthreads();
@@ -1750,12 +1714,13 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
         c.bt_flag = 1;  // reported below, after every thread has decided
         c.r = 0;
       } else {
-        c.r = below128(j < 32 ? c.draws[j] : draw(J.seed, J.domain, idx, j),
+        c.r = below128(j < 32 ? c.draws[j] : draw_late(J.seed, J.domain, idx, j),
                        ent_sig<PK>(T, T.hkv[px], (uint32_t)px));
       }
       // scan whichever is shorter: the row of x, or the previous level
       c.mode = ((long long)(phi - plo) * 16 < (long long)deg) ? 1 : 0;
       c.ecount = 0;  // candidates found in the previous level (mode 1)
+      c.pick = -1;
     }
     __syncthreads();
     if (c.bt_flag) {
@@ -1763,8 +1728,10 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
       return;
     }
     const unsigned long long r = c.r;
-    if (c.mode == 1) {
+    bool by_level = c.mode == 1;
+    if (by_level) {
       // previous-level nodes adjacent to x, collected as (node, hash position)
+#pragma unroll 1
       for (int i = plo + tid; i < phi; i += NT) {
         const int y = list_node<PK>(T, i);
         const int a = __ldg(&frow[y]), b = __ldg(&frow[y + 1]);
@@ -1775,13 +1742,10 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
         }
       }
       __syncthreads();
-      if (c.ecount > min(T.frcap, 128)) {
-        if (tid == 0) c.mode = 0;  // many predecessors: scan the row instead
-        __syncthreads();
-      }
+      if (c.ecount > min(T.frcap, 128)) by_level = false;  // many predecessors: scan the row instead
     }
     int y_pick = -1, pos_pick = 0;
-    if (c.mode == 1) {
+    if (by_level) {
       const int nc = c.ecount;
       const int pick = block_pick_by_key(
           nc, r, c, [&](int i) { return (unsigned long long)(uint32_t)T.pr[i].x; },
@@ -1815,7 +1779,6 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
     }
     if (y_pick < 0) {
       if (tid == 0) c.flags |= F_INTERNAL;
-      __syncthreads();
       return;
     }
     if (tid == 0) {
@@ -1828,34 +1791,113 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
   }
 }
 
-// Clears what the last sample left in the hash table (key and sigma of every
-// entry it inserted): the whole table in shared memory (cheaper than
-// locating the entries) or after a capacity failure (entries beyond the
-// lists), else the entries at the positions the lists recorded.
-template <bool PK>
-__device__ void reset_tables(const Tables& T, Ctl& c, bool whole) {
+// Clears what the last sample left in the hash table of a global-memory tier
+// (key and sigma of every entry it inserted): the whole table after a
+// capacity failure (entries beyond the lists), else the entries at the
+// positions the lists recorded.
+__device__ void reset_tables(const Tables& T, Ctl& c) {
   const int tid = threadIdx.x;
-  if (whole || (c.flags & F_CAP)) {
+  if (c.flags & F_CAP) {
+#pragma unroll 1
     for (uint32_t i = tid; i <= T.hmask; i += NT) {
       T.hkv[i] = EMPTY;
-      if (!PK) T.hsig[i] = 0ull;
+      T.hsig[i] = 0ull;
     }
   } else {
     const int nl = min(c.nlist, T.lcap);
+#pragma unroll 1
     for (int i = tid; i < nl; i += NT) {
-      const uint32_t pos = lpos_get<PK>(T, i);
+      const uint32_t pos = lpos_get<false>(T, i);
       T.hkv[pos] = EMPTY;
-      if (!PK) T.hsig[pos] = 0ull;
+      T.hsig[pos] = 0ull;
     }
   }
   __syncthreads();
+}
+
+// Empties a shared-memory table (cheaper than locating a sample's entries):
+// every warp but the first, which meanwhile sets up the next sample.
+__device__ __forceinline__ void clear_table(const Tables& T) {
+  int4* h = reinterpret_cast<int4*>(T.hkv);
+#pragma unroll 1
+  for (uint32_t i = threadIdx.x - 32; i < (T.hmask + 1) / 2; i += NT - 32) h[i] = make_int4(-1, -1, -1, -1);
+}
+
+// The draw and control state of a sample (warp 0; the roots go into the
+// table afterwards).  Every lane draws one of the sample's first 32 Philox
+// blocks ((s,t), candidate edge, backtracking steps), so the serial steps
+// only read them.
+__device__ __forceinline__ void begin_sample(const SampleParams& P, const Tables& T, Ctl& c, uint64_t idx,
+                                             int64_t out_i) {
+  const int lane = lane_id();
+  const GraphDev& G = c.job.g;
+  const uint4 b = draw(c.job.seed, c.job.domain, idx, (uint32_t)lane);
+  c.draws[lane] = b;
+  const uint64_t u = (uint64_t)__shfl_sync(FULL, b.x, 0) | ((uint64_t)__shfl_sync(FULL, b.y, 0) << 32);
+  const uint64_t u2 = (uint64_t)__shfl_sync(FULL, b.z, 0) | ((uint64_t)__shfl_sync(FULL, b.w, 0) << 32);
+  const int s = (int)__umul64hi(u, (uint64_t)G.n);
+  const int tp = (int)__umul64hi(u2, (uint64_t)(G.n - 1));
+  const int t = tp + (tp >= s ? 1 : 0);
+  int bound = 0;  // lanes 0..3: the two roots' row bounds
+  if (lane < 4) bound = __ldg((lane < 2 ? G.rp + s : G.rrp + t) + (lane & 1));
+  if (lane < KADABRA_NSTAT) c.stat[lane] = lane == KADABRA_STAT_DIST ? -1 : 0;
+  const int deg = __shfl_down_sync(FULL, bound, 1) - bound;
+  if (lane == 0) {
+    c.s = s;
+    c.t = t;
+    c.flags = 0;
+    c.lvl_flags = 0;
+    c.bt_flag = 0;
+    c.npi = 0;
+    c.pick = -1;
+    c.acc[0] = c.acc[1] = c.hacc[0] = c.hacc[1] = 0;
+    c.nlist = 2;
+    lvl_lo(T, 0, 0) = 0;
+    lvl_hi(T, 0, 0) = 1;
+    lvl_lo(T, 1, 0) = 1;
+    lvl_hi(T, 1, 0) = 2;
+    c.fside = -1;
+    c.nlong = 0;
+    c.cost[0] = (unsigned)deg;
+  }
+  if (lane == 0 || lane == 2) c.fr[lane >> 1][0] = make_int2(bound, deg);
+  if (lane == 2) c.cost[1] = (unsigned)deg;
+  if (out_i >= 0 && P.paths)
+#pragma unroll 1
+    for (int q = lane; q < P.max_len; q += 32) P.paths[out_i * (int64_t)P.max_len + q] = -1;
+  __syncwarp();
+}
+
+// s and t into the (empty) table: the level 0 of both sides (warp 0)
+template <bool PK>
+__device__ __forceinline__ void insert_roots(const Tables& T, Ctl& c) {
+  if (threadIdx.x == 0) {
+    uint32_t ps = 0, pt = 0;
+    if (tab_insert(T, c.s, ent_word<PK>(c.s, pack_val(0, 0), 1ull), &ps) != 1) c.flags |= F_INTERNAL;
+    if (tab_insert(T, c.t, ent_word<PK>(c.t, pack_val(1, 0), 1ull), &pt) != 1) c.flags |= F_INTERNAL;
+    if (!PK) {
+      T.hsig[ps] = 1ull;
+      T.hsig[pt] = 1ull;
+      T.lnode[0] = c.s;
+      T.lnode[1] = c.t;
+    }
+    lpos_set<PK>(T, 0, ps);
+    lpos_set<PK>(T, 1, pt);
+  }
+  __syncwarp();
 }
 
 // global-memory tiers share one body per scan kind, compiled outside the kernel
 template <bool RG>
 __device__ __noinline__ void run_sample_global(const SampleParams& P, const Job& J, const Tables& T, Ctl& c,
                                                uint64_t idx, int64_t out_i) {
+  if (warp_id() == 0) {
+    begin_sample(P, T, c, idx, out_i);
+    insert_roots<false>(T, c);
+  }
+  __syncthreads();
   run_sample<false, RG>(P, J, T, c, idx, out_i);
+  __syncthreads();
 }
 
 // layout of one CTA's tables in global memory (tiers M and L)
@@ -1888,6 +1930,7 @@ __device__ inline Tables gm_tables(unsigned char* base, int hlog, int lcap, int 
   T.lcap = lcap;
   T.frcap = lcap;
   T.lpos16 = nullptr;
+  T.lr = nullptr;  // set by the kernel
   T.bits = nullptr;
   T.fwords = 0;
   T.fshift = 32;
@@ -1907,7 +1950,8 @@ constexpr int FRONTIER_SEG = KD_FRONTIER_SEG;
 #ifndef KD_LOAD_QUARTERS
 #define KD_LOAD_QUARTERS 3
 #endif
-template <int HLOG, int L8, int FSEG, int FLOG, int MAXD>
+constexpr size_t CTL_BYTES = (sizeof(Ctl) + 15) & ~size_t(15);
+template <int HLOG, int L8, int FSEG, int FLOG, int MAXD, bool LR>
 struct SLayout {
   static constexpr int SLOTS_LOG = HLOG;
   // nodes a table takes before the sample moves on to the next tier (the
@@ -1919,12 +1963,13 @@ struct SLayout {
   static constexpr int FSHIFT = 32 - FLOG;
   static constexpr int LEVELS = MAXD;
   static_assert(MAXD <= 126, "the packed entry's dist field");
-  static constexpr size_t HKV = (sizeof(Ctl) + 15) & ~size_t(15);
+  static constexpr size_t HKV = CTL_BYTES;
   static constexpr size_t PR = HKV + (sizeof(unsigned long long) << HLOG);
   static constexpr size_t LPOS = PR + sizeof(int2) * (FRCAP + 1);
   static constexpr size_t LVL = LPOS + sizeof(uint16_t) * LCAP;
   static constexpr size_t BITS = (LVL + sizeof(int) * 4 * (MAXD + 2) + 15) & ~size_t(15);
-  static constexpr size_t BYTES = BITS + sizeof(uint32_t) * FWORDS;
+  static constexpr size_t LONG = BITS + sizeof(uint32_t) * FWORDS;
+  static constexpr size_t BYTES = LONG + (LR ? sizeof(LongRows) : 0);
   static_assert(HLOG <= 16, "16-bit list positions");
   // the radix selection's histogram (256 u64 + 256 u32) in the frontier array
   static_assert(sizeof(int2) * (FRCAP + 1) >= 256 * (sizeof(unsigned long long) + sizeof(unsigned)),
@@ -1942,9 +1987,9 @@ struct SLayout {
 #ifndef KD_CMP_MAXD
 #define KD_CMP_MAXD 38
 #endif
-using FastLayout = SLayout<FAST_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD>;
-using CompactLayout = SLayout<FAST_HLOG, KD_CMP_L8, 512, KD_CMP_FLOG, KD_CMP_MAXD>;
-using BigLayout = SLayout<BIG_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD>;
+using FastLayout = SLayout<FAST_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
+using CompactLayout = SLayout<FAST_HLOG, KD_CMP_L8, 512, KD_CMP_FLOG, KD_CMP_MAXD, false>;
+using BigLayout = SLayout<BIG_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
 // the tier-S layout a k_sample instance uses (SL)
 constexpr int SL_FAST = 0;
 constexpr int SL_COMPACT = 1;
@@ -1960,6 +2005,7 @@ __device__ inline Tables smem_tables(unsigned char* smem) {
   T.lpos16 = reinterpret_cast<uint16_t*>(smem + L::LPOS);
   T.lvl = reinterpret_cast<int*>(smem + L::LVL);
   T.bits = reinterpret_cast<uint32_t*>(smem + L::BITS);
+  T.lr = L::BYTES > L::LONG ? reinterpret_cast<LongRows*>(smem + L::LONG) : nullptr;
   T.fwords = L::FWORDS;
   T.fshift = L::FSHIFT;
   T.hlog = L::SLOTS_LOG;
@@ -1975,7 +2021,7 @@ constexpr int TF_SKIP_S = 1;
 constexpr int TF_SKIP_B = 2;
 constexpr int TF_SKIP_M = 4;
 constexpr int TF_WARP = 8;  // tier W first, whatever the launch's variant
-constexpr int TF_VEC = 16;  // tier S's level scans read long row stretches with 16-byte loads
+constexpr int TF_VEC = 16;  // pass 1 searches long rows (graphs beyond the L2)
 constexpr int TF_SEG64 = 32;  // shared-memory tiers scan frontiers in 64-node segments (tests)
 constexpr int TF_COMPACT = 64;  // tier S in the compact layout, whatever the launch's variant
 
@@ -1997,23 +2043,50 @@ __device__ void enqueue(const SampleParams& P, int size_ctr, unsigned long long*
     atomicCAS(P.status, 0, (int)KADABRA_ERR_CAPACITY);
 }
 
-// Adds the CTA's accumulated work counters to their job's totals.
+// Adds the CTA's accumulated work counters to their job's totals (warp 0).
 __device__ void flush_totals(const SampleParams& P, Ctl& c) {
-  if (c.tot_job >= 0) {
-    long long* t = P.jobs ? P.jobs[c.tot_job].totals : P.job0.totals;
-    if (t)
-      for (int q = 0; q < KADABRA_NSTAT; ++q)
-        if (c.tot[q]) atomicAdd((unsigned long long*)&t[q], (unsigned long long)c.tot[q]);
+  const int q = lane_id();
+  if (q < KADABRA_NSTAT) {
+    if (c.tot_job >= 0) {
+      long long* t = P.jobs ? P.jobs[c.tot_job].totals : P.job0.totals;
+      if (t && c.tot[q]) atomicAdd((unsigned long long*)&t[q], (unsigned long long)c.tot[q]);
+    }
+    c.tot[q] = 0;
   }
-  for (int q = 0; q < KADABRA_NSTAT; ++q) c.tot[q] = 0;
+  __syncwarp();
 }
 
-// Records the outcome of one sample (per-sample outputs, totals, status).
-__device__ void finish_sample(const SampleParams& P, Ctl& c, uint64_t idx, int64_t out_i) {
+// The job of work index k into c.job (warp 0).
+__device__ __forceinline__ void take_job(const SampleParams& P, Ctl& c, unsigned long long k) {
+  int j = 0;
+  if (P.jobs) {
+    int lo = 0, hi = P.njobs;
+#pragma unroll 1
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (P.jobs[mid].work_begin <= k)
+        lo = mid;
+      else
+        hi = mid;
+    }
+    j = lo;
+  }
+  if (j == c.tot_job) return;
+  flush_totals(P, c);  // the counters so far belong to another job
+  static_assert(sizeof(Job) % 4 == 0 && sizeof(Job) / 4 <= 32, "a lane copies one word");
+  const int q = lane_id();
+  if (q < (int)(sizeof(Job) / 4))
+    reinterpret_cast<uint32_t*>(&c.job)[q] = reinterpret_cast<const uint32_t*>(P.jobs ? &P.jobs[j] : &P.job0)[q];
+  if (q == 0) c.tot_job = j;
+  __syncwarp();
+}
+
+// Records the outcome of one sample (per-sample outputs, totals, status; warp 0).
+__device__ void finish_sample(const SampleParams& P, Ctl& c, int64_t out_i) {
+  int flags = c.flags;
 #ifdef KADABRA_CHECKED
-  if (*(volatile unsigned long long*)&g_checked) c.flags |= F_INTERNAL;
+  if (*(volatile unsigned long long*)&g_checked) flags |= F_INTERNAL;
 #endif
-  const int flags = c.flags;
   int st = KADABRA_OK;
   if (flags & F_INTERNAL)
     st = KADABRA_ERR_INTERNAL;
@@ -2021,25 +2094,20 @@ __device__ void finish_sample(const SampleParams& P, Ctl& c, uint64_t idx, int64
     st = KADABRA_ERR_SIGMA_OVERFLOW;
   else if (flags & F_CAP)
     st = KADABRA_ERR_CAPACITY;
-  if (st != KADABRA_OK) atomicCAS(P.status, 0, st);
-  for (int q = 0; q < KADABRA_NSTAT; ++q)
-    if (q != KADABRA_STAT_SIGMA_LO && q != KADABRA_STAT_SIGMA_HI && q != KADABRA_STAT_DIST) c.tot[q] += c.stat[q];
-  if (out_i >= 0) {
+  const int q = lane_id();
+  if (q == 0 && st != KADABRA_OK) atomicCAS(P.status, 0, st);
+  if (q < KADABRA_NSTAT) {
+    const long long x = c.stat[q];
+    if (q != KADABRA_STAT_SIGMA_LO && q != KADABRA_STAT_SIGMA_HI && q != KADABRA_STAT_DIST) c.tot[q] += x;
+    if (out_i >= 0 && P.stats) P.stats[out_i * KADABRA_NSTAT + q] = x;
+  }
+  if (q == 0 && out_i >= 0) {
     P.st_out[2 * out_i] = c.s;
     P.st_out[2 * out_i + 1] = c.t;
     if (P.path_len) P.path_len[out_i] = (int32_t)c.stat[KADABRA_STAT_PATH_NODES];
-    if (P.stats)
-      for (int q = 0; q < KADABRA_NSTAT; ++q) P.stats[out_i * KADABRA_NSTAT + q] = c.stat[q];
     if (P.sstatus) P.sstatus[out_i] = st;
   }
-}
-
-__device__ void clear_path_row(const SampleParams& P, int64_t out_i) {
-  if (threadIdx.x == 0 && out_i >= 0 && P.paths) {
-    int32_t* row = P.paths + out_i * (int64_t)P.max_len;
-    for (int q = 0; q < P.max_len; ++q) row[q] = -1;
-  }
-  __syncthreads();
+  __syncwarp();
 }
 
 // MODE 0: every sample of the batch, on tier S; overflow -> tier-B queue.
@@ -2047,9 +2115,8 @@ __device__ void clear_path_row(const SampleParams& P, int64_t out_i) {
 // MODE 1: the tier-L queue, on tier L.
 // SL: the tier-S layout of MODE 0; the compact one fits one more CTA per SM
 // and gives the same results (samples that outgrow it go on to tier B as
-// usual).  RG (the default layout only): the level scans read long row
-// stretches with 16-byte loads and search long rows (for graphs whose CSR
-// exceeds L2); same results.
+// usual).  RG (the default layout only): pass 1 searches long rows (for
+// graphs whose CSR exceeds L2); same results.
 template <int MODE, int SL = SL_FAST, bool RG = false>
 __global__ void __launch_bounds__(NT, MODE != 0 ? 2 : SL == SL_FAST ? KD_MIN_BLOCKS : KD_MIN_BLOCKS + 1)
     k_sample(SampleParams P) {
@@ -2064,12 +2131,15 @@ __global__ void __launch_bounds__(NT, MODE != 0 ? 2 : SL == SL_FAST ? KD_MIN_BLO
     TM = gm_tables(P.med_base + (size_t)blockIdx.x * P.med_stride, P.med_hlog, P.med_lcap, MED_MAXD);
   }
   if (MODE == 1) TM = gm_tables(P.gm_base + (size_t)blockIdx.x * P.gm_stride, P.gm_hlog, P.gm_lcap, GM_MAXD);
+  if (MODE == 2) TM.lr = TS.lr;
+  if (MODE == 1) TM.lr = reinterpret_cast<LongRows*>(smem + CTL_BYTES);
   TS.pi = TM.pi = pi;
   TS.pcap = TM.pcap = P.pcap;
   if (MODE != 1 && (P.tier_flags & TF_SEG64)) TS.frcap = min(TS.frcap, 64);
 
   const int tid = threadIdx.x;
   if (tid == 0) {
+#pragma unroll 1
     for (int k = 0; k < KADABRA_NSTAT; ++k) c.tot[k] = 0;
     c.tot_job = -1;
     c.ntotal = MODE == 0 ? (P.q0 ? min(P.ctr[Q_SIZE_S], (unsigned long long)P.deferred_cap)
@@ -2080,84 +2150,70 @@ __global__ void __launch_bounds__(NT, MODE != 0 ? 2 : SL == SL_FAST ? KD_MIN_BLO
   __syncthreads();
   const unsigned long long ntotal = c.ntotal;
   if (ntotal == 0) return;  // nothing queued for this tier: skip the table set-up (the whole block)
-  if (MODE != 1) {
-    for (uint32_t i = tid; i <= TS.hmask; i += NT) TS.hkv[i] = EMPTY;
-    __syncthreads();
-  }
 
+  // Between two samples (two barriers) warp 0 records the last one, takes
+  // the next index and sets its sample up, while the other warps empty the
+  // shared-memory table.
+  bool finish = false;       // a sample to record (warp 0)
+#pragma unroll 1
   for (;;) {
-    if (tid == 0) c.cur = atomicAdd(&P.ctr[MODE == 0 ? Q_NEXT_A : MODE == 2 ? Q_NEXT_B : Q_NEXT_L], 1ull);
-    __syncthreads();
-    if (c.cur >= ntotal) break;
-    // k: the sample's index in the launch's work space; its job and sample index
-    const unsigned long long k = MODE == 0 ? (P.q0 ? P.q0[c.cur] : c.cur) : MODE == 2 ? P.qb[c.cur] : P.ql[c.cur];
-    if (tid == 0) {
-      int j = 0;
-      if (P.jobs) {
-        int lo = 0, hi = P.njobs;
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (P.jobs[mid].work_begin <= k)
-            lo = mid;
-          else
-            hi = mid;
+    if (tid < 32) {
+      unsigned long long cur = 0;
+      if (tid == 0) cur = atomicAdd(&P.ctr[MODE == 0 ? Q_NEXT_A : MODE == 2 ? Q_NEXT_B : Q_NEXT_L], 1ull);
+      if (finish) {
+        const unsigned long long k = c.k;  // the sample's index in the launch's work space
+        if (MODE != 1 && c.flags == F_CAP) {  // to the next tier
+          if (tid == 0) enqueue(P, MODE == 0 ? Q_SIZE_B : Q_SIZE_L, MODE == 0 ? P.qb : P.ql, k);
+        } else {
+          finish_sample(P, c, P.st_out ? (int64_t)k : -1);
         }
-        j = lo;
       }
-      if (j != c.tot_job) {  // the counters so far belong to another job
-        flush_totals(P, c);
-        c.tot_job = j;
+      finish = true;
+      cur = __shfl_sync(FULL, cur, 0);
+      if (cur < ntotal) {
+        const unsigned long long k = MODE == 0 ? (P.q0 ? P.q0[cur] : cur) : MODE == 2 ? P.qb[cur] : P.ql[cur];
+        take_job(P, c, k);
+        if (MODE != 1) begin_sample(P, TS, c, c.job.first_idx + (k - c.job.work_begin), P.st_out ? (int64_t)k : -1);
+        if (tid == 0) c.k = k;
       }
-      c.job = P.jobs ? P.jobs[j] : P.job0;
-      c.job_id = j;
+      if (tid == 0) c.cur = cur;
+    } else if (MODE != 1) {
+      clear_table(TS);
     }
     __syncthreads();
-    const uint64_t idx = c.job.first_idx + (k - c.job.work_begin);
-    const int64_t out_i = P.st_out ? (int64_t)k : -1;
-    bool done = false;
+    if (c.cur >= ntotal) break;
+    const uint64_t idx = c.job.first_idx + (c.k - c.job.work_begin);
+    const int64_t out_i = P.st_out ? (int64_t)c.k : -1;
     if (MODE == 0) {
       if (!(P.tier_flags & TF_SKIP_S)) {
-        clear_path_row(P, out_i);
-        run_sample<true, RG, SL == SL_FAST && (KD_FU_RG || !RG)>(P, c.job, TS, c, idx, out_i);
-        __syncthreads();
-        done = c.flags != F_CAP;
-        reset_tables<true>(TS, c, true);
+        if (tid < 32) insert_roots<true>(TS, c);
+        run_sample<true, RG, SL == SL_FAST || KD_FU_CMP>(P, c.job, TS, c, idx, out_i);
+      } else if (tid == 0) {
+        c.flags = F_CAP;
       }
-      if (!done) {
-        if (tid == 0) enqueue(P, Q_SIZE_B, P.qb, k);
-        __syncthreads();
-        continue;
-      }
+      __syncthreads();
     } else if (MODE == 2) {
+      bool done = false;
       if (!(P.tier_flags & TF_SKIP_B)) {
-        clear_path_row(P, out_i);
+        if (tid < 32) insert_roots<true>(TS, c);
         run_sample<true, RG>(P, c.job, TS, c, idx, out_i);
         __syncthreads();
         done = c.flags != F_CAP;
-        reset_tables<true>(TS, c, true);
+        __syncthreads();
       }
       if (!done && !(P.tier_flags & TF_SKIP_M)) {
-        clear_path_row(P, out_i);
         run_sample_global<RG>(P, c.job, TM, c, idx, out_i);
+        reset_tables(TM, c);
+      } else if (!done) {
+        if (tid == 0) c.flags = F_CAP;
         __syncthreads();
-        done = c.flags != F_CAP;
-        reset_tables<false>(TM, c, false);
-      }
-      if (!done) {
-        if (tid == 0) enqueue(P, Q_SIZE_L, P.ql, k);
-        __syncthreads();
-        continue;
       }
     } else {
-      clear_path_row(P, out_i);
       run_sample_global<RG>(P, c.job, TM, c, idx, out_i);
-      __syncthreads();
-      reset_tables<false>(TM, c, false);
+      reset_tables(TM, c);
     }
-    if (tid == 0) finish_sample(P, c, idx, out_i);
-    __syncthreads();
   }
-  if (tid == 0) flush_totals(P, c);
+  if (tid < 32) flush_totals(P, c);
 }
 
 // ============================================================== tier W: one warp per sample
@@ -3824,7 +3880,7 @@ struct kadabra_graph {
   int directed = 0;
   int32_t *rp = nullptr, *ci = nullptr, *rrp = nullptr, *rci = nullptr;
   int64_t vd = 0;
-  bool csr_beyond_l2 = false;  // forward (+ reverse) CSR larger than the L2: 16-byte scans of long rows
+  bool csr_beyond_l2 = false;  // forward (+ reverse) CSR larger than the L2: long rows are searched
   int device = 0;
   int num_sms = 0;
   uint32_t flags = 0;
@@ -3855,9 +3911,8 @@ struct kadabra_graph {
 };
 
 namespace {
-// internal launch flag: the graph's CSR exceeds the L2, so its level scans
-// read long row stretches with 16-byte loads (KADABRA_FLAG_ASYNC_SCAN asks
-// for that scan explicitly)
+// internal launch flag: the graph's CSR exceeds the L2, so pass 1 searches
+// its long rows (KADABRA_FLAG_ASYNC_SCAN asks for that explicitly)
 constexpr uint32_t FLAG_VEC_AUTO = 1u << 31;
 // the flags a launch shared by several graphs takes from any of them (they
 // change no result; the tier-skipping flags stay per graph)
@@ -4131,9 +4186,9 @@ kadabra_status launch_sampler_kernels(Workspace* w, SampleParams P, cudaStream_t
   P.pi_base = w->pi_gm;
   P.pcap = w->pcap_gm;
   if (rg)
-    k_sample<1, SL_FAST, true><<<w->grid_gm, NT, sizeof(Ctl), st>>>(P);
+    k_sample<1, SL_FAST, true><<<w->grid_gm, NT, CTL_BYTES + sizeof(LongRows), st>>>(P);
   else
-    k_sample<1><<<w->grid_gm, NT, sizeof(Ctl), st>>>(P);
+    k_sample<1><<<w->grid_gm, NT, CTL_BYTES + sizeof(LongRows), st>>>(P);
   KCK(cudaGetLastError());
   return KADABRA_OK;
 }
