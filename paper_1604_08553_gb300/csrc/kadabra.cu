@@ -3238,11 +3238,13 @@ __global__ void k_philox(uint64_t seed, uint32_t domain, uint32_t j, uint64_t fi
 // ============================================================== graph checks, VD
 // error bits: 1 offsets, 2 id range, 4 order/duplicate, 8 self-loop, 16 reverse mismatch
 //
-// The arc checks run arc-parallel: each thread takes LOAD_CHUNK consecutive
-// arcs, finds the row of the first by binary search over the (already
-// validated) offsets and steps through the rows from there.  A hub's row is
-// thus spread over many threads instead of serialising one warp.
-constexpr int LOAD_CHUNK = 16;
+// The arc passes run arc-parallel: a warp takes ARC_CHUNK consecutive arcs,
+// one per lane at a time, so the column array is read coalesced and a hub's
+// row is spread over many warps.
+// R-MAT scale 24's row checks, two passes of 263 M arcs: 16 arcs per thread
+// read with a stride of 64 bytes 3.09 ms; chunks of 128, 256, 512 arcs per
+// warp 2.94, 2.46, 2.18 ms (each chunk searches its first row).
+constexpr int ARC_CHUNK = 512;
 
 // offsets: 0 <= rp[v] <= rp[v+1] <= m (rp[0] = 0 and rp[n] = m are checked on the host)
 __global__ void k_validate_offsets(const int32_t* rp, int32_t n, int64_t m, unsigned* err) {
@@ -3254,51 +3256,119 @@ __global__ void k_validate_offsets(const int32_t* rp, int32_t n, int64_t m, unsi
   if (__any_sync(FULL, bad) && lane_id() == 0) atomicOr(err, 1u);
 }
 
-// the row u that holds arc e: the largest u with rp[u] <= e (rp monotone, e < rp[n])
-__device__ __forceinline__ int32_t row_of_arc(const int32_t* rp, int32_t n, int64_t e) {
-  int32_t lo = 0, hi = n;
-  while (lo < hi) {
-    const int32_t mid = (int32_t)(((int64_t)lo + hi + 1) >> 1);
-    if (rp[mid] <= e)
-      lo = mid;
-    else
-      hi = mid - 1;
+// The row u that holds arc e: the largest u with rp[u] <= e (rp monotone,
+// e < rp[n]), by one warp, 32 offsets per round.
+__device__ __forceinline__ int32_t warp_row_of_arc(const int32_t* rp, int32_t n, int64_t e) {
+  int32_t lo = 0, hi = n;  // rp[lo] <= e, and e < rp[hi]
+  while (hi - lo > 1) {
+    const int32_t step = (hi - lo + 31) / 32;
+    const int64_t i = lo + (int64_t)(lane_id() + 1) * step;
+    const int k = __popc(__ballot_sync(FULL, i < hi && __ldg(&rp[i]) <= e));
+    lo += k * step;
+    hi = min((int64_t)hi, (int64_t)lo + step);
   }
   return lo;
 }
 
-// Calls f(u, e, v) for every arc e = (u, v) of the thread's chunks.
-template <class F>
+// Calls f(ok, u, e, v) for arcs e[k] = (u[k], v[k]), D per lane (32 apart;
+// ok[k] = there is one), with all lanes of the warp.  The lanes' rows come
+// from the starts of the next rows, 32 at a time, counted by a search over
+// the lanes' registers (several rounds only where rows are so short, or
+// empty, that more than 32 start in a window).
+template <int D, class F>
 __device__ __forceinline__ void for_each_arc(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m, F f) {
-  const int64_t chunks = (m + LOAD_CHUNK - 1) / LOAD_CHUNK;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < chunks; c += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e0 = c * LOAD_CHUNK, e1 = e0 + LOAD_CHUNK < m ? e0 + LOAD_CHUNK : m;
-    int32_t u = row_of_arc(rp, n, e0);
-    int64_t next = rp[u + 1];
-    for (int64_t e = e0; e < e1; ++e) {
-      while (e >= next) next = rp[++u + 1];
-      f(u, e, ci[e]);
+  const int lane = lane_id();
+  const int64_t chunks = (m + ARC_CHUNK - 1) / ARC_CHUNK;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < chunks; c += nwarps) {
+    const int64_t e1 = min(m, (c + 1) * ARC_CHUNK);
+    int32_t row = warp_row_of_arc(rp, n, c * ARC_CHUNK);
+    for (int64_t base = c * ARC_CHUNK; base < e1; base += 32 * D) {
+      bool ok[D];
+      int32_t u[D], v[D];
+      int64_t e[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        e[k] = base + 32 * k + lane;
+        ok[k] = e[k] < e1;
+        v[k] = ok[k] ? __ldg(&ci[e[k]]) : 0;
+      }
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const int64_t last = base + 32 * k + 31;
+        u[k] = row;
+        for (int32_t r = row;; r += 32) {
+          const int32_t st = r + 1 + lane < n ? __ldg(&rp[r + 1 + lane]) : 0x7FFFFFFF;  // no arc has this index
+          if (!__any_sync(FULL, st <= last)) break;
+          int q = 0;  // how many of the 32 rows start at e or before
+#pragma unroll
+          for (int h = 16; h > 0; h >>= 1)
+            if (__shfl_sync(FULL, st, q + h - 1) <= e[k]) q += h;
+          if (__shfl_sync(FULL, st, q) <= e[k]) ++q;
+          if (q > 0) u[k] = r + q;
+          if (__shfl_sync(FULL, st, 31) > last) break;
+        }
+        row = __shfl_sync(FULL, u[k], 31);
+      }
+      f(ok, u, e, v);
     }
   }
 }
 
 // ids in range, rows strictly increasing (sorted, no repeats), no self-loops
-__global__ void k_validate_arcs(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m, unsigned* err) {
+__global__ void __launch_bounds__(256) k_validate_arcs(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m,
+                                                       unsigned* err) {
   unsigned bits = 0;
-  for_each_arc(rp, ci, n, m, [&](int32_t u, int64_t e, int32_t v) {
-    if (v < 0 || v >= n) bits |= 2u;
-    if (e > rp[u] && v <= ci[e - 1]) bits |= 4u;
-    if (v == u) bits |= 8u;
+  for_each_arc<4>(rp, ci, n, m, [&](const bool* ok, const int32_t* u, const int64_t* e, const int32_t* v) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      int32_t before = __shfl_up_sync(FULL, v[k], 1);
+      if (!ok[k]) continue;
+      const bool first = e[k] == __ldg(&rp[u[k]]);
+      if (lane_id() == 0 && !first) before = __ldg(&ci[e[k] - 1]);
+      if (v[k] < 0 || v[k] >= n) bits |= 2u;
+      if (!first && v[k] <= before) bits |= 4u;
+      if (v[k] == u[k]) bits |= 8u;
+    }
   });
   bits = __reduce_or_sync(FULL, bits);
   if (bits && lane_id() == 0) atomicOr(err, bits);
 }
 
-__device__ __forceinline__ bool row_has(const int32_t* rp, const int32_t* ci, int32_t v, int32_t y) {
-  int32_t lo = rp[v], hi = rp[v + 1];
+// Every PIVOT-th entry of the column array searched by the mirror test.
+// A binary search in a long row of a graph beyond the L2 reads HBM at most of
+// its steps, and that many scattered reads bound the test: one, two or four
+// searches per lane at once, and arcs taken in narrower windows, all took 32
+// to 33 ms on R-MAT scale 24 (263 M arcs).  Over the pivots (33 MB of its
+// 1.05 GB, which stay in the L2) a search leaves HBM its last PIVOT entries,
+// one 128-byte line: 15.6 ms; every 16th entry 15.6, every 64th 17.4 ms.
+// Graphs within the L2 have none.
+constexpr int PIVOT = 32;
+__global__ void k_pivots(const int32_t* ci, int64_t m, int32_t* piv) {
+  const int64_t k = (m + PIVOT - 1) / PIVOT;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < k; i += (int64_t)gridDim.x * blockDim.x)
+    piv[i] = ci[i * PIVOT];
+}
+
+// row v of a sorted CSR has y (piv: its pivots, or null)
+__device__ __forceinline__ bool row_has(const int32_t* rp, const int32_t* ci, const int32_t* piv, int32_t v, int32_t y) {
+  int32_t lo = __ldg(&rp[v]), hi = __ldg(&rp[v + 1]);
+  if (piv && hi - lo > PIVOT) {
+    int32_t a = lo / PIVOT, b = (hi - 1) / PIVOT;  // the last pivot in (a, b] not above y, or a if there is none
+    const int32_t b0 = b;
+    while (a < b) {
+      const int32_t mid = a + (b - a + 1) / 2;
+      if (__ldg(&piv[mid]) <= y)
+        a = mid;
+      else
+        b = mid - 1;
+    }
+    lo = max(lo, a * PIVOT);
+    if (a < b0) hi = (a + 1) * PIVOT;
+  }
   while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    const int32_t z = ci[mid];
+    const int32_t mid = lo + ((hi - lo) >> 1);
+    const int32_t z = __ldg(&ci[mid]);
     if (z == y) return true;
     if (z < y)
       lo = mid + 1;
@@ -3314,33 +3384,33 @@ __device__ __forceinline__ bool row_has(const int32_t* rp, const int32_t* ci, in
 // undirected graph is its own mirror: there only arcs with u < v are looked
 // up, and the arcs with u < v and u > v are counted (lt_gt[0], lt_gt[1]);
 // equal counts make the injection from the first kind into the second a
-// bijection, which is symmetry.  For a directed graph the same pass counts,
-// per node u, the arcs (u, v) whose reverse arc (v, u) exists (recip[u]),
-// for the degree of u in the underlying undirected graph.
-__global__ void k_validate_mirror(const int32_t* rp, const int32_t* ci, const int32_t* rrp, const int32_t* rci,
-                                  int32_t n, int64_t m, int undirected, unsigned* err, unsigned long long* lt_gt,
-                                  uint32_t* recip) {
+// bijection, which is symmetry.
+// For a directed graph the same pass counts, per node u that can be the root
+// r below, the arcs (u, v) whose reverse arc (v, u) exists (recip[u]): the
+// degree in the underlying undirected graph is at least max(out, in) and at
+// most out + in, so only the nodes whose out + in reaches the largest
+// max(out, in) of any node (*floor_deg) can be it.
+__global__ void __launch_bounds__(256) k_validate_mirror(const int32_t* rp, const int32_t* ci, const int32_t* rrp,
+                                                         const int32_t* rci, int32_t n, int64_t m, int undirected,
+                                                         unsigned* err, unsigned long long* lt_gt, uint32_t* recip,
+                                                         const int32_t* floor_deg, const int32_t* piv) {
   unsigned long long lt = 0, gt = 0;
   bool bad = false;
-  int32_t ru = -1;  // the node whose reciprocal arcs are being counted
-  uint32_t rc = 0;
-  for_each_arc(rp, ci, n, m, [&](int32_t u, int64_t, int32_t v) {
+  const int32_t floor = undirected ? 0 : *floor_deg;
+  for_each_arc<1>(rp, ci, n, m, [&](const bool* ok, const int32_t* uu, const int64_t*, const int32_t* vv) {
+    if (!ok[0]) return;
+    const int32_t u = uu[0], v = vv[0];
     if (undirected && v < u) {
       ++gt;
       return;
     }
     ++lt;
-    if (!row_has(rrp, rci, v, u)) bad = true;
+    if (!row_has(rrp, rci, piv, v, u)) bad = true;
     if (!undirected) {
-      if (u != ru) {
-        if (rc) atomicAdd(&recip[ru], rc);
-        ru = u;
-        rc = 0;
-      }
-      if (row_has(rrp, rci, u, v)) ++rc;
+      const int64_t both = (int64_t)(__ldg(&rp[u + 1]) - __ldg(&rp[u])) + (__ldg(&rrp[u + 1]) - __ldg(&rrp[u]));
+      if (both >= floor && row_has(rrp, rci, piv, u, v)) atomicAdd(&recip[u], 1u);
     }
   });
-  if (rc) atomicAdd(&recip[ru], rc);
   if (__any_sync(FULL, bad) && lane_id() == 0) atomicOr(err, 16u);
   if (undirected) {
     lt = warp_sum_u64(lt);
@@ -3352,9 +3422,19 @@ __global__ void k_validate_mirror(const int32_t* rp, const int32_t* ci, const in
   }
 }
 
+// the largest max(out, in) of any node (directed graphs; offsets already validated)
+__global__ void k_floor_degree(const int32_t* rp, const int32_t* rrp, int32_t n, int32_t* floor_deg) {
+  int32_t d = 0;
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    d = max(d, max(rp[v + 1] - rp[v], rrp[v + 1] - rrp[v]));
+  d = __reduce_max_sync(FULL, d);
+  if (lane_id() == 0) atomicMax(floor_deg, d);
+}
+
 // The root r of the VD bound: the lowest-id node of maximum degree in the
 // underlying undirected graph, |out(v) U in(v)| = out + in - reciprocal arcs
-// (directed), as a key degree << 32 | ~id under atomicMax.
+// (directed; the nodes whose reciprocal arcs were not counted stay below the
+// others), as a key degree << 32 | ~id under atomicMax.
 __global__ void k_und_degree_key(const int32_t* rp, const int32_t* rrp, const uint32_t* recip, int32_t n,
                                  int directed, unsigned long long* best) {
   unsigned long long mine = 0;
@@ -3389,9 +3469,10 @@ struct BfsItem {
   int32_t v, begin, end, pad;
 };
 
-// scans arcs [a, b) of row c and appends the newly reached heads to next
-__device__ __forceinline__ void bfs_scan(const int32_t* c, int32_t a, int32_t b, int32_t* next, int32_t* nnext,
-                                         int32_t* dist, int32_t level) {
+// scans arcs [a, b) of row c and appends the newly reached heads to next, and
+// their rows' arcs to nnext[2]
+__device__ __forceinline__ void bfs_scan(const int32_t* tr, const int32_t* c, int32_t a, int32_t b, int32_t* next,
+                                         int32_t* nnext, int32_t* dist, int32_t level) {
   const int lane = lane_id();
   for (int32_t base = a; base < b; base += 32) {  // bounds uniform in the warp
     const int32_t e = base + lane;
@@ -3408,25 +3489,34 @@ __device__ __forceinline__ void bfs_scan(const int32_t* c, int32_t a, int32_t b,
       if (lane == 0) at = atomicAdd(nnext, __popc(got));
       at = __shfl_sync(FULL, at, 0);
       if (mine) next[at + __popc(got & ((1u << lane) - 1u))] = y;
+      const int32_t arcs = __reduce_add_sync(FULL, mine ? tr[y + 1] - tr[y] : 0);
+      if (lane == 0 && arcs) atomicAdd(nnext + 2, arcs);
     }
   }
 }
 
 // The frontier's size is read on the device (*nfront_dev, or 1 for the root's
 // level when it is null), so the host can queue several levels at once.
-// A frontier of more than n / BFS_BOTTOM_UP nodes is expanded bottom-up
-// (Beamer et al.'s direction-optimising BFS): every unvisited node looks in
-// its row of the opposite CSR (br, bc) for a node at the current level and
-// stops at the first.  Either direction yields the same next level.
+// A frontier of more than n / BFS_BOTTOM_UP nodes, or whose rows hold more
+// than m / BFS_BOTTOM_UP_ARCS arcs, is expanded bottom-up (Beamer et al.'s
+// direction-optimising BFS): every unvisited node looks in its row of the
+// opposite CSR (br, bc) for a node at the current level and stops at the
+// first, after m / (frontier arcs) looks or so.  Either direction yields the
+// same next level.  The arcs count for themselves: the neighbours of a
+// power-law graph's largest hub are few, but hold most arcs (both BFS of
+// R-MAT scale 24: 6.7 -> 4.0 ms; m/2 to m/16 measure the same there, and the
+// Chung-Lu graph of 10^6 nodes takes 0.42 ms with m/8 and 0.33 with m/16).
 constexpr int BFS_BOTTOM_UP = 16;
+constexpr int BFS_BOTTOM_UP_ARCS = 16;
 
 __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t* br, const int32_t* bc,
                             const int32_t* front, const int32_t* nfront_dev, int32_t* next, int32_t* nnext,
                             int32_t* dist, int32_t level, BfsItem* items, int32_t* nitems, int32_t items_cap,
-                            int32_t n) {
+                            int32_t n, int64_t m) {
   const int lane = lane_id();
   const int32_t nfront = nfront_dev ? *nfront_dev : 1;
-  if (nfront > n / BFS_BOTTOM_UP) {
+  const int32_t arcs = nfront_dev ? nfront_dev[2] : 0;
+  if (nfront > n / BFS_BOTTOM_UP || arcs > m / BFS_BOTTOM_UP_ARCS) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;  // a multiple of 32: warps stay whole
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
       const int64_t v = base + threadIdx.x;
@@ -3445,6 +3535,8 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
         if (lane == 0) at = atomicAdd(nnext, __popc(got));
         at = __shfl_sync(FULL, at, 0);
         if (mine) next[at + __popc(got & ((1u << lane) - 1u))] = (int32_t)v;
+        const int32_t own = __reduce_add_sync(FULL, mine ? tr[v + 1] - tr[v] : 0);
+        if (lane == 0 && own) atomicAdd(nnext + 2, own);
       }
     }
     return;
@@ -3455,7 +3547,7 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
     const int32_t v = front[i];
     const int32_t a = tr[v], b = tr[v + 1];
     if (b - a <= BFS_CHUNK) {
-      bfs_scan(tc, a, b, next, nnext, dist, level);
+      bfs_scan(tr, tc, a, b, next, nnext, dist, level);
       continue;
     }
     const int32_t k = (b - a + BFS_CHUNK - 1) / BFS_CHUNK;  // items of this row
@@ -3468,19 +3560,19 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
         items[at + q] = BfsItem{v, s, s + BFS_CHUNK < b ? s + BFS_CHUNK : b, 0};
       }
     }
-    if (at + k > items_cap) bfs_scan(tc, a + (items_cap > at ? items_cap - at : 0) * BFS_CHUNK, b, next, nnext,
+    if (at + k > items_cap) bfs_scan(tr, tc, a + (items_cap > at ? items_cap - at : 0) * BFS_CHUNK, b, next, nnext,
                                      dist, level);  // items beyond the buffer: this warp scans them
   }
 }
 
-__global__ void k_bfs_items(const int32_t* tc, const BfsItem* items, const int32_t* nitems, int32_t items_cap,
+__global__ void k_bfs_items(const int32_t* tr, const int32_t* tc, const BfsItem* items, const int32_t* nitems, int32_t items_cap,
                             int32_t* next, int32_t* nnext, int32_t* dist, int32_t level) {
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int32_t k = *nitems < items_cap ? *nitems : items_cap;
   for (int64_t i = w0; i < k; i += nwarps) {
     const BfsItem it = items[i];
-    bfs_scan(tc, it.begin, it.end, next, nnext, dist, level);
+    bfs_scan(tr, tc, it.begin, it.end, next, nnext, dist, level);
   }
 }
 
@@ -3628,33 +3720,41 @@ __global__ void k_vd_sizes(const int32_t* lab, int32_t n, int32_t* sz) {
 }
 
 __global__ void k_vd_indeg(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m, const int32_t* lab,
-                           int32_t* cnt) {
-  // each thread counts a run of arcs into one label before it adds
-  int32_t cur = -1, k = 0;
-  for_each_arc(rp, ci, n, m, [&](int32_t u, int64_t, int32_t v) {
-    const int32_t lv = lab[v];
-    if (lab[u] == lv) return;
-    if (lv != cur) {
-      if (k) atomicAdd(&cnt[cur], k);
-      cur = lv;
-      k = 0;
+                           const unsigned long long* best, int32_t* cnt) {
+  const int32_t root = key_root(*best);
+  // the arcs into the root's component, most of all, are counted per warp
+  unsigned into_root = 0;
+  for_each_arc<4>(rp, ci, n, m, [&](const bool* ok, const int32_t* u, const int64_t*, const int32_t* v) {
+    int32_t lu[4], lv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      lu[k] = ok[k] ? __ldg(&lab[u[k]]) : 0;
+      lv[k] = ok[k] ? __ldg(&lab[v[k]]) : 0;
     }
-    ++k;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (lu[k] == lv[k]) continue;
+      if (lv[k] == root)
+        ++into_root;
+      else
+        atomicAdd(&cnt[lv[k]], 1);
+    }
   });
-  if (k) atomicAdd(&cnt[cur], k);
+  into_root = __reduce_add_sync(FULL, into_root);
+  if (into_root && lane_id() == 0) atomicAdd(&cnt[root], (int32_t)into_root);
 }
 
 // The heaviest path of the condensation, level by level in topological order
 // (Kahn): a component is ready once every arc entering it has been
 // processed; its heaviest path ending in it weighs w + best[label].
 // Single-node components join the node frontier; a larger component ready at
-// level l is marked rdy[label] = l, and at that level a pass over all arcs
-// (balanced, whatever the rows' lengths) takes its nodes' arcs.  slot[0] of
+// level l is marked rdy[label] = l, and at that level a pass over the in-arcs
+// (balanced, whatever the rows' lengths) takes the arcs that leave it.  slot[0] of
 // level l: the next frontier's size; slot[1]: a larger component is ready at
 // level l + 1.
 
 struct VdKahn {
-  const int32_t *rp, *ci, *lab, *sz;
+  const int32_t *rp, *ci, *rrp, *rci, *lab, *sz;
   int32_t* cnt;
   long long* best;
   int32_t* rdy;
@@ -3696,33 +3796,44 @@ __global__ void k_vd_kahn_init(VdKahn K, int32_t* front, int32_t* slot) {
   }
 }
 
-// one ready node u, by a warp: its path weight, then its arcs into other components
-__device__ void vd_kahn_node(const VdKahn& K, int32_t u, int32_t level, int32_t* next, int32_t* slot) {
+// What a warp has for the root's component and for the bound, added once at
+// its end: millions of nodes enter that component, and every node's path
+// weight is a candidate, so each adding for itself queued on one address
+// (the levels of R-MAT scale 24: 10.1 -> 3.1 ms).
+struct VdWarp {
+  long long vd, root_w;  // the largest path weight; the largest of an arc into the root's component
+  int32_t into_root;     // those arcs
+};
+
+// The arcs a .. b of one ready single-node component u (path weight w) into
+// other components, by a warp.
+__device__ __forceinline__ void vd_kahn_row(const VdKahn& K, int32_t u, long long w, int32_t a, int32_t b,
+                                            int32_t level, int32_t* next, int32_t* slot, VdWarp& W) {
   const int lane = lane_id();
-  const int32_t L = K.lab[u];
-  const long long w = vd_weight(K, L) + K.best[L];
-  if (lane == 0 && L == u) atomicMax(K.vd, w);  // once per component: its representative
-  const int32_t a = K.rp[u], b = K.rp[u + 1];
   for (int32_t base = a; base < b; base += 32) {
     const int32_t e = base + lane;
     bool push = false;
-    int32_t y = 0;
-    int32_t Ly = L;  // this lane's arc enters no other component unless set below
-    if (e < b) {
-      y = K.ci[e];
-      Ly = K.lab[y];
+    int32_t Ly = u;  // this lane's arc enters no other component unless set below
+    if (e < b) Ly = K.lab[K.ci[e]];
+    const int32_t k0 = __popc(__ballot_sync(FULL, Ly != u && Ly == K.root_label));
+    if (k0) {
+      W.into_root += k0;
+      W.root_w = w > W.root_w ? w : W.root_w;
     }
     // lanes whose arcs enter the same component update it once
-    const unsigned same = __match_any_sync(FULL, Ly);
-    if (Ly != L && lane == __ffs(same) - 1) {
-      atomicMax(&K.best[Ly], w);
-      const int k = __popc(same);
-      if (atomicSub(&K.cnt[Ly], k) == k) {
-        if (K.sz[Ly] == 1) {
-          push = true;  // a single-node component: its node is y (only one arc can enter it last)
-        } else {
-          K.rdy[Ly] = level + 1;
-          slot[1] = 1;
+    const bool on = Ly != u && Ly != K.root_label;
+    if (__any_sync(FULL, on)) {
+      const unsigned same = __match_any_sync(FULL, Ly);
+      if (on && lane == __ffs(same) - 1) {
+        atomicMax(&K.best[Ly], w);
+        const int k = __popc(same);
+        if (atomicSub(&K.cnt[Ly], k) == k) {
+          if (K.sz[Ly] == 1) {
+            push = true;  // a single-node component is its node
+          } else {
+            K.rdy[Ly] = level + 1;
+            slot[1] = 1;
+          }
         }
       }
     }
@@ -3731,33 +3842,53 @@ __device__ void vd_kahn_node(const VdKahn& K, int32_t u, int32_t level, int32_t*
       int32_t at = 0;
       if (lane == 0) at = atomicAdd(&slot[0], __popc(got));
       at = __shfl_sync(FULL, at, 0);
-      if (push) next[at + __popc(got & ((1u << lane) - 1u))] = y;
-    }
-  }
-}
-
-// an arc u -> y of a component that is ready (path weight w to its end)
-__device__ __forceinline__ void vd_kahn_arc(const VdKahn& K, int32_t L, long long w, int32_t y, int32_t level,
-                                            int32_t* next, int32_t* slot) {
-  const int32_t Ly = K.lab[y];
-  if (Ly == L) return;
-  atomicMax(&K.best[Ly], w);
-  if (atomicSub(&K.cnt[Ly], 1) == 1) {
-    if (K.sz[Ly] == 1) {
-      next[atomicAdd(&slot[0], 1)] = y;
-    } else {
-      K.rdy[Ly] = level + 1;
-      slot[1] = 1;
+      if (push) next[at + __popc(got & ((1u << lane) - 1u))] = Ly;
     }
   }
 }
 
 __global__ void k_vd_kahn_level(VdKahn K, int64_t m, const int32_t* front, const int32_t* prev, int32_t* next,
                                 int32_t* slot, int32_t level) {
-  const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int32_t nfront = prev[0];
-  for (int64_t i = w0; i < nfront; i += nwarps) vd_kahn_node(K, front[i], level, next, slot);
+  const int64_t nfront = prev[0];
+  VdWarp W = {0, 0, 0};
+  // a warp takes 32 ready nodes at a time, and the rows of those that have one
+  for (int64_t i0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ~31ll; i0 < nfront;
+       i0 += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = lane_id();
+    int32_t u = 0, a = 0, b = 0;
+    long long w = 0;
+    if (i0 + lane < nfront) {
+      u = front[i0 + lane];
+      a = K.rp[u];
+      b = K.rp[u + 1];
+      w = vd_weight(K, u) + K.best[u];  // a single-node component's label is its node
+    }
+    W.vd = w > W.vd ? w : W.vd;
+    for (unsigned rows = __ballot_sync(FULL, b > a); rows; rows &= rows - 1) {
+      const int j = __ffs(rows) - 1;
+      vd_kahn_row(K, __shfl_sync(FULL, u, j), __shfl_sync(FULL, w, j), __shfl_sync(FULL, a, j),
+                  __shfl_sync(FULL, b, j), level, next, slot, W);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long x = __shfl_xor_sync(FULL, W.vd, o);
+    W.vd = x > W.vd ? x : W.vd;
+  }
+  if (lane_id() == 0) {
+    if (W.vd > 0) atomicMax(K.vd, W.vd);
+    if (W.into_root) {
+      atomicMax(&K.best[K.root_label], W.root_w);
+      if (atomicSub(&K.cnt[K.root_label], W.into_root) == W.into_root) {
+        if (K.sz[K.root_label] == 1) {
+          next[atomicAdd(&slot[0], 1)] = K.root_label;
+        } else {
+          K.rdy[K.root_label] = level + 1;
+          slot[1] = 1;
+        }
+      }
+    }
+  }
   if (!prev[1]) return;
   // larger components ready at this level: their representatives' path
   // weights, then every arc leaving one of their nodes
@@ -3766,18 +3897,37 @@ __global__ void k_vd_kahn_level(VdKahn K, int64_t m, const int32_t* front, const
     const int32_t L = K.lab[v];
     if (L == (int32_t)v && K.sz[L] > 1 && K.rdy[L] == level) atomicMax(K.vd, vd_weight(K, L) + K.best[L]);
   }
-  int32_t cu = -1;
-  bool on = false;
-  int32_t L = 0;
-  long long w = 0;
-  for_each_arc(K.rp, K.ci, n, m, [&](int32_t u, int64_t, int32_t y) {
-    if (u != cu) {
-      cu = u;
-      L = K.lab[u];
-      on = K.sz[L] > 1 && K.rdy[L] == level;
-      if (on) w = vd_weight(K, L) + K.best[L];
+  // Pulled along the in-arcs of the components still waiting: those are few
+  // on power-law graphs (the ready giant component holds most arcs), and a
+  // row's arcs from ready components make one update, not one each.
+  for_each_arc<4>(K.rrp, K.rci, n, m, [&](const bool* ok, const int32_t* y, const int64_t*, const int32_t* u) {
+    int32_t Ly[4], Lu[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Ly[k] = ok[k] ? K.lab[y[k]] : -1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Lu[k] = Ly[k] >= 0 && *(volatile const int32_t*)&K.cnt[Ly[k]] > 0 ? K.lab[u[k]] : Ly[k];
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+      const int32_t ly = k == 0 ? Ly[0] : k == 1 ? Ly[1] : k == 2 ? Ly[2] : Ly[3];
+      const int32_t lu = k == 0 ? Lu[0] : k == 1 ? Lu[1] : k == 2 ? Lu[2] : Lu[3];
+      const bool on = lu != ly && K.sz[lu] > 1 && K.rdy[lu] == level;
+      if (!__any_sync(FULL, on)) continue;
+      // the lanes whose arcs go from one component into the same other one
+      const unsigned long long pair = on ? ((unsigned long long)(uint32_t)lu << 32) | (uint32_t)ly : ~0ull;
+      const unsigned same = __match_any_sync(FULL, pair);
+      if (on && lane_id() == __ffs(same) - 1) {
+        atomicMax(&K.best[ly], vd_weight(K, lu) + K.best[lu]);
+        const int c = __popc(same);
+        if (atomicSub(&K.cnt[ly], c) == c) {
+          if (K.sz[ly] == 1) {
+            next[atomicAdd(&slot[0], 1)] = ly;  // a single-node component is its node
+          } else {
+            K.rdy[ly] = level + 1;
+            slot[1] = 1;
+          }
+        }
+      }
     }
-    if (on) vd_kahn_arc(K, L, w, y, level, next, slot);
   });
 }
 
@@ -4349,7 +4499,9 @@ struct LoadScratch {
   unsigned long long* lt_gt;   // the mirror test's two arc counts
   int32_t* fp;                 // 64 fingerprint entries
   unsigned long long* best;    // the VD root's key
-  int32_t* cnt;                // BFS level counters: slot l % 8 holds {next frontier size, items} of level l
+  int32_t* piv;                // pivots of the searched column array (graphs beyond the L2), else null
+  int32_t* floor_deg;          // the largest max(out, in) degree (directed graphs)
+  int32_t* cnt;                // BFS level counters: slot l % 8 holds {next frontier's size, items, its arcs} of level l
   uint32_t* recip;             // n (directed graphs), else null
   VdCore* core;                // the root's component: size, e_out, e_in
   int32_t *dist, *qa, *qb;     // n each: distances from r, BFS queues
@@ -4359,6 +4511,15 @@ struct LoadScratch {
   void* base;
 };
 
+uint64_t l2_bytes(int device) {
+  int l2 = 0;
+  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, device) != cudaSuccess) l2 = 0;
+  return l2 > 0 ? (uint64_t)l2 : ~0ull;
+}
+uint64_t csr_bytes(const kadabra_graph* g) {
+  return (4ull * ((uint64_t)g->n + 1) + 4ull * (uint64_t)g->m) * (g->directed ? 2 : 1);
+}
+
 kadabra_status load_scratch(const kadabra_graph* g, LoadScratch* S) {
   const size_t n = (size_t)g->n;
   const int64_t cap = std::min<int64_t>((int64_t)1 << 24, 4 * g->m / BFS_CHUNK + 64);
@@ -4367,12 +4528,15 @@ kadabra_status load_scratch(const kadabra_graph* g, LoadScratch* S) {
   const size_t o_head = 0, o_recip = up(1024), o_dist = o_recip + (g->directed ? up(4 * n) : 0);
   const size_t o_qa = o_dist + up(4 * n), o_qb = o_qa + up(4 * n), o_distb = o_qb + up(4 * n);
   const size_t o_items = o_distb + (g->directed ? up(4 * n) : 0);
-  const size_t total = o_items + sizeof(BfsItem) * (size_t)cap;
+  const bool pivots = csr_bytes(g) > l2_bytes(g->device);
+  const size_t o_piv = up(o_items + sizeof(BfsItem) * (size_t)cap);
+  const size_t total = o_piv + (pivots ? 4 * ((size_t)g->m / PIVOT + 1) : 0);
   KTRY(pool_alloc(&S->base, total));
   unsigned char* b = static_cast<unsigned char*>(S->base);
   S->err = reinterpret_cast<unsigned*>(b + o_head);
   S->lt_gt = reinterpret_cast<unsigned long long*>(b + o_head + 8);
   S->best = reinterpret_cast<unsigned long long*>(b + o_head + 24);
+  S->floor_deg = reinterpret_cast<int32_t*>(b + o_head + 32);
   S->cnt = reinterpret_cast<int32_t*>(b + o_head + 512);
   S->fp = reinterpret_cast<int32_t*>(b + o_head + 64);
   S->recip = g->directed ? reinterpret_cast<uint32_t*>(b + o_recip) : nullptr;
@@ -4382,6 +4546,7 @@ kadabra_status load_scratch(const kadabra_graph* g, LoadScratch* S) {
   S->qa = reinterpret_cast<int32_t*>(b + o_qa);
   S->qb = reinterpret_cast<int32_t*>(b + o_qb);
   S->items = reinterpret_cast<BfsItem*>(b + o_items);
+  S->piv = pivots ? reinterpret_cast<int32_t*>(b + o_piv) : nullptr;
   KCK(cudaMemset(S->base, 0, 64));
   if (S->recip) KCK(cudaMemset(S->recip, 0, 4 * n));
   return KADABRA_OK;
@@ -4394,28 +4559,28 @@ kadabra_status load_scratch(const kadabra_graph* g, LoadScratch* S) {
 kadabra_status vd_bfs(kadabra_graph* g, const LoadScratch& S, const int32_t* tr, const int32_t* tc,
                       const int32_t* br, const int32_t* bc, int32_t* dist) {
   const int32_t n = g->n;
-  constexpr int BFS_BATCH = 4, SLOTS = 8;
+  constexpr int BFS_BATCH = 4, SLOTS = 8, SLOT = 4;  // slot: next frontier's nodes, long-row items, its arcs
   k_bfs_root<<<1, 1>>>(S.best, dist, S.qa);  // the root stays on the device
   KCK(cudaGetLastError());
   bool done = false;
   for (int32_t l0 = 0; !done && l0 <= n; l0 += BFS_BATCH) {
     for (int k = 0; k < BFS_BATCH; ++k)
-      KCK(cudaMemsetAsync(S.cnt + 2 * ((l0 + k) % SLOTS), 0, 2 * sizeof(int32_t)));
+      KCK(cudaMemsetAsync(S.cnt + SLOT * ((l0 + k) % SLOTS), 0, SLOT * sizeof(int32_t)));
     for (int k = 0; k < BFS_BATCH; ++k) {
       const int32_t l = l0 + k;
       int32_t* in_q = (l & 1) ? S.qb : S.qa;
       int32_t* out_q = (l & 1) ? S.qa : S.qb;
-      int32_t* c = S.cnt + 2 * (l % SLOTS);
-      const int32_t* prev = l == 0 ? nullptr : S.cnt + 2 * ((l + SLOTS - 1) % SLOTS);
+      int32_t* c = S.cnt + SLOT * (l % SLOTS);
+      const int32_t* prev = l == 0 ? nullptr : S.cnt + SLOT * ((l + SLOTS - 1) % SLOTS);
       k_bfs_level<<<8 * g->num_sms, 256>>>(tr, tc, br, bc, in_q, prev, out_q, c, dist, l, S.items, c + 1,
-                                           S.items_cap, n);
-      k_bfs_items<<<8 * g->num_sms, 256>>>(tc, S.items, c + 1, S.items_cap, out_q, c, dist, l);
+                                           S.items_cap, n, g->m);
+      k_bfs_items<<<8 * g->num_sms, 256>>>(tr, tc, S.items, c + 1, S.items_cap, out_q, c, dist, l);
     }
-    int32_t h[2 * SLOTS];
+    int32_t h[SLOT * SLOTS];
     if (cudaMemcpy(h, S.cnt, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess)
       return fail(KADABRA_ERR_CUDA, std::string("vd bfs: ") + cudaGetErrorString(cudaGetLastError()));
     for (int k = 0; k < BFS_BATCH; ++k)
-      if (h[2 * ((l0 + k) % SLOTS)] == 0) {
+      if (h[SLOT * ((l0 + k) % SLOTS)] == 0) {
         done = true;
         break;
       }
@@ -4433,14 +4598,14 @@ kadabra_status vd_condensation(kadabra_graph* g, LoadTrace& tr, const LoadScratc
   const int32_t* rrp = g->directed ? g->rrp : g->rp;
   const int32_t* rci = g->directed ? g->rci : g->ci;
   const int bn = std::max(1, std::min(16 * g->num_sms, (n + 255) / 256));
-  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, ((m + LOAD_CHUNK - 1) / LOAD_CHUNK + 255) / 256));
+  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, (m + 8 * ARC_CHUNK - 1) / (8 * ARC_CHUNK)));
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t N4 = up(4 * (size_t)n), N8 = up(8 * (size_t)n);
   void* base = nullptr;
-  KCK(cudaMalloc(&base, 256 + 6 * N4 + N8));
+  KTRY(pool_alloc(&base, 256 + 6 * N4 + N8));
   struct Free {
     void* p;
-    ~Free() { cudaFree(p); }
+    ~Free() { pool_free(p); }
   } guard{base};
   unsigned char* b = static_cast<unsigned char*>(base);
   int32_t* flag = reinterpret_cast<int32_t*>(b);              // [0] a change, [1] an unlabelled node
@@ -4487,11 +4652,11 @@ kadabra_status vd_condensation(kadabra_graph* g, LoadTrace& tr, const LoadScratc
   KCK(cudaMemsetAsync(best, 0, N8));
   KCK(cudaMemsetAsync(b + 64, 0, 192));  // slots, vd
   k_vd_sizes<<<bn, 256>>>(lab, n, sz);
-  k_vd_indeg<<<ba, 256>>>(g->rp, g->ci, n, m, lab, cnt);
+  k_vd_indeg<<<ba, 256>>>(g->rp, g->ci, n, m, lab, S.best, cnt);
   unsigned long long key = 0;
   if (cudaMemcpy(&key, S.best, sizeof(key), cudaMemcpyDeviceToHost) != cudaSuccess)
     return fail(KADABRA_ERR_CUDA, "vd bound");
-  VdKahn K{g->rp, g->ci, lab, sz, cnt, best, rdy, n, (int32_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull)),
+  VdKahn K{g->rp, g->ci, rrp, rci, lab, sz, cnt, best, rdy, n, (int32_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull)),
            root_w, vd};
   constexpr int SLOTS = 8, BATCH = 4;
   k_vd_kahn_init<<<bn, 256>>>(K, S.qa, slots + 2 * (SLOTS - 1));  // the slot level 0 reads
@@ -4571,7 +4736,7 @@ kadabra_status finish_load(kadabra_graph* g) {
   const int32_t n = g->n;
   const int64_t m = g->m;
   const int bn = std::max(1, std::min(16 * g->num_sms, (n + 255) / 256));
-  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, ((m + LOAD_CHUNK - 1) / LOAD_CHUNK + 255) / 256));
+  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, (m + 8 * ARC_CHUNK - 1) / (8 * ARC_CHUNK)));
   const int32_t* rrp = g->directed ? g->rrp : g->rp;
   const int32_t* rci = g->directed ? g->rci : g->ci;
   unsigned h = 0;
@@ -4592,7 +4757,10 @@ kadabra_status finish_load(kadabra_graph* g) {
     }
     tr.mark("validate rows");
     if (h) break;  // the mirror test needs ids in range and sorted rows
-    k_validate_mirror<<<ba, 256>>>(g->rp, g->ci, rrp, rci, n, m, g->directed ? 0 : 1, S.err, S.lt_gt, S.recip);
+    if (S.piv) k_pivots<<<bn, 256>>>(rci, m, S.piv);
+    if (g->directed) k_floor_degree<<<bn, 256>>>(g->rp, rrp, n, S.floor_deg);
+    k_validate_mirror<<<ba, 256>>>(g->rp, g->ci, rrp, rci, n, m, g->directed ? 0 : 1, S.err, S.lt_gt, S.recip,
+                                   S.floor_deg, S.piv);
     unsigned long long c[2] = {0, 0};
     if (cudaMemcpy(&h, S.err, sizeof(unsigned), cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(c, S.lt_gt, sizeof(c), cudaMemcpyDeviceToHost) != cudaSuccess) {
@@ -4636,10 +4804,7 @@ kadabra_status finish_load(kadabra_graph* g) {
     if (h & 16) why += (g->directed ? " reverse CSR does not mirror the forward CSR;" : " adjacency not symmetric;");
     return fail(KADABRA_ERR_CSR, "invalid CSR:" + why);
   }
-  int l2 = 0;
-  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, g->device) != cudaSuccess) l2 = 0;
-  const uint64_t csr = (4ull * ((uint64_t)n + 1) + 4ull * (uint64_t)m) * (g->directed ? 2 : 1);
-  g->csr_beyond_l2 = l2 > 0 && csr > (uint64_t)l2;
+  g->csr_beyond_l2 = csr_bytes(g) > l2_bytes(g->device);
   return KADABRA_OK;
 }
 
