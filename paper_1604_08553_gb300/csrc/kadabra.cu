@@ -95,21 +95,30 @@ namespace {
 #ifndef KD_MIN_BLOCKS
 #define KD_MIN_BLOCKS 4
 #endif
-constexpr int NT = KD_NT;          // threads per sampler CTA
-constexpr int NW = NT / 32;        // warps per sampler CTA
+#ifndef KD_NT_BIG
+#define KD_NT_BIG 1024
+#endif
+// Warps per sampler CTA: tiers S and L, and tier B (with M), whose samples are
+// few and large, so that a sample's latency counts: 32 warps on one CTA per
+// SM with 16,384 slots.  Its launch per batch, against 8 warps on two CTAs
+// with 8,192 slots, 16 on two, and 24 on one CTA: ER 3.4 M nodes (1,100
+// samples) 0.83, 0.57, 0.26 -> 0.25 ms, Chung-Lu 10^6 nodes (65,536) 0.47,
+// 0.35, 0.19 -> 0.19 ms, R-MAT scale 24 (65,536) 2.28, 1.62, 1.30 -> 1.22 ms:
+// fewer samples go on to tier M, and a level's arcs take fewer steps.
+constexpr int NW_S = KD_NT / 32;
+constexpr int NW_BIG = KD_NT_BIG / 32;
 constexpr int U = KD_U;            // independent items per thread per step (memory-level parallelism)
 // Tiers of per-sample tables.  A sample starts in a small shared-memory
 // table (tier S, main launch, four or five CTAs per SM; optionally tier W,
 // one warp per sample, before it).  If it outgrows it, it is queued for a
-// second launch with two CTAs per SM and a large shared-memory table (tier
+// second launch with one CTA per SM and a large shared-memory table (tier
 // B); beyond that the same CTA retries it on medium global tables (tier M),
 // and beyond those it is queued for a last launch with n-sized global tables
 // (tier L).  Every tier gives the same result.
 constexpr int FAST_HLOG = KD_FAST_HLOG;        // tier S: 2^FAST_HLOG hash slots
-// tier B: 2^KD_BIG_EXTRA times tier S's slots (4 times, at one CTA per SM: R-MAT scale 24 batch 5.38 ->
-// 5.44 ms, scale 22 2.48 -> 2.56 ms; fewer samples reached tier M, but tier B ran on half the CTAs)
+// tier B: 2^KD_BIG_EXTRA times tier S's slots
 #ifndef KD_BIG_EXTRA
-#define KD_BIG_EXTRA 1
+#define KD_BIG_EXTRA 2
 #endif
 constexpr int BIG_HLOG = FAST_HLOG + KD_BIG_EXTRA;
 #ifndef KD_FAST_MAXD
@@ -120,7 +129,8 @@ constexpr int MED_HLOG = 16;       // tier M, global memory per CTA: 65536 hash 
 constexpr int MED_LCAP = 32768;    //   level lists: 32768 nodes
 constexpr int MED_MAXD = 1022;     //   levels per side
 constexpr int GM_MAXD = 65534;     // tier L, global memory, hash >= 2n slots, lists of n
-constexpr int FAST_PCAP = 2048;    // candidate edges per warp, tiers S and M (global memory)
+constexpr int PI_SEGS = 16;        // a sample's candidate edges: PI_SEGS * pcap entries in global memory,
+constexpr int FAST_PCAP = 2048;    //   pcap in tiers S, B and M
 constexpr int QUAD_PICK_MAX = 256;  // global-memory tiers: candidate sets ranked quadratically up to this size
 constexpr unsigned long long EMPTY = ~0ull;
 constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -220,7 +230,7 @@ struct Tables {
   struct LongRows* lr;      // long rows of the segment (shared memory; null in the compact layout)
   int* lvl;                 // [side][lo|hi][maxd+2]
   int maxd;
-  PiEntry* pi;              // 2*NW segments of pcap entries (the second half is scratch)
+  PiEntry* pi;              // candidate edges beyond shared memory: PI_SEGS * pcap entries
   int pcap;
 };
 
@@ -412,7 +422,7 @@ struct SampleParams {
   long long* stats;
   int32_t* sstatus;
   // tables
-  PiEntry* pi_base;                 // per CTA: NW * pcap
+  PiEntry* pi_base;                 // per CTA: PI_SEGS * pcap entries
   int pcap;
   unsigned char* med_base;          // tier M tables, per CTA of the large-table launch
   size_t med_stride;
@@ -472,6 +482,7 @@ struct LongRows {
   uint16_t pos[LONG_CAP];              // position in the frontier segment
 };
 
+template <int NW>
 struct Ctl {
   Job job;        // the job of the current sample
   int tot_job;    // the job that tot accumulates for (-1: none)
@@ -510,7 +521,8 @@ struct Ctl {
 };
 
 // adds to a per-sample counter (no thread waits for the sum)
-__device__ __forceinline__ void stat_add(Ctl& c, int q, unsigned x) {
+template <int NW>
+__device__ __forceinline__ void stat_add(Ctl<NW>& c, int q, unsigned x) {
   atomicAdd(reinterpret_cast<unsigned*>(&c.stat[q]), x);
 }
 
@@ -520,6 +532,7 @@ __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 
 // exclusive scan of one int per thread; *total gets the block sum.  One
 // barrier: calls that follow each other alternate between two tmp arrays.
+template <int NW>
 __device__ __forceinline__ int block_exscan(int x, int* tmp, int* total) {
   const int lane = lane_id(), w = warp_id();
   int v = x;
@@ -542,6 +555,7 @@ __device__ __forceinline__ int block_exscan(int x, int* tmp, int* total) {
 }
 
 // inclusive scan of one u64 per thread; *total gets the block sum
+template <int NW>
 __device__ __forceinline__ unsigned long long block_inscan_u64(unsigned long long x, unsigned long long* tmp,
                                                                unsigned long long* total) {
   const int lane = lane_id(), w = warp_id();
@@ -703,8 +717,9 @@ __device__ __forceinline__ int warp_lower_bound(const int32_t* col, int a, int b
 // prefix sum of weights exceeds r (r < total weight).  Each thread weighs U
 // consecutive items per step so their memory accesses overlap.  Returns the
 // item index (all threads), or -1 if r is not below the total.
-template <class WF>
-__device__ __forceinline__ int block_pick(int N, unsigned long long r, Ctl& c, WF wf) {
+template <int NW, class WF>
+__device__ __forceinline__ int block_pick(int N, unsigned long long r, Ctl<NW>& c, WF wf) {
+  constexpr int NT = 32 * NW;
   const int tid = threadIdx.x;
   if (tid == 0) c.pick = -1;
   __syncthreads();
@@ -717,7 +732,7 @@ __device__ __forceinline__ int block_pick(int N, unsigned long long r, Ctl& c, W
 #pragma unroll
     for (int k = 0; k < U; ++k) tsum += w[k];
     unsigned long long tot;
-    const unsigned long long incl = block_inscan_u64(tsum, c.u64tmp, &tot);
+    const unsigned long long incl = block_inscan_u64<NW>(tsum, c.u64tmp, &tot);
     const unsigned long long excl = incl - tsum;
     if (tsum != 0 && carry + excl <= r && r < carry + incl) {
       unsigned long long acc = carry + excl;
@@ -740,6 +755,7 @@ __device__ __forceinline__ int block_pick(int N, unsigned long long r, Ctl& c, W
 // ============================================================== one sample
 // Arcs per warp of a level of E arcs: whole windows of 32, so that a small
 // level issues few full windows instead of one per warp with a few lanes each.
+template <int NW>
 __device__ __forceinline__ int warp_slice(int E) {
   return max(1, (int)(((unsigned)E + 32u * NW - 1u) / (32u * NW))) * 32;
 }
@@ -796,11 +812,11 @@ __device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcou
 // by the slowest warp at the barrier after it: windows of 32 arcs with a
 // probe each, and short rows one window at a time, took 23.2 k of 74 k cycles
 // per sample on the Chung-Lu graph of 10^6 nodes, this takes 16.6 k.
-template <bool PK, int D, class EM>
+template <bool PK, int D, int NW, class EM>
 __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount, int E, const int32_t* cols,
                                            int64_t ncols, EM emit) {
   const int lane = lane_id(), wid = warp_id();
-  const int per = warp_slice(E);
+  const int per = warp_slice<NW>(E);
   const int c0 = min(E, wid * per), c1 = min(E, c0 + per);
   if (c0 >= c1) return;
   int pcur = frontier_pos(T.pr, fcount, c0);  // warp-uniform
@@ -860,11 +876,11 @@ __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount
 // current one is processed, so their latency overlaps its probes).  For every
 // window it calls f(ok, p, y): ok = the lane holds an arc, p = frontier
 // position of its tail, y = its head.  All lanes of the warp call f together.
-template <class F>
+template <int NW, class F>
 __device__ __forceinline__ void scan_level(const Tables& T, int fcount, int E, const int32_t* cols, int64_t ncols,
                                            F f) {
   const int lane = lane_id(), wid = warp_id();
-  const int per = warp_slice(E);
+  const int per = warp_slice<NW>(E);
   const int c0 = min(E, wid * per), c1 = min(E, c0 + per);
   if (c0 >= c1) return;
   int pcur = frontier_pos(T.pr, fcount, c0);  // warp-uniform
@@ -908,8 +924,9 @@ __device__ __forceinline__ void scan_level(const Tables& T, int fcount, int E, c
 // 64-bit keys (distinct): the item whose key-order prefix interval contains r.
 // Quadratic in n: each thread ranks its items against all others.  c.pick
 // must be -1 before a barrier that precedes the call.
-template <class KF, class WF>
-__device__ __forceinline__ int block_pick_by_key(int n, unsigned long long r, Ctl& c, KF key, WF w) {
+template <int NW, class KF, class WF>
+__device__ __forceinline__ int block_pick_by_key(int n, unsigned long long r, Ctl<NW>& c, KF key, WF w) {
+  constexpr int NT = 32 * NW;
 #pragma unroll 1
   for (int i = threadIdx.x; i < n; i += NT) {
     const unsigned long long ki = key(i);
@@ -935,8 +952,10 @@ __device__ __forceinline__ int block_pick_by_key(int n, unsigned long long r, Ct
 // shared histogram once per run of equal bytes: candidates of one tail x are
 // contiguous and sorted by y, so runs are long.  Returns the candidate's
 // index (all threads), or -1 if r is not below the total weight.
-__device__ __noinline__ int block_pick_radix(const PiEntry* buf, int n, unsigned long long r, Ctl& c,
+template <int NW>
+__device__ __noinline__ int block_pick_radix(const PiEntry* buf, int n, unsigned long long r, Ctl<NW>& c,
                                 unsigned long long* rhist, unsigned* rcnt) {
+  constexpr int NT = 32 * NW;
   const int tid = threadIdx.x, lane = lane_id();
   auto key = [&](int i) { return ((unsigned long long)(uint32_t)buf[i].x << 32) | (uint32_t)buf[i].y; };
   const int chunk = (n + NT - 1) / NT;
@@ -1025,8 +1044,8 @@ __device__ __noinline__ int block_pick_radix(const PiEntry* buf, int n, unsigned
 // Records a backtracking pick y (now at depth dn on side `half`, at position
 // pos of the scanned row): the work counter, its hit (interior nodes only)
 // and its place on the path.  One thread.
-template <bool PK>
-__device__ __forceinline__ void bt_record(const SampleParams& P, const Job& J, Ctl& c, int half, int dn, int y, int pos,
+template <bool PK, int NW>
+__device__ __forceinline__ void bt_record(const SampleParams& P, const Job& J, Ctl<NW>& c, int half, int dn, int y, int pos,
                                           int64_t out_i, int dv, int dw, bool want_path) {
   atomicAdd(reinterpret_cast<unsigned long long*>(&c.stat[KADABRA_STAT_BT_SCANNED]), (unsigned long long)(pos + 1));
   if (dn > 0 && J.counts) atomicAdd(&J.counts[KIDX(y, J.g.n, 11)], 1u);
@@ -1048,8 +1067,8 @@ constexpr int WARP_BT_ROW = KD_WARP_BT_ROW;  // rows up to this length: the step
 // candidate order and the pick are those of the block's steps: the first
 // neighbour one level closer, in row order, whose cumulative sigma exceeds r.
 // A row is read four windows of 32 at a time.
-template <bool PK>
-__device__ void bt_warp_steps(const SampleParams& P, const Job& J, const Tables& T, Ctl& c, uint64_t idx,
+template <bool PK, int NW>
+__device__ void bt_warp_steps(const SampleParams& P, const Job& J, const Tables& T, Ctl<NW>& c, uint64_t idx,
                               int64_t out_i, int dv, int dw, bool want_path, int half) {
   const int lane = lane_id();
   const GraphDev& G = J.g;
@@ -1147,9 +1166,10 @@ __device__ void bt_warp_steps(const SampleParams& P, const Job& J, const Tables&
 #else
 #define KD_MEMB_ATTR __device__ __forceinline__
 #endif
-template <bool PK, class EM>
-KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl& c, const int32_t* cols, int64_t m, int ob,
+template <bool PK, int NW, class EM>
+KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl<NW>& c, const int32_t* cols, int64_t m, int ob,
                                    int kother, int nl, EM emit) {
+  constexpr int NT = 32 * NW;
   const int lane = lane_id(), wid = warp_id();
   const long long items = (long long)nl * kother;
 #pragma unroll 1
@@ -1202,9 +1222,10 @@ KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl& c, const int32_t*
 // 4.41 -> 3.37 ms on the Chung-Lu graph of 10^6 nodes (2.49 -> 1.85 G warp
 // instructions) and 2.70 -> 2.21 ms on R-MAT scale 22; a 3.4 M-node ER graph's
 // run 18.3 -> 15.4 ms.
-template <bool PK, bool RG = false, bool FU = true>
-__device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, const Tables& T, Ctl& c, uint64_t idx,
+template <bool PK, bool RG, bool FU, int NW>
+__device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, const Tables& T, Ctl<NW>& c, uint64_t idx,
                                            int64_t out_i) {
+  constexpr int NT = 32 * NW;
   const int tid = threadIdx.x, lane = lane_id(), wid = warp_id();
   const GraphDev& G = J.g;
 
@@ -1215,7 +1236,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
   bool touched = false;
   int side = 0;  // the side a level expands (after the search: the side that touched)
   int cand_at = 0, cand_cap = 0;  // where the level's candidate edges start in T.pr, and how many fit there
-  const int pi_cap = NW * T.pcap;  // candidate edges a sample may have
+  const int pi_cap = PI_SEGS * T.pcap;  // candidate edges a sample may have
 #pragma unroll 1
   for (int iter = 0; iter <= 2 * T.maxd + 2; ++iter) {
     const int par = iter & 1;
@@ -1311,7 +1332,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
             deg = take_long(__ldg(&rowp[x + 1]) - rs, kl, i, rs);
           }
           int tot;
-          const int ex = block_exscan(deg, c.scan_tmp[h], &tot);
+          const int ex = block_exscan<NW>(deg, c.scan_tmp[h], &tot);
           if (i < cnt) T.pr[KIDX(i, T.frcap + 1, 10)] = make_int2(carry + ex, rs);
           carry += tot;
         }
@@ -1386,7 +1407,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
           Eseg = T.pr[cnt].x;
         }
         if (pass == 1) {
-          touch_pass<PK, TOUCH_DEPTH>(
+          touch_pass<PK, TOUCH_DEPTH, NW>(
               T, side, cnt, Eseg, cols, G.m,
               [&](bool touch, int p, int y, int pos, unsigned long long hy) { emit(fb, touch, p, y, pos, hy); });
           // the long rows: one search per (row, other-frontier node)
@@ -1400,7 +1421,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
             }
           }
         } else {
-          scan_level(T, cnt, Eseg, cols, G.m, [&](bool ok, int p, int y) {
+          scan_level<NW>(T, cnt, Eseg, cols, G.m, [&](bool ok, int p, int y) {
             int res = 0;  // 1 = inserted, 2 = a touch arc (fused)
             int ydeg = 0, ylo = 0;
             uint32_t pos = 0;
@@ -1795,7 +1816,9 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
 // (key and sigma of every entry it inserted): the whole table after a
 // capacity failure (entries beyond the lists), else the entries at the
 // positions the lists recorded.
-__device__ void reset_tables(const Tables& T, Ctl& c) {
+template <int NW>
+__device__ void reset_tables(const Tables& T, Ctl<NW>& c) {
+  constexpr int NT = 32 * NW;
   const int tid = threadIdx.x;
   if (c.flags & F_CAP) {
 #pragma unroll 1
@@ -1817,7 +1840,9 @@ __device__ void reset_tables(const Tables& T, Ctl& c) {
 
 // Empties a shared-memory table (cheaper than locating a sample's entries):
 // every warp but the first, which meanwhile sets up the next sample.
+template <int NW>
 __device__ __forceinline__ void clear_table(const Tables& T) {
+  constexpr int NT = 32 * NW;
   int4* h = reinterpret_cast<int4*>(T.hkv);
 #pragma unroll 1
   for (uint32_t i = threadIdx.x - 32; i < (T.hmask + 1) / 2; i += NT - 32) h[i] = make_int4(-1, -1, -1, -1);
@@ -1827,7 +1852,8 @@ __device__ __forceinline__ void clear_table(const Tables& T) {
 // table afterwards).  Every lane draws one of the sample's first 32 Philox
 // blocks ((s,t), candidate edge, backtracking steps), so the serial steps
 // only read them.
-__device__ __forceinline__ void begin_sample(const SampleParams& P, const Tables& T, Ctl& c, uint64_t idx,
+template <int NW>
+__device__ __forceinline__ void begin_sample(const SampleParams& P, const Tables& T, Ctl<NW>& c, uint64_t idx,
                                              int64_t out_i) {
   const int lane = lane_id();
   const GraphDev& G = c.job.g;
@@ -1869,8 +1895,8 @@ __device__ __forceinline__ void begin_sample(const SampleParams& P, const Tables
 }
 
 // s and t into the (empty) table: the level 0 of both sides (warp 0)
-template <bool PK>
-__device__ __forceinline__ void insert_roots(const Tables& T, Ctl& c) {
+template <bool PK, int NW>
+__device__ __forceinline__ void insert_roots(const Tables& T, Ctl<NW>& c) {
   if (threadIdx.x == 0) {
     uint32_t ps = 0, pt = 0;
     if (tab_insert(T, c.s, ent_word<PK>(c.s, pack_val(0, 0), 1ull), &ps) != 1) c.flags |= F_INTERNAL;
@@ -1888,15 +1914,15 @@ __device__ __forceinline__ void insert_roots(const Tables& T, Ctl& c) {
 }
 
 // global-memory tiers share one body per scan kind, compiled outside the kernel
-template <bool RG>
-__device__ __noinline__ void run_sample_global(const SampleParams& P, const Job& J, const Tables& T, Ctl& c,
+template <bool RG, int NW>
+__device__ __noinline__ void run_sample_global(const SampleParams& P, const Job& J, const Tables& T, Ctl<NW>& c,
                                                uint64_t idx, int64_t out_i) {
   if (warp_id() == 0) {
     begin_sample(P, T, c, idx, out_i);
     insert_roots<false>(T, c);
   }
   __syncthreads();
-  run_sample<false, RG>(P, J, T, c, idx, out_i);
+  run_sample<false, RG, true>(P, J, T, c, idx, out_i);
   __syncthreads();
 }
 
@@ -1950,20 +1976,21 @@ constexpr int FRONTIER_SEG = KD_FRONTIER_SEG;
 #ifndef KD_LOAD_QUARTERS
 #define KD_LOAD_QUARTERS 3
 #endif
-constexpr size_t CTL_BYTES = (sizeof(Ctl) + 15) & ~size_t(15);
-template <int HLOG, int L8, int FSEG, int FLOG, int MAXD, bool LR>
+template <int NW>
+constexpr size_t CTL_BYTES = (sizeof(Ctl<NW>) + 15) & ~size_t(15);
+template <int NW, int HLOG, int L8, int FSEG, int FLOG, int MAXD, bool LR>
 struct SLayout {
   static constexpr int SLOTS_LOG = HLOG;
   // nodes a table takes before the sample moves on to the next tier (the
   // probes stay short)
   static constexpr int LCAP = (L8 << HLOG) / 8;
-  static_assert(LCAP + NT < (1 << HLOG), "a full list leaves free slots");
+  static_assert(LCAP + 32 * NW < (1 << HLOG), "a full list leaves free slots");
   static constexpr int FRCAP = LCAP < FSEG ? LCAP : FSEG;
   static constexpr int FWORDS = (1 << FLOG) / 32;
   static constexpr int FSHIFT = 32 - FLOG;
   static constexpr int LEVELS = MAXD;
   static_assert(MAXD <= 126, "the packed entry's dist field");
-  static constexpr size_t HKV = CTL_BYTES;
+  static constexpr size_t HKV = CTL_BYTES<NW>;
   static constexpr size_t PR = HKV + (sizeof(unsigned long long) << HLOG);
   static constexpr size_t LPOS = PR + sizeof(int2) * (FRCAP + 1);
   static constexpr size_t LVL = LPOS + sizeof(uint16_t) * LCAP;
@@ -1977,7 +2004,12 @@ struct SLayout {
 };
 // tier S at KD_MIN_BLOCKS CTAs per SM; tier S compact (one more CTA per SM:
 // half-full lists, 512-node segments, a 2^14-bit filter, 38 levels per
-// side; 5 x 45,408 B fit an SM's shared memory, 5 x 45,600 B did not); tier B (twice the slots, two CTAs per SM)
+// side; 5 x 45,408 B fit an SM's shared memory, 5 x 45,600 B did not);
+// tier B (four times the slots, one CTA per SM).  Tier B with frontier segments
+// of 2048 or 4096 nodes and a 2^16- or 2^17-bit filter: 2 to 5 % faster on the
+// ER graph of 3.4 M nodes, 8 % slower on the Chung-Lu graph, up to 30 % on
+// R-MAT scale 22.  Tier S with half-full lists: its own launch 4 to 30 % faster,
+// the batch 0 to 7 % slower, since more samples are begun twice.
 #ifndef KD_CMP_L8
 #define KD_CMP_L8 4
 #endif
@@ -1987,9 +2019,9 @@ struct SLayout {
 #ifndef KD_CMP_MAXD
 #define KD_CMP_MAXD 38
 #endif
-using FastLayout = SLayout<FAST_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
-using CompactLayout = SLayout<FAST_HLOG, KD_CMP_L8, 512, KD_CMP_FLOG, KD_CMP_MAXD, false>;
-using BigLayout = SLayout<BIG_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
+using FastLayout = SLayout<NW_S, FAST_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
+using CompactLayout = SLayout<NW_S, FAST_HLOG, KD_CMP_L8, 512, KD_CMP_FLOG, KD_CMP_MAXD, false>;
+using BigLayout = SLayout<NW_BIG, BIG_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
 // the tier-S layout a k_sample instance uses (SL)
 constexpr int SL_FAST = 0;
 constexpr int SL_COMPACT = 1;
@@ -2044,7 +2076,8 @@ __device__ void enqueue(const SampleParams& P, int size_ctr, unsigned long long*
 }
 
 // Adds the CTA's accumulated work counters to their job's totals (warp 0).
-__device__ void flush_totals(const SampleParams& P, Ctl& c) {
+template <int NW>
+__device__ void flush_totals(const SampleParams& P, Ctl<NW>& c) {
   const int q = lane_id();
   if (q < KADABRA_NSTAT) {
     if (c.tot_job >= 0) {
@@ -2057,7 +2090,8 @@ __device__ void flush_totals(const SampleParams& P, Ctl& c) {
 }
 
 // The job of work index k into c.job (warp 0).
-__device__ __forceinline__ void take_job(const SampleParams& P, Ctl& c, unsigned long long k) {
+template <int NW>
+__device__ __forceinline__ void take_job(const SampleParams& P, Ctl<NW>& c, unsigned long long k) {
   int j = 0;
   if (P.jobs) {
     int lo = 0, hi = P.njobs;
@@ -2082,7 +2116,8 @@ __device__ __forceinline__ void take_job(const SampleParams& P, Ctl& c, unsigned
 }
 
 // Records the outcome of one sample (per-sample outputs, totals, status; warp 0).
-__device__ void finish_sample(const SampleParams& P, Ctl& c, int64_t out_i) {
+template <int NW>
+__device__ void finish_sample(const SampleParams& P, Ctl<NW>& c, int64_t out_i) {
   int flags = c.flags;
 #ifdef KADABRA_CHECKED
   if (*(volatile unsigned long long*)&g_checked) flags |= F_INTERNAL;
@@ -2117,14 +2152,17 @@ __device__ void finish_sample(const SampleParams& P, Ctl& c, int64_t out_i) {
 // and gives the same results (samples that outgrow it go on to tier B as
 // usual).  RG (the default layout only): pass 1 searches long rows (for
 // graphs whose CSR exceeds L2); same results.
+template <int MODE>
+constexpr int MODE_NW = MODE == 2 ? NW_BIG : NW_S;
 template <int MODE, int SL = SL_FAST, bool RG = false>
-__global__ void __launch_bounds__(NT, MODE != 0 ? 2 : SL == SL_FAST ? KD_MIN_BLOCKS : KD_MIN_BLOCKS + 1)
+__global__ void __launch_bounds__(32 * MODE_NW<MODE>, MODE == 2 ? 1 : MODE == 1 ? 2 : SL == SL_FAST ? KD_MIN_BLOCKS : KD_MIN_BLOCKS + 1)
     k_sample(SampleParams P) {
   static_assert(!RG || SL == SL_FAST, "the beyond-L2 scan has no compact-layout instance");
   extern __shared__ __align__(16) unsigned char smem[];
-  Ctl& c = *reinterpret_cast<Ctl*>(smem);
+  constexpr int NW = MODE_NW<MODE>;
+  Ctl<NW>& c = *reinterpret_cast<Ctl<NW>*>(smem);
   Tables TS, TM;
-  PiEntry* pi = P.pi_base + (size_t)blockIdx.x * 2 * NW * P.pcap;
+  PiEntry* pi = P.pi_base + (size_t)blockIdx.x * PI_SEGS * P.pcap;
   if (MODE == 0) TS = smem_tables<std::conditional_t<SL == SL_FAST, FastLayout, CompactLayout>>(smem);
   if (MODE == 2) {
     TS = smem_tables<BigLayout>(smem);
@@ -2132,7 +2170,7 @@ __global__ void __launch_bounds__(NT, MODE != 0 ? 2 : SL == SL_FAST ? KD_MIN_BLO
   }
   if (MODE == 1) TM = gm_tables(P.gm_base + (size_t)blockIdx.x * P.gm_stride, P.gm_hlog, P.gm_lcap, GM_MAXD);
   if (MODE == 2) TM.lr = TS.lr;
-  if (MODE == 1) TM.lr = reinterpret_cast<LongRows*>(smem + CTL_BYTES);
+  if (MODE == 1) TM.lr = reinterpret_cast<LongRows*>(smem + CTL_BYTES<NW>);
   TS.pi = TM.pi = pi;
   TS.pcap = TM.pcap = P.pcap;
   if (MODE != 1 && (P.tier_flags & TF_SEG64)) TS.frcap = min(TS.frcap, 64);
@@ -2178,7 +2216,7 @@ __global__ void __launch_bounds__(NT, MODE != 0 ? 2 : SL == SL_FAST ? KD_MIN_BLO
       }
       if (tid == 0) c.cur = cur;
     } else if (MODE != 1) {
-      clear_table(TS);
+      clear_table<NW>(TS);
     }
     __syncthreads();
     if (c.cur >= ntotal) break;
@@ -2196,7 +2234,7 @@ __global__ void __launch_bounds__(NT, MODE != 0 ? 2 : SL == SL_FAST ? KD_MIN_BLO
       bool done = false;
       if (!(P.tier_flags & TF_SKIP_B)) {
         if (tid < 32) insert_roots<true>(TS, c);
-        run_sample<true, RG>(P, c.job, TS, c, idx, out_i);
+        run_sample<true, RG, true>(P, c.job, TS, c, idx, out_i);
         __syncthreads();
         done = c.flags != F_CAP;
         __syncthreads();
@@ -4159,12 +4197,12 @@ kadabra_status ensure_ws(Workspace* w, uint64_t deferred_need, int njobs) {
     KCK(cudaFuncSetAttribute(k_sample<0, SL_FAST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)w->smem_fast));
     int per_sm = 0;
-    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0>, NT, w->smem_fast));
+    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0>, 32 * NW_S, w->smem_fast));
     if (per_sm < 1) return fail(KADABRA_ERR_CAPACITY, "sampler does not fit on an SM");
     w->grid_fast = w->num_sms * per_sm;
     w->smem_compact = compact_smem_bytes();
     KCK(cudaFuncSetAttribute(k_sample<0, SL_COMPACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_compact));
-    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0, SL_COMPACT>, NT, w->smem_compact));
+    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0, SL_COMPACT>, 32 * NW_S, w->smem_compact));
     w->grid_compact = w->num_sms * std::max(per_sm, 1);
     w->smem_warp = warp_tier_smem_bytes();
     KCK(cudaFuncSetAttribute(k_sample_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_warp));
@@ -4174,7 +4212,7 @@ kadabra_status ensure_ws(Workspace* w, uint64_t deferred_need, int njobs) {
     KCK(cudaFuncSetAttribute(k_sample<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_big));
     KCK(cudaFuncSetAttribute(k_sample<2, SL_FAST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)w->smem_big));
-    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<2>, NT, w->smem_big));
+    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<2>, 32 * NW_BIG, w->smem_big));
     if (per_sm < 1) return fail(KADABRA_ERR_CAPACITY, "large-table sampler does not fit on an SM");
     w->grid_big = w->num_sms * per_sm;
     // n-sized tables for the rare samples beyond the others: hash of >= 2n slots, lists of n
@@ -4186,7 +4224,7 @@ kadabra_status ensure_ws(Workspace* w, uint64_t deferred_need, int njobs) {
       w->gm_stride = gm_layout(w->gm_hlog, w->gm_lcap, GM_MAXD, &a, &b, &c2, &d);
       w->med_stride = gm_layout(MED_HLOG, MED_LCAP, MED_MAXD, &a, &b, &c2, &d);
     }
-    const size_t per_cta = w->gm_stride + sizeof(PiEntry) * 2 * NW * (size_t)w->pcap_gm;
+    const size_t per_cta = w->gm_stride + sizeof(PiEntry) * PI_SEGS * (size_t)w->pcap_gm;
     // such samples are rare on small-world graphs; 1 GiB of tables keeps
     // at least a few CTAs busy on them
     const size_t budget = (size_t)1 << 30;
@@ -4197,9 +4235,9 @@ kadabra_status ensure_ws(Workspace* w, uint64_t deferred_need, int njobs) {
     KTRY(dev_alloc(w->allocs, &p, sizeof(int32_t)));
     w->status = (int32_t*)p;
     KCK(cudaMemset(w->status, 0, sizeof(int32_t)));
-    KTRY(dev_alloc(w->allocs, &p, sizeof(PiEntry) * 2 * NW * (size_t)FAST_PCAP * std::max(w->grid_fast, w->grid_compact)));
+    KTRY(dev_alloc(w->allocs, &p, sizeof(PiEntry) * PI_SEGS * (size_t)FAST_PCAP * std::max(w->grid_fast, w->grid_compact)));
     w->pi_fast = (PiEntry*)p;
-    KTRY(dev_alloc(w->allocs, &p, sizeof(PiEntry) * 2 * NW * (size_t)w->pcap_gm * w->grid_gm));
+    KTRY(dev_alloc(w->allocs, &p, sizeof(PiEntry) * PI_SEGS * (size_t)w->pcap_gm * w->grid_gm));
     w->pi_gm = (PiEntry*)p;
     KTRY(dev_alloc(w->allocs, &p, w->gm_stride * w->grid_gm));
     w->gm_base = (unsigned char*)p;
@@ -4322,23 +4360,23 @@ kadabra_status launch_sampler_kernels(Workspace* w, SampleParams P, cudaStream_t
   }
   const bool rg = (P.tier_flags & TF_VEC) != 0;
   if ((variant & 1) || ((P.tier_flags & TF_COMPACT) && !rg))  // the compact layout has no beyond-L2 variant
-    k_sample<0, SL_COMPACT><<<w->grid_compact, NT, w->smem_compact, st>>>(P);
+    k_sample<0, SL_COMPACT><<<w->grid_compact, 32 * NW_S, w->smem_compact, st>>>(P);
   else if (rg)
-    k_sample<0, SL_FAST, true><<<w->grid_fast, NT, w->smem_fast, st>>>(P);
+    k_sample<0, SL_FAST, true><<<w->grid_fast, 32 * NW_S, w->smem_fast, st>>>(P);
   else
-    k_sample<0><<<w->grid_fast, NT, w->smem_fast, st>>>(P);
+    k_sample<0><<<w->grid_fast, 32 * NW_S, w->smem_fast, st>>>(P);
   KCK(cudaGetLastError());
   if (rg)  // tier B (and M): the scan kind of tier S
-    k_sample<2, SL_FAST, true><<<w->grid_big, NT, w->smem_big, st>>>(P);
+    k_sample<2, SL_FAST, true><<<w->grid_big, 32 * NW_BIG, w->smem_big, st>>>(P);
   else
-    k_sample<2><<<w->grid_big, NT, w->smem_big, st>>>(P);
+    k_sample<2><<<w->grid_big, 32 * NW_BIG, w->smem_big, st>>>(P);
   KCK(cudaGetLastError());
   P.pi_base = w->pi_gm;
   P.pcap = w->pcap_gm;
   if (rg)
-    k_sample<1, SL_FAST, true><<<w->grid_gm, NT, CTL_BYTES + sizeof(LongRows), st>>>(P);
+    k_sample<1, SL_FAST, true><<<w->grid_gm, 32 * NW_S, CTL_BYTES<NW_S> + sizeof(LongRows), st>>>(P);
   else
-    k_sample<1><<<w->grid_gm, NT, CTL_BYTES + sizeof(LongRows), st>>>(P);
+    k_sample<1><<<w->grid_gm, 32 * NW_S, CTL_BYTES<NW_S> + sizeof(LongRows), st>>>(P);
   KCK(cudaGetLastError());
   return KADABRA_OK;
 }
@@ -6425,7 +6463,7 @@ void reset_result(kadabra_result* r) {
 #define KD_NA_PCAP 512
 #endif
 constexpr int NA_MAX_CTAS = KD_NA_MAX_CTAS;   // CTAs per launch at most (2 per SM on 152 SMs)
-constexpr int NA_PCAP = KD_NA_PCAP;           // candidate edges per warp
+constexpr int NA_PCAP = KD_NA_PCAP;           // a sample has at most PI_SEGS * NA_PCAP candidate edges
 constexpr int NA_MED_CTAS = 32;               // CTAs of the large-table launch (each with one tier-M table)
 constexpr uint64_t NA_MAX_BATCH = 65536;      // samples per call
 constexpr size_t NA_OFF_CTR = 0;              // Q_COUNT counters, then the status word
@@ -6434,7 +6472,7 @@ constexpr size_t NA_HEADER = 256;             // cleared on every call
 constexpr size_t NA_OFF_QB = NA_HEADER;
 constexpr size_t NA_OFF_QL = NA_OFF_QB + sizeof(unsigned long long) * NA_MAX_BATCH;
 constexpr size_t NA_OFF_PI = NA_OFF_QL + sizeof(unsigned long long) * NA_MAX_BATCH;
-constexpr size_t NA_OFF_MED = NA_OFF_PI + sizeof(PiEntry) * (size_t)NA_MAX_CTAS * 2 * NW * NA_PCAP;
+constexpr size_t NA_OFF_MED = NA_OFF_PI + sizeof(PiEntry) * (size_t)NA_MAX_CTAS * PI_SEGS * NA_PCAP;
 constexpr int NA_MED_HLOG = 15;               // its tier-M tables: 32768 hash slots,
 constexpr int NA_MED_LCAP = 16384;            //   lists of 16384 nodes
 // one tier-M table (gm_layout of NA_MED_HLOG, NA_MED_LCAP, MED_MAXD), 256-byte aligned
@@ -6473,10 +6511,10 @@ kadabra_status noalloc_setup(int dev, NoAllocDevice** out) {
     d.smem_b = big_smem_bytes();
     KCK(cudaFuncSetAttribute(k_sample<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.smem_s));
     KCK(cudaFuncSetAttribute(k_sample<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.smem_b));
-    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0>, NT, d.smem_s));
+    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0>, 32 * NW_S, d.smem_s));
     if (per_sm < 1) return fail(KADABRA_ERR_CAPACITY, "sampler does not fit on an SM");
     d.grid_s = std::min(sms * per_sm, NA_MAX_CTAS);
-    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<2>, NT, d.smem_b));
+    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<2>, 32 * NW_BIG, d.smem_b));
     if (per_sm < 1) return fail(KADABRA_ERR_CAPACITY, "large-table sampler does not fit on an SM");
     d.grid_b = std::min(sms * per_sm, NA_MED_CTAS);
     void* ptr = nullptr;
@@ -6889,9 +6927,9 @@ kadabra_status kadabra_sample_batch_noalloc(int32_t n, int64_t m, const int32_t*
   P.med_lcap = NA_MED_LCAP;
   P.tier_flags = 0;  // tiers S, B and M; samples beyond tier M end the call with KADABRA_ERR_CAPACITY
   KCK(cudaMemsetAsync(d->scratch, 0, NA_HEADER, st));
-  k_sample<0><<<d->grid_s, NT, d->smem_s, st>>>(P);
+  k_sample<0><<<d->grid_s, 32 * NW_S, d->smem_s, st>>>(P);
   KCK(cudaGetLastError());
-  k_sample<2><<<d->grid_b, NT, d->smem_b, st>>>(P);
+  k_sample<2><<<d->grid_b, 32 * NW_BIG, d->smem_b, st>>>(P);
   KCK(cudaGetLastError());
   unsigned long long left = 0;
   int32_t status = 0;
