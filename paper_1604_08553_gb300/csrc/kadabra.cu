@@ -3316,12 +3316,15 @@ __device__ __forceinline__ int32_t warp_row_of_arc(const int32_t* rp, int32_t n,
 template <int D, class F>
 __device__ __forceinline__ void for_each_arc(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m, F f) {
   const int lane = lane_id();
-  const int64_t chunks = (m + ARC_CHUNK - 1) / ARC_CHUNK;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  // a graph with less than ARC_CHUNK arcs per warp is spread over all of them
+  const int64_t per = (m + nwarps - 1) / nwarps;
+  const int64_t chunk = per < ARC_CHUNK ? (per + 31) / 32 * 32 : ARC_CHUNK;
+  const int64_t chunks = (m + chunk - 1) / chunk;
   for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < chunks; c += nwarps) {
-    const int64_t e1 = min(m, (c + 1) * ARC_CHUNK);
-    int32_t row = warp_row_of_arc(rp, n, c * ARC_CHUNK);
-    for (int64_t base = c * ARC_CHUNK; base < e1; base += 32 * D) {
+    const int64_t e1 = min(m, (c + 1) * chunk);
+    int32_t row = warp_row_of_arc(rp, n, c * chunk);
+    for (int64_t base = c * chunk; base < e1; base += 32 * D) {
       bool ok[D];
       int32_t u[D], v[D];
       int64_t e[D];
@@ -3542,10 +3545,11 @@ __device__ __forceinline__ void bfs_scan(const int32_t* tr, const int32_t* c, in
 // first, after m / (frontier arcs) looks or so.  Either direction yields the
 // same next level.  The arcs count for themselves: the neighbours of a
 // power-law graph's largest hub are few, but hold most arcs (both BFS of
-// R-MAT scale 24: 6.7 -> 4.0 ms; m/2 to m/16 measure the same there, and the
-// Chung-Lu graph of 10^6 nodes takes 0.42 ms with m/8 and 0.33 with m/16).
+// R-MAT scale 24: 6.7 -> 4.0 ms).  Whole loads with m, m/16, m/32 and m/64:
+// R-MAT scale 20 3.03, 2.17, 2.17, 2.17 ms, Chung-Lu of 10^6 nodes 0.82, 0.73,
+// 0.74, 0.74 ms, BA of 300,000 nodes 0.58, 0.59, 0.51, 0.51 ms.
 constexpr int BFS_BOTTOM_UP = 16;
-constexpr int BFS_BOTTOM_UP_ARCS = 16;
+constexpr int BFS_BOTTOM_UP_ARCS = 32;
 
 __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t* br, const int32_t* bc,
                             const int32_t* front, const int32_t* nfront_dev, int32_t* next, int32_t* nnext,
@@ -4636,7 +4640,7 @@ kadabra_status vd_condensation(kadabra_graph* g, LoadTrace& tr, const LoadScratc
   const int32_t* rrp = g->directed ? g->rrp : g->rp;
   const int32_t* rci = g->directed ? g->rci : g->ci;
   const int bn = std::max(1, std::min(16 * g->num_sms, (n + 255) / 256));
-  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, (m + 8 * ARC_CHUNK - 1) / (8 * ARC_CHUNK)));
+  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, (m + 255) / 256));
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t N4 = up(4 * (size_t)n), N8 = up(8 * (size_t)n);
   void* base = nullptr;
@@ -4774,7 +4778,7 @@ kadabra_status finish_load(kadabra_graph* g) {
   const int32_t n = g->n;
   const int64_t m = g->m;
   const int bn = std::max(1, std::min(16 * g->num_sms, (n + 255) / 256));
-  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, (m + 8 * ARC_CHUNK - 1) / (8 * ARC_CHUNK)));
+  const int ba = (int)std::max<int64_t>(1, std::min<int64_t>(16 * g->num_sms, (m + 255) / 256));
   const int32_t* rrp = g->directed ? g->rrp : g->rp;
   const int32_t* rci = g->directed ? g->rci : g->ci;
   unsigned h = 0;
