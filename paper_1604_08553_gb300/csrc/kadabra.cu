@@ -174,6 +174,15 @@ __device__ __noinline__ uint4 draw_late(uint64_t seed, uint32_t domain, uint64_t
   return draw(seed, domain, idx, j);
 }
 
+// the ordered pair s != t of a sample's block 0
+__device__ __forceinline__ void draw_pair(uint4 b, int32_t n, int* s, int* t) {
+  const uint64_t u = (uint64_t)b.x | ((uint64_t)b.y << 32);
+  const uint64_t u2 = (uint64_t)b.z | ((uint64_t)b.w << 32);
+  *s = (int)__umul64hi(u, (uint64_t)n);
+  const int tp = (int)__umul64hi(u2, (uint64_t)(n - 1));
+  *t = tp + (tp >= *s ? 1 : 0);
+}
+
 // floor(U * S / 2^128) for the 128-bit block U (x least significant)
 __device__ __forceinline__ uint64_t below128(uint4 b, uint64_t S) {
   const uint64_t lo = (uint64_t)b.x | ((uint64_t)b.y << 32);
@@ -405,7 +414,7 @@ struct SampleParams {
   Job job0;                         // the job, when the launch has only one
   const Job* jobs;                  // device array of njobs jobs, or null (then job0)
   int njobs;
-  uint64_t total_work;              // sum of the jobs' counts
+  uint64_t total_work;              // sum of the jobs' counts (with total_dev, about)
   const unsigned long long* total_dev;  // if set: the sum, read from device memory at launch
   unsigned long long* ctr;          // queue counters, Q_*
   unsigned long long* qb;           // sample indices queued for tier B
@@ -1859,11 +1868,10 @@ __device__ __forceinline__ void begin_sample(const SampleParams& P, const Tables
   const GraphDev& G = c.job.g;
   const uint4 b = draw(c.job.seed, c.job.domain, idx, (uint32_t)lane);
   c.draws[lane] = b;
-  const uint64_t u = (uint64_t)__shfl_sync(FULL, b.x, 0) | ((uint64_t)__shfl_sync(FULL, b.y, 0) << 32);
-  const uint64_t u2 = (uint64_t)__shfl_sync(FULL, b.z, 0) | ((uint64_t)__shfl_sync(FULL, b.w, 0) << 32);
-  const int s = (int)__umul64hi(u, (uint64_t)G.n);
-  const int tp = (int)__umul64hi(u2, (uint64_t)(G.n - 1));
-  const int t = tp + (tp >= s ? 1 : 0);
+  int s, t;
+  draw_pair(make_uint4(__shfl_sync(FULL, b.x, 0), __shfl_sync(FULL, b.y, 0), __shfl_sync(FULL, b.z, 0),
+                       __shfl_sync(FULL, b.w, 0)),
+            G.n, &s, &t);
   int bound = 0;  // lanes 0..3: the two roots' row bounds
   if (lane < 4) bound = __ldg((lane < 2 ? G.rp + s : G.rrp + t) + (lane & 1));
   if (lane < KADABRA_NSTAT) c.stat[lane] = lane == KADABRA_STAT_DIST ? -1 : 0;
@@ -2056,6 +2064,7 @@ constexpr int TF_WARP = 8;  // tier W first, whatever the launch's variant
 constexpr int TF_VEC = 16;  // pass 1 searches long rows (graphs beyond the L2)
 constexpr int TF_SEG64 = 32;  // shared-memory tiers scan frontiers in 64-node segments (tests)
 constexpr int TF_COMPACT = 64;  // tier S in the compact layout, whatever the launch's variant
+constexpr int TF_SCREEN = 128;  // k_screen first: tier S takes only the samples whose roots have arcs
 
 // queue counters in SampleParams::ctr
 constexpr int Q_NEXT_A = 0;   // next sample index of the batch
@@ -2252,6 +2261,73 @@ __global__ void __launch_bounds__(32 * MODE_NW<MODE>, MODE == 2 ? 1 : MODE == 1 
     }
   }
   if (tid < 32) flush_totals(P, c);
+}
+
+// ============================================================== screening
+// The samples whose s has no out-arc or whose t has no in-arc end at their
+// first level: one level, one expanded node, no arc.  One thread draws and
+// records such a sample; the others' work indices go to tier S's queue.  On
+// directed graphs with many such nodes most samples end here (R-MAT scale 22:
+// 65,536 samples 1.81 -> 1.65 ms).
+__global__ void __launch_bounds__(256) k_screen(const __grid_constant__ SampleParams P) {
+  const int lane = lane_id();
+  const unsigned long long ntotal = P.total_dev ? *P.total_dev : P.total_work;
+  for (unsigned long long base = blockIdx.x * 256ull; base < ntotal; base += gridDim.x * 256ull) {
+    const unsigned long long k = base + threadIdx.x;
+    bool idle = false, push = false;
+    int j = 0;
+    if (k < ntotal) {
+      if (P.jobs) {
+        int lo = 0, hi = P.njobs;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (P.jobs[mid].work_begin <= k)
+            lo = mid;
+          else
+            hi = mid;
+        }
+        j = lo;
+      }
+      const Job& J = P.jobs ? P.jobs[j] : P.job0;
+      int s, t;
+      draw_pair(draw(J.seed, J.domain, J.first_idx + (k - J.work_begin), 0), J.g.n, &s, &t);
+      idle = __ldg(&J.g.rp[s]) == __ldg(&J.g.rp[s + 1]) || __ldg(&J.g.rrp[t]) == __ldg(&J.g.rrp[t + 1]);
+      push = !idle;
+      if (idle && P.st_out) {
+        P.st_out[2 * k] = s;
+        P.st_out[2 * k + 1] = t;
+        if (P.path_len) P.path_len[k] = 0;
+        if (P.paths)
+          for (int q = 0; q < P.max_len; ++q) P.paths[(int64_t)k * P.max_len + q] = -1;
+        if (P.stats)
+          for (int q = 0; q < KADABRA_NSTAT; ++q)
+            P.stats[(int64_t)k * KADABRA_NSTAT + q] =
+                q == KADABRA_STAT_LEVELS || q == KADABRA_STAT_EXPANDED ? 1 : q == KADABRA_STAT_DIST ? -1 : 0;
+        if (P.sstatus) P.sstatus[k] = KADABRA_OK;
+      }
+    }
+    const unsigned go = __ballot_sync(FULL, push);
+    if (go) {
+      unsigned long long at = 0;
+      if (lane == 0) at = atomicAdd(&P.ctr[Q_SIZE_S], (unsigned long long)__popc(go));
+      at = __shfl_sync(FULL, at, 0) + __popc(go & ((1u << lane) - 1u));
+      if (push) {
+        if (at < P.deferred_cap)
+          P.q0[at] = k;
+        else
+          atomicCAS(P.status, 0, (int)KADABRA_ERR_CAPACITY);
+      }
+    }
+    // the idle samples' counters, once per warp and job
+    const unsigned same = __match_any_sync(FULL, idle ? j : -1);
+    if (idle && lane == __ffs(same) - 1) {
+      long long* tot = P.jobs ? P.jobs[j].totals : P.job0.totals;
+      if (tot) {
+        atomicAdd((unsigned long long*)&tot[KADABRA_STAT_LEVELS], (unsigned long long)__popc(same));
+        atomicAdd((unsigned long long*)&tot[KADABRA_STAT_EXPANDED], (unsigned long long)__popc(same));
+      }
+    }
+  }
 }
 
 // ============================================================== tier W: one warp per sample
@@ -3476,16 +3552,26 @@ __global__ void k_floor_degree(const int32_t* rp, const int32_t* rrp, int32_t n,
 // underlying undirected graph, |out(v) U in(v)| = out + in - reciprocal arcs
 // (directed; the nodes whose reciprocal arcs were not counted stay below the
 // others), as a key degree << 32 | ~id under atomicMax.
+// Also counts the nodes without out-arcs and those without in-arcs (idle).
 __global__ void k_und_degree_key(const int32_t* rp, const int32_t* rrp, const uint32_t* recip, int32_t n,
-                                 int directed, unsigned long long* best) {
+                                 int directed, unsigned long long* best, uint32_t* idle) {
   unsigned long long mine = 0;
+  uint32_t no_out = 0, no_in = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     int64_t d = rp[v + 1] - rp[v];
+    no_out += d == 0;
+    no_in += rrp[v + 1] == rrp[v];
     if (directed) d += (int64_t)(rrp[v + 1] - rrp[v]) - recip[v];
     const unsigned long long key = ((unsigned long long)d << 32) | (0xFFFFFFFFu - (uint32_t)v);
     mine = key > mine ? key : mine;
   }
   atomicMax(best, mine);
+  no_out = __reduce_add_sync(FULL, no_out);
+  no_in = __reduce_add_sync(FULL, no_in);
+  if (lane_id() == 0) {
+    if (no_out) atomicAdd(&idle[0], no_out);
+    if (no_in) atomicAdd(&idle[1], no_in);
+  }
 }
 
 __device__ __forceinline__ int32_t key_root(unsigned long long key) {
@@ -3632,6 +3718,7 @@ __global__ void k_bfs_items(const int32_t* tr, const int32_t* tc, const BfsItem*
 struct VdCore {
   unsigned long long size;  // |C_r|
   int32_t e_out, e_in;
+  uint32_t idle[2];         // nodes without out-arcs, without in-arcs
 };
 
 __global__ void k_vd_core(const int32_t* df, const int32_t* db, int32_t n, VdCore* out) {
@@ -4038,7 +4125,7 @@ struct Workspace {
   int32_t* status = nullptr;
   unsigned long long* qb = nullptr;  // queue for tier B
   unsigned long long* ql = nullptr;  // queue for tier L
-  unsigned long long* qs = nullptr;  // queue for tier S (fed by tier W)
+  unsigned long long* qs = nullptr;  // queue for tier S (fed by tier W or k_screen)
   uint64_t deferred_cap = 0;
   PiEntry* pi_fast = nullptr;
   PiEntry* pi_gm = nullptr;
@@ -4072,6 +4159,7 @@ struct kadabra_graph {
   int directed = 0;
   int32_t *rp = nullptr, *ci = nullptr, *rrp = nullptr, *rci = nullptr;
   int64_t vd = 0;
+  bool screened = false;       // enough samples end at a root without arcs: k_screen runs first
   bool csr_beyond_l2 = false;  // forward (+ reverse) CSR larger than the L2: long rows are searched
   int device = 0;
   int num_sms = 0;
@@ -4106,11 +4194,21 @@ namespace {
 // internal launch flag: the graph's CSR exceeds the L2, so pass 1 searches
 // its long rows (KADABRA_FLAG_ASYNC_SCAN asks for that explicitly)
 constexpr uint32_t FLAG_VEC_AUTO = 1u << 31;
+// internal launch flag: k_screen before tier S, for graphs on which at least
+// SCREEN_MIN of the samples end at a root without arcs, in launches of at
+// least SCREEN_SAMPLES samples.  It costs a launch (3 to 5 us); 1,000, 8,192,
+// 16,384 and 65,536 samples, without and with it: 109 and 114 us (R-MAT scale
+// 17), 445 and 436 (scale 20), 249 and 238 (scale 17), 1,092 and 996 (scale 20).
+constexpr uint32_t FLAG_SCREEN_AUTO = 1u << 30;
+constexpr double SCREEN_MIN = 0.25;
+constexpr uint64_t SCREEN_SAMPLES = 8192;
 // the flags a launch shared by several graphs takes from any of them (they
 // change no result; the tier-skipping flags stay per graph)
-constexpr uint32_t SHARED_LAUNCH_FLAGS = KADABRA_FLAG_WARP_TIER | KADABRA_FLAG_ASYNC_SCAN | FLAG_VEC_AUTO;
+constexpr uint32_t SHARED_LAUNCH_FLAGS = KADABRA_FLAG_WARP_TIER | KADABRA_FLAG_ASYNC_SCAN | FLAG_VEC_AUTO | FLAG_SCREEN_AUTO;
 
-uint32_t launch_flags(const kadabra_graph* g) { return g->flags | (g->csr_beyond_l2 ? FLAG_VEC_AUTO : 0u); }
+uint32_t launch_flags(const kadabra_graph* g) {
+  return g->flags | (g->csr_beyond_l2 ? FLAG_VEC_AUTO : 0u) | (g->screened ? FLAG_SCREEN_AUTO : 0u);
+}
 }  // namespace
 
 // G graphs whose CSRs share one device arena
@@ -4339,6 +4437,7 @@ SampleParams ws_params(const Workspace* w, uint32_t flags) {
   if (flags & (KADABRA_FLAG_ASYNC_SCAN | FLAG_VEC_AUTO)) P.tier_flags |= TF_VEC;
   if (flags & KADABRA_FLAG_FRONTIER_SEGMENTS) P.tier_flags |= TF_SEG64;
   if (flags & KADABRA_FLAG_COMPACT_TABLES) P.tier_flags |= TF_COMPACT;
+  if (flags & FLAG_SCREEN_AUTO) P.tier_flags |= TF_SCREEN;
   return P;
 }
 
@@ -4360,6 +4459,10 @@ kadabra_status launch_sampler_kernels(Workspace* w, SampleParams P, cudaStream_t
   if (((variant & 2) || (P.tier_flags & TF_WARP)) && !(P.tier_flags & TF_SKIP_S)) {
     P.q0 = w->qs;  // tier W's overflow queue, tier S's input
     k_sample_warp<<<w->grid_warp, 32 * WT_WARPS, w->smem_warp, st>>>(P);
+    KCK(cudaGetLastError());
+  } else if ((P.tier_flags & TF_SCREEN) && !(P.tier_flags & TF_SKIP_S) && P.total_work >= SCREEN_SAMPLES) {
+    P.q0 = w->qs;
+    k_screen<<<2 * w->num_sms, 256, 0, st>>>(P);
     KCK(cudaGetLastError());
   }
   const bool rg = (P.tier_flags & TF_VEC) != 0;
@@ -4743,7 +4846,7 @@ kadabra_status compute_vd(kadabra_graph* g, LoadTrace& tr, const LoadScratch& S)
   KCK(cudaMemsetAsync(S.dist, 0xFF, sizeof(int32_t) * (size_t)n));
   if (g->directed) KCK(cudaMemsetAsync(S.dist_b, 0xFF, sizeof(int32_t) * (size_t)n));
   KCK(cudaMemsetAsync(S.core, 0, sizeof(VdCore)));
-  k_und_degree_key<<<blocks, 256>>>(g->rp, rrp, S.recip, n, g->directed, S.best);
+  k_und_degree_key<<<blocks, 256>>>(g->rp, rrp, S.recip, n, g->directed, S.best, S.core->idle);
   KCK(cudaGetLastError());
   tr.mark("vd root");
   KTRY(vd_bfs(g, S, g->rp, g->ci, rrp, rci, S.dist));
@@ -4757,6 +4860,8 @@ kadabra_status compute_vd(kadabra_graph* g, LoadTrace& tr, const LoadScratch& S)
   if (cudaMemcpy(&core, S.core, sizeof(core), cudaMemcpyDeviceToHost) != cudaSuccess)
     return fail(KADABRA_ERR_CUDA, std::string("vd: ") + cudaGetErrorString(cudaGetLastError()));
   tr.mark("vd bfs");
+  const double idle = 1.0 - (1.0 - (double)core.idle[0] / n) * (1.0 - (double)core.idle[1] / n);
+  g->screened = idle >= SCREEN_MIN;
   const long long root_w = (long long)core.e_out + core.e_in + 1;
   if (core.size == (unsigned long long)n) {
     g->vd = root_w;
@@ -5143,6 +5248,7 @@ kadabra_status run_loop_graph(LoopCache& L, Workspace* w, cudaStream_t st, std::
   P.jobs = d_job;
   P.njobs = G;
   P.total_dev = &d_state->total_work;
+  for (const LoopRun& r : R) P.total_work += r.K;  // about; the launch reads total_dev
   int64_t max_n = 1;
   for (const LoopRun& r : R) max_n = std::max<int64_t>(max_n, r.g->n);
   const int64_t want = (4 * (int64_t)w->num_sms + G - 1) / G;

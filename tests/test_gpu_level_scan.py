@@ -73,3 +73,37 @@ def test_candidate_counts(kd, orc, gg, p, q):
     e += [(p + q, p + q + 2), (p + q + 1, p + q + 3)]
     g = gg.from_edges(p + q + 4, e, name=f"K{p},{q}+")
     _equal(kd, orc, g, (0, kd.FLAG_COMPACT_TABLES, kd.FLAG_MEDIUM_TABLES, kd.FLAG_FRONTIER_SEGMENTS), count=1500)
+
+
+@pytest.mark.parametrize("count", [8191, 8192, 20000])
+def test_screened_batches(kd, orc, gg, count):
+    """Directed graphs most of whose samples end at a root without arcs: the
+    launches large enough for the screening kernel, and those just below,
+    give the oracle's hits and work counters; several graphs in one launch
+    give each graph's own run."""
+    import torch
+    g = gg.rmat(12, 8, 0.57, 0.19, 0.19, 10)
+    _, c_ref, t_ref = orc.accumulate(g, 5, 0, 100, count)
+    G = kd.kadabra_load_csr(g)
+    try:
+        c = torch.zeros(g.n, dtype=torch.int32, device="cuda")
+        t = torch.zeros(kd.NSTAT, dtype=torch.int64, device="cuda")
+        kd.kadabra_sample_batch(G, 5, 0, 100, count, c, t)
+        kd.kadabra_sync_status(G)
+    finally:
+        G.free()
+    assert np.array_equal(c.cpu().numpy(), c_ref)
+    assert np.array_equal(t.cpu().numpy()[:8], np.asarray(t_ref)[:8])
+
+
+def test_screened_batch_run(kd, gg):
+    graphs = [gg.rmat(11, 8, 0.57, 0.19, 0.19, 3), gg.erdos_renyi(2000, 8.0, 1), gg.rmat(12, 6, 0.57, 0.19, 0.19, 4)]
+    B = kd.Batch(graphs)
+    try:
+        rs = B.run([0.02] * 3, [0.1] * 3, [7, 8, 9], check_interval=4096)
+        for i, r in enumerate(rs):
+            one = kd.kadabra_run(B.views[i], 0.02, 0.1, 0, 7 + i, check_interval=4096)
+            assert r.tau == one.tau and np.array_equal(r.counts, one.counts)
+            assert np.array_equal(r.totals, one.totals) and (r.max_f, r.max_g) == (one.max_f, one.max_g)
+    finally:
+        B.free()
