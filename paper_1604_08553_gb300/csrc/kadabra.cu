@@ -873,7 +873,10 @@ __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount
           if (k == j) yy = y[j];
         pos = tab_probe(T, yy, &hy);
         touch = pos >= 0 && val_side(ent_val<PK>(hy)) != side;
-        if (touch) p = frontier_pos(T.pr, fcount, wb + 32 * k + lane);
+        if (touch) {
+          const int e = wb + 32 * k + lane;
+          p = e < nxt ? pcur : frontier_next(T.pr, pcur + 1, fcount, e);
+        }
       }
       emit(touch, p, yy, pos, hy);
     }
@@ -1101,14 +1104,43 @@ __device__ void bt_warp_steps(const SampleParams& P, const Job& J, const Tables&
     const int plo = lvl_lo(T, half, dx - 1), phi = lvl_hi(T, half, dx - 1);
     const int r0 = __ldg(&brow[x]), deg = __ldg(&brow[x + 1]) - r0;
     const bool single = phi - plo == 1;
-    if (!single && deg > WARP_BT_ROW) break;  // the block takes this step
+    const bool by_level = phi - plo <= 32 && (phi - plo) * 16 < deg;
+    if (!single && !by_level && deg > WARP_BT_ROW) break;  // the block takes this step
     int y = -1, pos = -1;
     if (single) {
       // a single node one level closer: it is x's only predecessor
       y = list_node<PK>(T, plo);
       const uint32_t q = lpos_get<PK>(T, plo);
       sx = ent_sig<PK>(T, T.hkv[q], q);
-      pos = warp_lower_bound(bcol, r0, r0 + deg, y) - r0;
+    } else if (by_level) {
+      // the previous level's nodes, one per lane: those adjacent to x are the
+      // candidates, in id order (a long row of x takes more steps to scan)
+      const unsigned long long r = below128(j < 32 ? c.draws[j] : draw_late(J.seed, J.domain, idx, j), sx);
+      const int32_t* frow = half == 0 ? G.rp : G.rrp;
+      const int32_t* fcol = half == 0 ? G.ci : G.rci;
+      int yy = 0x7FFFFFFF;
+      unsigned long long w = 0;
+      if (plo + lane < phi) {
+        yy = list_node<PK>(T, plo + lane);
+        const int b = __ldg(&frow[yy + 1]);
+        const int at = lower_bound_row(fcol, __ldg(&frow[yy]), b, x);
+        if (at < b && __ldg(&fcol[KIDX((int64_t)at, G.m, 12)]) == x) {
+          const uint32_t q = lpos_get<PK>(T, plo + lane);
+          w = ent_sig<PK>(T, T.hkv[q], q);
+        }
+      }
+      unsigned long long below = 0;
+      for (unsigned m = __ballot_sync(FULL, w != 0); m; m &= m - 1) {
+        const int k = __ffs(m) - 1;
+        const int yk = __shfl_sync(FULL, yy, k);
+        const unsigned long long wk = __shfl_sync(FULL, w, k);
+        if (yk < yy) below += wk;
+      }
+      const unsigned hit = __ballot_sync(FULL, w != 0 && below <= r && r - below < w);
+      if (hit) {
+        y = __shfl_sync(FULL, yy, __ffs(hit) - 1);
+        sx = __shfl_sync(FULL, w, __ffs(hit) - 1);
+      }
     } else {
       const unsigned long long r = below128(j < 32 ? c.draws[j] : draw_late(J.seed, J.domain, idx, j), sx);
       const uint32_t want = pack_val(half, dx - 1);
@@ -1155,6 +1187,7 @@ __device__ void bt_warp_steps(const SampleParams& P, const Job& J, const Tables&
       if (lane == 0) c.bt_flag = 1;
       return;
     }
+    if (pos < 0) pos = warp_lower_bound(bcol, r0, r0 + deg, y) - r0;
     if (lane == 0) bt_record<PK>(P, J, c, half, dx - 1, y, pos, out_i, dv, dw, want_path);
     x = y;
     dx -= 1;
