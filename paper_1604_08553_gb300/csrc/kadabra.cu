@@ -105,7 +105,13 @@ namespace {
 // samples) 0.83, 0.57, 0.26 -> 0.25 ms, Chung-Lu 10^6 nodes (65,536) 0.47,
 // 0.35, 0.19 -> 0.19 ms, R-MAT scale 24 (65,536) 2.28, 1.62, 1.30 -> 1.22 ms:
 // fewer samples go on to tier M, and a level's arcs take fewer steps.
+// The compact tier-S layout: 6 warps, which leaves five CTAs per SM 64 registers
+// a thread and so the fused pass; with 8 warps (48 registers) it spilled.
+// 65,536 samples with 8 warps, with 6, and in the default layout: Chung-Lu of
+// 10^5 nodes 2.07, 1.57, 1.73 ms, of 10^6 nodes 3.45, 2.97, 2.95 ms; 8,192 of
+// ER 2,000 nodes 266, 188, 214 us; 16,384 of BA 300,000 nodes 800, 656, 713 us.
 constexpr int NW_S = KD_NT / 32;
+constexpr int NW_CMP = 6;
 constexpr int NW_BIG = KD_NT_BIG / 32;
 constexpr int U = KD_U;            // independent items per thread per step (memory-level parallelism)
 // Tiers of per-sample tables.  A sample starts in a small shared-memory
@@ -467,9 +473,6 @@ struct SampleParams {
 constexpr int LONG_CAP = KD_LONG_CAP;
 #ifndef KD_FUSE_MAX
 #define KD_FUSE_MAX 256
-#endif
-#ifndef KD_FU_CMP
-#define KD_FU_CMP 0  // the fused pass in the compact layout
 #endif
 #ifndef KD_TD
 #define KD_TD 4
@@ -1251,7 +1254,7 @@ KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl<NW>& c, const int3
 // One sample, from the state begin_sample and insert_roots left (warp 0's
 // insertions need no barrier: the first level's frontier is read by warp 0,
 // and the other warps read the table only after that level's first barrier).
-// FU: small levels take the fused pass.  The caller puts a barrier after it.
+// The caller puts a barrier after it.
 //
 // What a level costs beside its arcs is barriers and the latency of the steps
 // one thread or warp takes while the others wait, so a level has as few of
@@ -1264,7 +1267,7 @@ KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl<NW>& c, const int3
 // 4.41 -> 3.37 ms on the Chung-Lu graph of 10^6 nodes (2.49 -> 1.85 G warp
 // instructions) and 2.70 -> 2.21 ms on R-MAT scale 22; a 3.4 M-node ER graph's
 // run 18.3 -> 15.4 ms.
-template <bool PK, bool RG, bool FU, int NW>
+template <bool PK, bool RG, int NW>
 __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, const Tables& T, Ctl<NW>& c, uint64_t idx,
                                            int64_t out_i) {
   constexpr int NT = 32 * NW;
@@ -1304,7 +1307,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
     // A level of at most FUSE_MAX arcs that cannot fill the lists skips pass
     // 1: pass 2 then tests for touches while it inserts, and undoes its
     // insertions if it finds one.
-    const bool fused = FU && E <= FUSE_MAX && nseg == 1 && list_before + E <= T.lcap;
+    const bool fused = E <= FUSE_MAX && nseg == 1 && list_before + E <= T.lcap;
     // pass 1 uses a filter of the other side's frontier, kept while that
     // frontier stays the same
     const bool new_filter = PK && !fused && (c.fside != 1 - side || c.fdepth != od);
@@ -1504,7 +1507,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
                       else
                         of = true;
                     }
-                  } else if (FU && fused && val_side(v) != side) {
+                  } else if (fused && val_side(v) != side) {
                     res = 2;
                   }
                   break;
@@ -1530,7 +1533,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
                 }
               }
             }
-            if (FU && fused) emit(fb, res == 2, p, y, (int)pos, w);
+            if (fused) emit(fb, res == 2, p, y, (int)pos, w);
           });
         }
         if (sg + 1 < nseg) {
@@ -1565,7 +1568,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
       const int lf = (of ? LF_SIGMA : 0) | (cap ? LF_CAP : 0) | (sigma_of ? LF_TOUCH_SIGMA : 0);
       if (lf) atomicOr(&c.lvl_flags, lf);
       __syncthreads();
-      if (FU && fused && c.npi > 0) {
+      if (fused && c.npi > 0) {
         // the level touches: undo its insertions (slots that were empty
         // before it) and choose among its touch arcs, as after pass 1
 #pragma unroll 1
@@ -1963,7 +1966,7 @@ __device__ __noinline__ void run_sample_global(const SampleParams& P, const Job&
     insert_roots<false>(T, c);
   }
   __syncthreads();
-  run_sample<false, RG, true>(P, J, T, c, idx, out_i);
+  run_sample<false, RG>(P, J, T, c, idx, out_i);
   __syncthreads();
 }
 
@@ -2061,7 +2064,7 @@ struct SLayout {
 #define KD_CMP_MAXD 38
 #endif
 using FastLayout = SLayout<NW_S, FAST_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
-using CompactLayout = SLayout<NW_S, FAST_HLOG, KD_CMP_L8, 512, KD_CMP_FLOG, KD_CMP_MAXD, false>;
+using CompactLayout = SLayout<NW_CMP, FAST_HLOG, KD_CMP_L8, 512, KD_CMP_FLOG, KD_CMP_MAXD, false>;
 using BigLayout = SLayout<NW_BIG, BIG_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
 // the tier-S layout a k_sample instance uses (SL)
 constexpr int SL_FAST = 0;
@@ -2194,14 +2197,14 @@ __device__ void finish_sample(const SampleParams& P, Ctl<NW>& c, int64_t out_i) 
 // and gives the same results (samples that outgrow it go on to tier B as
 // usual).  RG (the default layout only): pass 1 searches long rows (for
 // graphs whose CSR exceeds L2); same results.
-template <int MODE>
-constexpr int MODE_NW = MODE == 2 ? NW_BIG : NW_S;
+template <int MODE, int SL = SL_FAST>
+constexpr int MODE_NW = MODE == 2 ? NW_BIG : SL == SL_COMPACT ? NW_CMP : NW_S;
 template <int MODE, int SL = SL_FAST, bool RG = false>
-__global__ void __launch_bounds__(32 * MODE_NW<MODE>, MODE == 2 ? 1 : MODE == 1 ? 2 : SL == SL_FAST ? KD_MIN_BLOCKS : KD_MIN_BLOCKS + 1)
+__global__ void __launch_bounds__(32 * MODE_NW<MODE, SL>, MODE == 2 ? 1 : MODE == 1 ? 2 : SL == SL_FAST ? KD_MIN_BLOCKS : KD_MIN_BLOCKS + 1)
     k_sample(SampleParams P) {
   static_assert(!RG || SL == SL_FAST, "the beyond-L2 scan has no compact-layout instance");
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int NW = MODE_NW<MODE>;
+  constexpr int NW = MODE_NW<MODE, SL>;
   Ctl<NW>& c = *reinterpret_cast<Ctl<NW>*>(smem);
   Tables TS, TM;
   PiEntry* pi = P.pi_base + (size_t)blockIdx.x * PI_SEGS * P.pcap;
@@ -2267,7 +2270,7 @@ __global__ void __launch_bounds__(32 * MODE_NW<MODE>, MODE == 2 ? 1 : MODE == 1 
     if (MODE == 0) {
       if (!(P.tier_flags & TF_SKIP_S)) {
         if (tid < 32) insert_roots<true>(TS, c);
-        run_sample<true, RG, SL == SL_FAST || KD_FU_CMP>(P, c.job, TS, c, idx, out_i);
+        run_sample<true, RG>(P, c.job, TS, c, idx, out_i);
       } else if (tid == 0) {
         c.flags = F_CAP;
       }
@@ -2276,7 +2279,7 @@ __global__ void __launch_bounds__(32 * MODE_NW<MODE>, MODE == 2 ? 1 : MODE == 1 
       bool done = false;
       if (!(P.tier_flags & TF_SKIP_B)) {
         if (tid < 32) insert_roots<true>(TS, c);
-        run_sample<true, RG, true>(P, c.job, TS, c, idx, out_i);
+        run_sample<true, RG>(P, c.job, TS, c, idx, out_i);
         __syncthreads();
         done = c.flags != F_CAP;
         __syncthreads();
@@ -4337,7 +4340,7 @@ kadabra_status ensure_ws(Workspace* w, uint64_t deferred_need, int njobs) {
     w->grid_fast = w->num_sms * per_sm;
     w->smem_compact = compact_smem_bytes();
     KCK(cudaFuncSetAttribute(k_sample<0, SL_COMPACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_compact));
-    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0, SL_COMPACT>, 32 * NW_S, w->smem_compact));
+    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0, SL_COMPACT>, 32 * NW_CMP, w->smem_compact));
     w->grid_compact = w->num_sms * std::max(per_sm, 1);
     w->smem_warp = warp_tier_smem_bytes();
     KCK(cudaFuncSetAttribute(k_sample_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_warp));
@@ -4500,7 +4503,7 @@ kadabra_status launch_sampler_kernels(Workspace* w, SampleParams P, cudaStream_t
   }
   const bool rg = (P.tier_flags & TF_VEC) != 0;
   if ((variant & 1) || ((P.tier_flags & TF_COMPACT) && !rg))  // the compact layout has no beyond-L2 variant
-    k_sample<0, SL_COMPACT><<<w->grid_compact, 32 * NW_S, w->smem_compact, st>>>(P);
+    k_sample<0, SL_COMPACT><<<w->grid_compact, 32 * NW_CMP, w->smem_compact, st>>>(P);
   else if (rg)
     k_sample<0, SL_FAST, true><<<w->grid_fast, 32 * NW_S, w->smem_fast, st>>>(P);
   else
