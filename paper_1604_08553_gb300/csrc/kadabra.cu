@@ -335,10 +335,6 @@ __device__ __forceinline__ uint32_t hash_pos(int32_t v, int hlog) {
 constexpr int FILTER_LOG = KD_FILTER_LOG;  // the default layout's filter: 2^FILTER_LOG bits
 // fshift = 32 - log2(the filter's bits)
 __device__ __forceinline__ uint32_t filter_slot(int32_t v, int fshift) { return ((uint32_t)v * 0x9E3779B1u) >> fshift; }
-__device__ __forceinline__ bool filter_has(const uint32_t* bits, int32_t v, int fshift) {
-  const uint32_t h = filter_slot(v, fshift);
-  return (bits[h >> 5] >> (h & 31)) & 1u;
-}
 
 // position of v's entry (its word in *wout), or -1
 __device__ __forceinline__ int tab_probe(const Tables& T, int32_t v, unsigned long long* wout) {
@@ -475,12 +471,11 @@ constexpr int LONG_CAP = KD_LONG_CAP;
 #define KD_FUSE_MAX 256
 #endif
 #ifndef KD_TD
-#define KD_TD 4
+#define KD_TD 6
 #endif
 // Pass 1: arcs per lane in flight.  Batches of 65,536 samples on the Chung-Lu
-// graph of 10^6 nodes and R-MAT scale 22 with 2, 3, 4, 6 (and 8): 4.16, 3.99,
-// 3.91, 3.88 ms and 2.45, 2.36, 2.32, 2.27 ms; the small ER graph's runs lose
-// 2 % from 4 to 6 to the longer code.
+// graph of 10^6 nodes and the run of 64 BA graphs with 4 and 6: 2.85 and 2.81,
+// 93.4 and 92.0 ms; the small ER graph's runs 1.07 ms with either.
 constexpr int TOUCH_DEPTH = KD_TD;
 constexpr int FUSE_MAX = KD_FUSE_MAX;  // levels of at most this many arcs insert and test for touches in one pass
 __device__ __forceinline__ bool row_is_long(int deg, int k) {
@@ -820,10 +815,13 @@ __device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcou
 // heads, so a step tests its heads against the filter only; the lanes that
 // pass then probe the table together.  Calls emit(touch, x's frontier
 // position, y, y's table position and word) with all lanes of the warp, in
-// no particular order.  Bound by instruction issue (about 130 per step) and
-// by the slowest warp at the barrier after it: windows of 32 arcs with a
-// probe each, and short rows one window at a time, took 23.2 k of 74 k cycles
-// per sample on the Chung-Lu graph of 10^6 nodes, this takes 16.6 k.
+// no particular order.  Bound by instruction issue and by the slowest warp at
+// the barrier after it: windows of 32 arcs with a probe each, and short rows
+// one window at a time, took 23.2 k of 74 k cycles per sample on the Chung-Lu
+// graph of 10^6 nodes; this takes 16 k of 57 k.  Run twice, it adds 36 % to a
+// batch's instructions and 35 % to its time; without the branches around each
+// filter test a batch of 65,536 went 2.97 -> 2.85 ms.  Queueing the heads that
+// pass the filter and probing them 32 at a time changed nothing (2.96 -> 3.01).
 template <bool PK, int D, int NW, class EM>
 __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount, int E, const int32_t* cols,
                                            int64_t ncols, EM emit) {
@@ -854,14 +852,22 @@ __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount
         a[k] = q.y + (wb + 32 * k + lane - q.x);
       }
     }
+    const int left = c1 - wb - lane;  // the lane's arc k exists if left > 32 k
     int y[D];
 #pragma unroll
     for (int k = 0; k < D; ++k)
-      y[k] = wb + 32 * k + lane < c1 ? __ldg(&cols[KIDX((int64_t)a[k], ncols, 8)]) : 0;
-    unsigned hit = 0;  // bit k: head y[k] may touch
+      y[k] = left > 32 * k ? __ldg(&cols[KIDX((int64_t)a[k], ncols, 8)]) : 0;
+    // bit k: head y[k] may touch (tested without branches; the heads of lanes
+    // beyond the slice are masked)
+    unsigned hit = PK ? 0u : (1u << D) - 1u;
+    if (PK) {
 #pragma unroll
-    for (int k = 0; k < D; ++k)
-      if (wb + 32 * k + lane < c1 && (!PK || filter_has(T.bits, y[k], T.fshift))) hit |= 1u << k;
+      for (int k = 0; k < D; ++k) {
+        const uint32_t h = filter_slot(y[k], T.fshift);
+        hit |= (__funnelshift_r(T.bits[h >> 5], 0u, h) & 1u) << k;
+      }
+    }
+    if (left <= 32 * (D - 1)) hit &= left > 0 ? (2u << ((left - 1) >> 5)) - 1u : 0u;
 #pragma unroll 1
     while (__any_sync(FULL, hit != 0)) {
       bool touch = false;
