@@ -57,7 +57,7 @@ METRIC = "paths/sec & time-to-(lambda,delta) per graph, batched vs plain on GPU;
 WORKLOADS = {
     "chung_lu_1m": dict(family="chung_lu", n=1_000_000, beta=2.5, mean_deg=16.0, max_deg=10_000.0, graph_seed=1,
                         lcc=True, lam=0.005, delta=0.1, check_interval=1 << 16,
-                        sampler_dram_bytes=99_782_571 + 23_815_338 + 64_768),
+                        sampler_dram_bytes=77_228_203 + 11_709_013 + 66_133),
     "erdos_renyi_2k": dict(family="erdos_renyi", n=2000, mean_deg=8.0, graph_seed=1, lcc=True, lam=0.01,
                            delta=0.1, check_interval=1000, sampler_dram_bytes=None),
     "rmat_24": dict(family="rmat", scale=24, edge_factor=16, a=0.57, b=0.19, c=0.19, graph_seed=1, lam=0.0025,
@@ -65,7 +65,7 @@ WORKLOADS = {
     # the scale-22 graph of the same recipe: the size the ncu counters are captured at
     "rmat_22": dict(family="rmat", scale=22, edge_factor=16, a=0.57, b=0.19, c=0.19, graph_seed=1, lam=0.0025,
                     delta=0.1, check_interval=1 << 16,
-                    sampler_dram_bytes=632_693_077 + 149_157_888 + 65_792),
+                    sampler_dram_bytes=10_442_667 + 578_775_296 + 69_229_056 + 65_792),
     "rmat_24_topk": dict(family="rmat", scale=24, edge_factor=16, a=0.57, b=0.19, c=0.19, graph_seed=1, lam=0.0025,
                          delta=0.1, check_interval=1 << 16, sampler_dram_bytes=None, k=10),
 }
@@ -281,8 +281,10 @@ def run_launches(r, w):
 def sampler_launches_per_batch(r=None):
     """Kernels of one sampler batch: the shared-memory tier and the two
     escalation tiers (which exit at once when nothing was queued to them),
-    plus the one-warp-per-sample tier in front when the run used it."""
-    return 3 + (1 if r is not None and getattr(r, "warp_tier", 0) else 0)
+    plus the kernel in front: the one-warp-per-sample tier when the run used
+    it, or the screening of the R-MAT workloads' idle samples."""
+    warp = r is not None and getattr(r, "warp_tier", 0)
+    return 3 + (1 if warp or WORKLOAD["family"] == "rmat" else 0)
 
 
 def cpu_baseline(g, seconds_cap=20.0):
