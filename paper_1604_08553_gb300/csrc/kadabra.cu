@@ -3553,37 +3553,91 @@ __global__ void __launch_bounds__(256) k_validate_arcs(const int32_t* rp, const 
   if (bits && lane_id() == 0) atomicOr(err, bits);
 }
 
-// Every PIVOT-th entry of the column array searched by the mirror test.
-// A binary search in a long row of a graph beyond the L2 reads HBM at most of
-// its steps, and that many scattered reads bound the test: one, two or four
-// searches per lane at once, and arcs taken in narrower windows, all took 32
-// to 33 ms on R-MAT scale 24 (263 M arcs).  Over the pivots (33 MB of its
-// 1.05 GB, which stay in the L2) a search leaves HBM its last PIVOT entries,
-// one 128-byte line: 15.6 ms; every 16th entry 15.6, every 64th 17.4 ms.
-// Graphs within the L2 have none.
-constexpr int PIVOT = 32;
-__global__ void k_pivots(const int32_t* ci, int64_t m, int32_t* piv) {
-  const int64_t k = (m + PIVOT - 1) / PIVOT;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < k; i += (int64_t)gridDim.x * blockDim.x)
-    piv[i] = ci[i * PIVOT];
+// An 8-ary tree over the column array that the mirror test searches, for
+// graphs beyond the L2: level k holds every (2^TREE_SHIFT * 8^k)-th entry, and
+// an aligned group of 8 of them, one 32-byte load, settles one octal digit of
+// a position.
+// What bounds the test is the number of scattered loads per arc: each lane's
+// goes to another line, and L1 takes one line per cycle.  A binary search
+// costs one per bit, the tree one per three bits, and the two levels that are
+// not L2-resident cost HBM one sector each.  The mirror test of R-MAT scale 24
+// (263 M arcs): binary search 32 to 33 ms (one, two or four searches per lane
+// at once), binary over every 32nd entry first 15.6, this tree 9.6 ms (L1 at
+// 72 %, L2 61 %, issue 59 % on scale 22); with a last block of 16 or 32
+// entries (TREE_SHIFT 4, 5) 11.6, 14.0 ms.  Graphs within the L2 have no
+// tree: building it costs more than it saves (Chung-Lu 10^6 nodes 0.18 -> 0.23 ms).
+#ifndef KD_TREE_SHIFT
+#define KD_TREE_SHIFT 3
+#endif
+constexpr int TREE_SHIFT = KD_TREE_SHIFT;  // at least 3
+constexpr int TREE_LEVELS = (31 - TREE_SHIFT + 2) / 3;
+struct RowTree {
+  int32_t* lv[TREE_LEVELS];  // 32-byte aligned, whole groups of 8
+  int32_t levels;            // 0: no tree
+  int32_t groups;            // whole groups of 8 of the column array itself, 0 if it is not 32-byte aligned
+};
+
+__global__ void k_row_tree(const int32_t* ci, int64_t m, const __grid_constant__ RowTree t) {
+  const int64_t c = (m + (1ll << TREE_SHIFT) - 1) >> TREE_SHIFT;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t x = ci[i << TREE_SHIFT];
+    t.lv[0][i] = x;
+    int64_t q = i;
+    for (int k = 1; k < t.levels && (q & 7) == 0; ++k) {
+      q >>= 3;
+      t.lv[k][q] = x;
+    }
+  }
 }
 
-// row v of a sorted CSR has y (piv: its pivots, or null)
-__device__ __forceinline__ bool row_has(const int32_t* rp, const int32_t* ci, const int32_t* piv, int32_t v, int32_t y) {
-  int32_t lo = __ldg(&rp[v]), hi = __ldg(&rp[v + 1]);
-  if (piv && hi - lo > PIVOT) {
-    int32_t a = lo / PIVOT, b = (hi - 1) / PIVOT;  // the last pivot in (a, b] not above y, or a if there is none
-    const int32_t b0 = b;
-    while (a < b) {
-      const int32_t mid = a + (b - a + 1) / 2;
-      if (__ldg(&piv[mid]) <= y)
-        a = mid;
-      else
-        b = mid - 1;
-    }
-    lo = max(lo, a * PIVOT);
-    if (a < b0) hi = (a + 1) * PIVOT;
+// p: 32-byte aligned
+__device__ __forceinline__ void ldg8(const int32_t* p, int32_t (&w)[8]) {
+  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+      : "l"(p));
+}
+
+// entries [a, b], not none, of a sorted row have y
+__device__ __forceinline__ bool tree_has(const int32_t* ci, const RowTree& t, int32_t a, int32_t b, int32_t y) {
+  int32_t w[8];
+  const uint32_t diff = (uint32_t)(a ^ b) >> TREE_SHIFT;
+  for (int k = diff ? (31 - __clz(diff)) / 3 : -1; k >= 0; --k) {
+    // a and b lie under one group of this level; y, if it is there, lies under
+    // the last entry of the group within (a, b] that is not above it, or under a's
+    const int sh = TREE_SHIFT + 3 * k;
+    const int32_t pa = a >> sh, pb = b >> sh;
+    if (pa == pb) continue;
+    ldg8(t.lv[k] + (pa & ~7), w);
+    uint32_t le = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) le |= (w[q] <= y ? 1u : 0u) << q;
+    const int32_t i = pa + __popc(le & ((2u << (pb & 7)) - (2u << (pa & 7))));
+    if (i > pa) a = i << sh;
+    if (i < pb) b = ((i + 1) << sh) - 1;
   }
+  while ((a >> 3) != (b >> 3)) {  // TREE_SHIFT > 3: groups of 8 of the last block
+    const int32_t mid = ((a >> 3) + (b >> 3) + 1) >> 1;
+    if (__ldg(&ci[8 * mid]) <= y)
+      a = 8 * mid;
+    else
+      b = 8 * mid - 1;
+  }
+  if ((a >> 3) < t.groups) {
+    ldg8(ci + (a & ~7), w);
+    uint32_t eq = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) eq |= (w[q] == y ? 1u : 0u) << q;
+    return (eq & ((2u << (b & 7)) - (1u << (a & 7)))) != 0;
+  }
+  bool found = false;
+  for (; a <= b; ++a) found |= __ldg(&ci[a]) == y;
+  return found;
+}
+
+// row v of a sorted CSR has y
+__device__ __forceinline__ bool row_has(const int32_t* rp, const int32_t* ci, const RowTree& t, int32_t v, int32_t y) {
+  int32_t lo = __ldg(&rp[v]), hi = __ldg(&rp[v + 1]);
+  if (t.levels) return lo < hi && tree_has(ci, t, lo, hi - 1, y);
   while (lo < hi) {
     const int32_t mid = lo + ((hi - lo) >> 1);
     const int32_t z = __ldg(&ci[mid]);
@@ -3611,7 +3665,7 @@ __device__ __forceinline__ bool row_has(const int32_t* rp, const int32_t* ci, co
 __global__ void __launch_bounds__(256) k_validate_mirror(const int32_t* rp, const int32_t* ci, const int32_t* rrp,
                                                          const int32_t* rci, int32_t n, int64_t m, int undirected,
                                                          unsigned* err, unsigned long long* lt_gt, uint32_t* recip,
-                                                         const int32_t* floor_deg, const int32_t* piv) {
+                                                         const int32_t* floor_deg, const __grid_constant__ RowTree tree) {
   if (*(volatile const unsigned*)err & 15u) return;  // needs valid offsets, ids in range and sorted rows
   unsigned long long lt = 0, gt = 0;
   bool bad = false;
@@ -3624,10 +3678,10 @@ __global__ void __launch_bounds__(256) k_validate_mirror(const int32_t* rp, cons
       return;
     }
     ++lt;
-    if (!row_has(rrp, rci, piv, v, u)) bad = true;
+    if (!row_has(rrp, rci, tree, v, u)) bad = true;
     if (!undirected) {
       const int64_t both = (int64_t)(__ldg(&rp[u + 1]) - __ldg(&rp[u])) + (__ldg(&rrp[u + 1]) - __ldg(&rrp[u]));
-      if (both >= floor && row_has(rrp, rci, piv, u, v)) atomicAdd(&recip[u], 1u);
+      if (both >= floor && row_has(rrp, rci, tree, u, v)) atomicAdd(&recip[u], 1u);
     }
   });
   if (__any_sync(FULL, bad) && lane_id() == 0) atomicOr(err, 16u);
@@ -4762,7 +4816,7 @@ struct LoadScratch {
   unsigned long long* lt_gt;   // the mirror test's two arc counts
   int32_t* fp;                 // 64 fingerprint entries
   unsigned long long* best;    // the VD root's key
-  int32_t* piv;                // pivots of the searched column array (graphs beyond the L2), else null
+  RowTree tree;                // of the searched column array (graphs beyond the L2)
   int32_t* floor_deg;          // the largest max(out, in) degree (directed graphs)
   int32_t* cnt;                // BFS level counters: slot l % 8 holds {next frontier's size, items, its arcs} of level l
   uint32_t* recip;             // n (directed graphs), else null
@@ -4791,10 +4845,23 @@ kadabra_status load_scratch(const kadabra_graph* g, LoadScratch* S) {
   const size_t o_head = 0, o_recip = up(1024), o_dist = o_recip + (g->directed ? up(4 * n) : 0);
   const size_t o_qa = o_dist + up(4 * n), o_qb = o_qa + up(4 * n), o_distb = o_qb + up(4 * n);
   const size_t o_items = o_distb + (g->directed ? up(4 * n) : 0);
-  const bool pivots = csr_bytes(g) > l2_bytes(g->device);
-  const size_t o_piv = up(o_items + sizeof(BfsItem) * (size_t)cap);
-  const size_t total = o_piv + (pivots ? 4 * ((size_t)g->m / PIVOT + 1) : 0);
-  KTRY(pool_alloc(&S->base, total));
+  S->base = nullptr;
+  S->tree.levels = 0;
+  size_t total = up(o_items + sizeof(BfsItem) * (size_t)cap), o_lv[TREE_LEVELS];
+  if (csr_bytes(g) > l2_bytes(g->device)) {
+    for (int64_t c = (g->m + (1ll << TREE_SHIFT) - 1) >> TREE_SHIFT; S->tree.levels < TREE_LEVELS; c = (c + 7) / 8) {
+      o_lv[S->tree.levels++] = total;
+      total += up(4 * (size_t)c);
+      if (c <= 1) break;
+    }
+  }
+  if (S->tree.levels && pool_alloc(&S->base, total) != KADABRA_OK) {  // no room: binary searches
+    cudaGetLastError();
+    S->tree.levels = 0;
+    total = o_lv[0];
+    S->base = nullptr;
+  }
+  if (!S->base) KTRY(pool_alloc(&S->base, total));
   unsigned char* b = static_cast<unsigned char*>(S->base);
   LoadHead* head = reinterpret_cast<LoadHead*>(b + o_head);  // device addresses
   S->err = &head->err;
@@ -4810,7 +4877,9 @@ kadabra_status load_scratch(const kadabra_graph* g, LoadScratch* S) {
   S->qa = reinterpret_cast<int32_t*>(b + o_qa);
   S->qb = reinterpret_cast<int32_t*>(b + o_qb);
   S->items = reinterpret_cast<BfsItem*>(b + o_items);
-  S->piv = pivots ? reinterpret_cast<int32_t*>(b + o_piv) : nullptr;
+  for (int k = 0; k < S->tree.levels; ++k) S->tree.lv[k] = reinterpret_cast<int32_t*>(b + o_lv[k]);
+  const int32_t* searched = g->directed ? g->rci : g->ci;
+  S->tree.groups = (reinterpret_cast<uintptr_t>(searched) & 31) ? 0 : (int32_t)(g->m / 8);
   KCK(cudaMemset(S->base, 0, 64));
   if (S->recip) KCK(cudaMemset(S->recip, 0, 4 * n));
   return KADABRA_OK;
@@ -5015,10 +5084,10 @@ kadabra_status finish_load(kadabra_graph* g) {
     k_validate_arcs<<<ba, 256>>>(g->rp, g->ci, n, m, S.err);
     if (g->directed) k_validate_arcs<<<ba, 256>>>(g->rrp, g->rci, n, m, S.err);
     tr.mark("validate rows");
-    if (S.piv) k_pivots<<<bn, 256>>>(rci, m, S.piv);
+    if (S.tree.levels) k_row_tree<<<ba, 256>>>(rci, m, S.tree);
     if (g->directed) k_floor_degree<<<bn, 256>>>(g->rp, rrp, n, S.floor_deg);
     k_validate_mirror<<<ba, 256>>>(g->rp, g->ci, rrp, rci, n, m, g->directed ? 0 : 1, S.err, S.lt_gt, S.recip,
-                                   S.floor_deg, S.piv);
+                                   S.floor_deg, S.tree);
     k_fingerprint<<<1, 64>>>(g->rp, g->ci, n, m, S.fp);
     LoadHead head;
     if (cudaMemcpy(&head, S.base, sizeof(head), cudaMemcpyDeviceToHost) != cudaSuccess) {

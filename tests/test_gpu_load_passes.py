@@ -78,6 +78,32 @@ def test_changed_entry_is_refused_beyond_l2(kd, gg):
     _refused_after_changes(kd, g, np.random.default_rng(7), 8)
 
 
+@pytest.mark.parametrize("offset", [0, 1])
+def test_device_csr_beyond_l2(kd, gg, offset):
+    """Borrowed device arrays, aligned to 32 bytes or not, with a number of
+    arcs that is no multiple of 8; the very last entry changed is refused."""
+    import torch
+    g = gg.rmat(20, 18, 0.57, 0.19, 0.19, 4)
+    assert g.m % 8, "the last group of 8 has to be a partial one"
+
+    def dev(a):
+        t = torch.empty(a.size + offset, dtype=torch.int32, device="cuda")[offset:]
+        t.copy_(torch.from_numpy(a))
+        return t
+    rp, col, rrp, rcol = (dev(a) for a in (g.row_ptr, g.col, g.rrow_ptr, g.rcol))
+    G = kd.kadabra_load_csr_device(g.n, rp, col, True, rrp, rcol)
+    vd = G.vd
+    G.free()
+    assert vd == _vd(kd, g)
+    last = int(g.rcol[-1])
+    deg = np.diff(g.rrow_ptr)
+    row = int(np.nonzero(deg)[0][-1])
+    rcol[-1] = last + 1 if last + 1 != row and last + 1 < g.n else last - 1
+    with pytest.raises(kd.KadabraError) as e:
+        kd.kadabra_load_csr_device(g.n, rp, col, True, rrp, rcol)
+    assert e.value.status == kd.ERR_CSR
+
+
 def _refused_after_changes(kd, g, rng, changes):
     """Moves one entry of the searched CSR to a free id between its
     neighbours, in short and long rows, one at a time."""
