@@ -3759,10 +3759,10 @@ struct BfsItem {
   int32_t v, begin, end, pad;
 };
 
-// scans arcs [a, b) of row c and appends the newly reached heads to next, and
-// their rows' arcs to nnext[2]
+// scans arcs [a, b) of row c and appends the newly reached heads to next;
+// arcs: their rows' arcs, of this lane's heads
 __device__ __forceinline__ void bfs_scan(const int32_t* tr, const int32_t* c, int32_t a, int32_t b, int32_t* next,
-                                         int32_t* nnext, int32_t* dist, int32_t level) {
+                                         int32_t* nnext, int32_t* dist, int32_t level, int32_t& arcs) {
   const int lane = lane_id();
   for (int32_t base = a; base < b; base += 32) {  // bounds uniform in the warp
     const int32_t e = base + lane;
@@ -3779,9 +3779,37 @@ __device__ __forceinline__ void bfs_scan(const int32_t* tr, const int32_t* c, in
       if (lane == 0) at = atomicAdd(nnext, __popc(got));
       at = __shfl_sync(FULL, at, 0);
       if (mine) next[at + __popc(got & ((1u << lane) - 1u))] = y;
-      const int32_t arcs = __reduce_add_sync(FULL, mine ? tr[y + 1] - tr[y] : 0);
-      if (lane == 0 && arcs) atomicAdd(nnext + 2, arcs);
+      if (mine) arcs += tr[y + 1] - tr[y];
     }
+  }
+}
+
+// a warp's part of the next frontier's arcs (nnext[2])
+__device__ __forceinline__ void bfs_add_arcs(int32_t arcs, int32_t* nnext) {
+  arcs = __reduce_add_sync(FULL, arcs);
+  if (lane_id() == 0 && arcs) atomicAdd(nnext + 2, arcs);
+}
+
+// Passes over all nodes that fill a queue: a warp takes up to NODE_GROUPS
+// groups of 32 nodes per reservation, since its counter takes one update at a
+// time: a reservation and an arc count per 32 nodes were the time of a
+// bottom-up level (both BFS of R-MAT scale 24 3.97 ms; 4, 16, 32 groups and
+// one arc count per warp 1.21, 1.31, 1.36 ms).
+constexpr int NODE_GROUPS = 4;
+
+// appends this lane's nodes first + 32 * q + lane (bit q of bits, q < groups) to queue, size *count
+__device__ __forceinline__ void warp_append_groups(uint32_t bits, int groups, int64_t first, int32_t* queue,
+                                                   int32_t* count) {
+  const int lane = lane_id();
+  const int total = __reduce_add_sync(FULL, __popc(bits));
+  if (!total) return;
+  int32_t at = 0;
+  if (lane == 0) at = atomicAdd(count, total);
+  at = __shfl_sync(FULL, at, 0);
+  for (int q = 0; q < groups; ++q) {
+    const unsigned got = __ballot_sync(FULL, (bits >> q) & 1u);
+    if ((bits >> q) & 1u) queue[at + __popc(got & ((1u << lane) - 1u))] = (int32_t)(first + 32 * q + lane);
+    at += __popc(got);
   }
 }
 
@@ -3808,37 +3836,41 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
   const int32_t nfront = nfront_dev ? *nfront_dev : 1;
   const int32_t arcs = nfront_dev ? nfront_dev[2] : 0;
   if (nfront > n / BFS_BOTTOM_UP || arcs > m / BFS_BOTTOM_UP_ARCS) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;  // a multiple of 32: warps stay whole
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
-      const int64_t v = base + threadIdx.x;
-      bool mine = false;
-      if (v < n && dist[v] < 0) {
-        for (int32_t e = br[v]; e < br[v + 1]; ++e)
-          if (dist[bc[e]] == level) {
-            mine = true;
-            break;
+    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+    const int groups = n >= NODE_GROUPS * nthreads ? NODE_GROUPS : 1;  // of 32 nodes per reservation
+    int32_t own = 0;
+    for (int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32 * groups; base < n;
+         base += nthreads * groups) {
+      uint32_t bits = 0;
+      for (int q = 0; q < groups; ++q) {
+        const int64_t v = base + 32 * q + lane;
+        bool mine = false;
+        if (v < n && dist[v] < 0) {
+          for (int32_t e = br[v]; e < br[v + 1]; ++e)
+            if (dist[bc[e]] == level) {
+              mine = true;
+              break;
+            }
+          if (mine) {
+            dist[v] = level + 1;  // only this thread writes v's entry
+            own += tr[v + 1] - tr[v];
+            bits |= 1u << q;
           }
-        if (mine) dist[v] = level + 1;  // only this thread writes v's entry
+        }
       }
-      const unsigned got = __ballot_sync(FULL, mine);
-      if (got) {
-        int32_t at = 0;
-        if (lane == 0) at = atomicAdd(nnext, __popc(got));
-        at = __shfl_sync(FULL, at, 0);
-        if (mine) next[at + __popc(got & ((1u << lane) - 1u))] = (int32_t)v;
-        const int32_t own = __reduce_add_sync(FULL, mine ? tr[v + 1] - tr[v] : 0);
-        if (lane == 0 && own) atomicAdd(nnext + 2, own);
-      }
+      warp_append_groups(bits, groups, base, next, nnext);
     }
+    bfs_add_arcs(own, nnext);
     return;
   }
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int32_t own = 0;
   for (int64_t i = w0; i < nfront; i += nwarps) {
     const int32_t v = front[i];
     const int32_t a = tr[v], b = tr[v + 1];
     if (b - a <= BFS_CHUNK) {
-      bfs_scan(tr, tc, a, b, next, nnext, dist, level);
+      bfs_scan(tr, tc, a, b, next, nnext, dist, level, own);
       continue;
     }
     const int32_t k = (b - a + BFS_CHUNK - 1) / BFS_CHUNK;  // items of this row
@@ -3852,8 +3884,9 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
       }
     }
     if (at + k > items_cap) bfs_scan(tr, tc, a + (items_cap > at ? items_cap - at : 0) * BFS_CHUNK, b, next, nnext,
-                                     dist, level);  // items beyond the buffer: this warp scans them
+                                     dist, level, own);  // items beyond the buffer: this warp scans them
   }
+  bfs_add_arcs(own, nnext);
 }
 
 __global__ void k_bfs_items(const int32_t* tr, const int32_t* tc, const BfsItem* items, const int32_t* nitems, int32_t items_cap,
@@ -3861,10 +3894,12 @@ __global__ void k_bfs_items(const int32_t* tr, const int32_t* tc, const BfsItem*
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int32_t k = *nitems < items_cap ? *nitems : items_cap;
+  int32_t own = 0;
   for (int64_t i = w0; i < k; i += nwarps) {
     const BfsItem it = items[i];
-    bfs_scan(tr, tc, it.begin, it.end, next, nnext, dist, level);
+    bfs_scan(tr, tc, it.begin, it.end, next, nnext, dist, level, own);
   }
+  bfs_add_arcs(own, nnext);
 }
 
 // ---- VD bound from the condensation into strongly connected components.
@@ -4064,27 +4099,24 @@ __device__ __forceinline__ long long vd_weight(const VdKahn& K, int32_t L) {
 __global__ void k_vd_kahn_init(VdKahn K, int32_t* front, int32_t* slot) {
   const int32_t n = K.n;
   const int lane = lane_id();
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = base + threadIdx.x;
-    bool mine = false;
-    if (v < n) {
+  const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+  const int groups = n >= NODE_GROUPS * nthreads ? NODE_GROUPS : 1;
+  for (int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32 * groups; base < n;
+       base += nthreads * groups) {
+    uint32_t bits = 0;
+    for (int q = 0; q < groups; ++q) {
+      const int64_t v = base + 32 * q + lane;
+      if (v >= n) continue;
       const int32_t L = K.lab[v];
-      if (K.cnt[L] == 0) {
-        if (K.sz[L] == 1)
-          mine = true;
-        else if (L == (int32_t)v) {
-          K.rdy[L] = 0;
-          slot[1] = 1;
-        }
+      if (K.cnt[L] != 0) continue;
+      if (K.sz[L] == 1) {
+        bits |= 1u << q;
+      } else if (L == (int32_t)v) {
+        K.rdy[L] = 0;
+        slot[1] = 1;
       }
     }
-    const unsigned got = __ballot_sync(FULL, mine);
-    if (got) {
-      int32_t at = 0;
-      if (lane == 0) at = atomicAdd(&slot[0], __popc(got));
-      at = __shfl_sync(FULL, at, 0);
-      if (mine) front[at + __popc(got & ((1u << lane) - 1u))] = (int32_t)v;
-    }
+    warp_append_groups(bits, groups, base, front, &slot[0]);
   }
 }
 
@@ -4198,6 +4230,7 @@ __global__ void k_vd_kahn_level(VdKahn K, int64_t m, const int32_t* front, const
     for (int k = 0; k < 4; ++k) Ly[k] = ok[k] ? K.lab[y[k]] : -1;
 #pragma unroll
     for (int k = 0; k < 4; ++k) Lu[k] = Ly[k] >= 0 && *(volatile const int32_t*)&K.cnt[Ly[k]] > 0 ? K.lab[u[k]] : Ly[k];
+    unsigned ready = 0;  // bit k: this lane's update made Ly[k], a single node, ready
 #pragma unroll 1
     for (int k = 0; k < 4; ++k) {
       const int32_t ly = k == 0 ? Ly[0] : k == 1 ? Ly[1] : k == 2 ? Ly[2] : Ly[3];
@@ -4212,13 +4245,24 @@ __global__ void k_vd_kahn_level(VdKahn K, int64_t m, const int32_t* front, const
         const int c = __popc(same);
         if (atomicSub(&K.cnt[ly], c) == c) {
           if (K.sz[ly] == 1) {
-            next[atomicAdd(&slot[0], 1)] = ly;  // a single-node component is its node
+            ready |= 1u << k;
           } else {
             K.rdy[ly] = level + 1;
             slot[1] = 1;
           }
         }
       }
+    }
+    const int total = __reduce_add_sync(FULL, __popc(ready));
+    if (!total) return;
+    int32_t at = 0;
+    if (lane_id() == 0) at = atomicAdd(&slot[0], total);
+    at = __shfl_sync(FULL, at, 0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const unsigned got = __ballot_sync(FULL, (ready >> k) & 1u);
+      if ((ready >> k) & 1u) next[at + __popc(got & ((1u << lane_id()) - 1u))] = Ly[k];  // its node
+      at += __popc(got);
     }
   });
 }
