@@ -3946,10 +3946,61 @@ __global__ void k_vd_core(const int32_t* df, const int32_t* db, int32_t n, VdCor
 #define VD_FOR_NODES(v) \
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
 
+// On power-law graphs the nodes outside the root's component have short rows,
+// and few of the arcs: passes that need only their arcs then go by node.  One
+// longer row among them (*long_rows) and the passes go by arc instead, balanced
+// whatever the rows' lengths.  R-MAT scale 24, by arc and by node: arcs
+// entering the components 1.36 -> 0.22 ms, condensation levels 3.1 -> 0.95 ms.
+constexpr int VD_LONG_ROW = 1024;
+
 __global__ void k_vd_label_init(const int32_t* df, const int32_t* db, int32_t n, const unsigned long long* best,
-                                int32_t* lab) {
+                                int32_t* lab, const int32_t* rp, const int32_t* rrp, int32_t* long_rows) {
   const int32_t r = key_root(*best);
-  VD_FOR_NODES(v) lab[v] = (df[v] >= 0 && db[v] >= 0) ? r : -1;
+  bool any = false;
+  VD_FOR_NODES(v) {
+    const bool core = df[v] >= 0 && db[v] >= 0;
+    lab[v] = core ? r : -1;
+    any |= !core && max(rp[v + 1] - rp[v], rrp[v + 1] - rrp[v]) > VD_LONG_ROW;
+  }
+  if (any) *long_rows = 1;
+}
+
+// Each lane's row [a, b) of col (empty: none): how many of its entries x have
+// p(x, key) > 0, and the largest p.  All lanes of the warp; rows beyond 16
+// entries are read by the whole warp.
+struct VdRow {
+  int32_t count;
+  long long most;
+};
+template <class P>
+__device__ __forceinline__ VdRow vd_rows(const int32_t* col, int32_t a, int32_t b, int32_t key, P p) {
+  VdRow r = {0, 0};
+  const bool own = b - a <= 16;
+  if (own)
+    for (int32_t e = a; e < b; ++e) {
+      const long long w = p(__ldg(&col[e]), key);
+      r.count += w > 0;
+      r.most = w > r.most ? w : r.most;
+    }
+  for (unsigned rows = __ballot_sync(FULL, !own); rows; rows &= rows - 1) {
+    const int j = __ffs(rows) - 1;
+    const int32_t bj = __shfl_sync(FULL, b, j), kj = __shfl_sync(FULL, key, j);
+    int32_t c = 0;
+    long long most = 0;
+    for (int32_t e = __shfl_sync(FULL, a, j) + lane_id(); e < bj; e += 32) {
+      const long long w = p(__ldg(&col[e]), kj);
+      c += w > 0;
+      most = w > most ? w : most;
+    }
+    c = __reduce_add_sync(FULL, c);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long x = __shfl_xor_sync(FULL, most, o);
+      most = x > most ? x : most;
+    }
+    if (lane_id() == j) r = VdRow{c, most};
+  }
+  return r;
 }
 
 // One trimming round.  A node of a component with two or more nodes keeps an
@@ -4034,39 +4085,65 @@ __global__ void k_vd_assign(const int32_t* col, const int32_t* reach, int32_t n,
   VD_FOR_NODES(v) if (lab[v] < 0 && reach[v]) lab[v] = col[v];
 }
 
-// component sizes, and the arcs entering each component from another.  The
-// lanes of a warp that add to the same label add once (most nodes and most
-// entering arcs of a directed power-law graph belong to the root's label).
-__global__ void k_vd_sizes(const int32_t* lab, int32_t n, int32_t* sz) {
+// component sizes (the root's is known), and the arcs entering each component
+// from another.  The lanes of a warp that add to the same label add once.
+__global__ void k_vd_sizes(const int32_t* lab, int32_t n, const unsigned long long* best, const VdCore* core,
+                           int32_t* sz) {
+  const int32_t root = key_root(*best);
+  if (blockIdx.x == 0 && threadIdx.x == 0) sz[root] = (int32_t)core->size;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = base + threadIdx.x;
-    const int32_t L = v < n ? lab[v] : -1;
-    const unsigned same = __match_any_sync(FULL, L);
-    if (L >= 0 && lane_id() == __ffs(same) - 1) atomicAdd(&sz[L], __popc(same));
+    const int32_t L = v < n ? lab[v] : root;
+    if (__any_sync(FULL, L != root && L != v)) {
+      const unsigned same = __match_any_sync(FULL, L);
+      if (L != root && lane_id() == __ffs(same) - 1) atomicAdd(&sz[L], __popc(same));
+    } else if (L != root) {
+      atomicAdd(&sz[L], 1);
+    }
   }
 }
 
-__global__ void k_vd_indeg(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m, const int32_t* lab,
-                           const unsigned long long* best, int32_t* cnt) {
+__global__ void k_vd_indeg(const int32_t* rp, const int32_t* ci, const int32_t* rrp, const int32_t* rci, int32_t n,
+                           int64_t m, const int32_t* lab, const unsigned long long* best, const int32_t* long_rows,
+                           int32_t* cnt) {
   const int32_t root = key_root(*best);
   // the arcs into the root's component, most of all, are counted per warp
   unsigned into_root = 0;
-  for_each_arc<4>(rp, ci, n, m, [&](const bool* ok, const int32_t* u, const int64_t*, const int32_t* v) {
-    int32_t lu[4], lv[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      lu[k] = ok[k] ? __ldg(&lab[u[k]]) : 0;
-      lv[k] = ok[k] ? __ldg(&lab[v[k]]) : 0;
+  if (!*long_rows) {  // every entering arc leaves or enters a node outside the root's component
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
+      const int64_t v = base + threadIdx.x;
+      const int32_t L = v < n ? lab[v] : root;
+      if (!__any_sync(FULL, L != root)) continue;
+      int32_t a = 0, b = 0, ra = 0, rb = 0;
+      if (L != root) {
+        a = rp[v];
+        b = rp[v + 1];
+        ra = rrp[v];
+        rb = rrp[v + 1];
+      }
+      into_root += vd_rows(ci, a, b, root, [&](int32_t x, int32_t k) { return (long long)(__ldg(&lab[x]) == k); }).count;
+      const int32_t c =
+          vd_rows(rci, ra, rb, L, [&](int32_t x, int32_t k) { return (long long)(__ldg(&lab[x]) != k); }).count;
+      if (c) atomicAdd(&cnt[L], c);
     }
+  } else {
+    for_each_arc<4>(rp, ci, n, m, [&](const bool* ok, const int32_t* u, const int64_t*, const int32_t* v) {
+      int32_t lu[4], lv[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (lu[k] == lv[k]) continue;
-      if (lv[k] == root)
-        ++into_root;
-      else
-        atomicAdd(&cnt[lv[k]], 1);
-    }
-  });
+      for (int k = 0; k < 4; ++k) {
+        lu[k] = ok[k] ? __ldg(&lab[u[k]]) : 0;
+        lv[k] = ok[k] ? __ldg(&lab[v[k]]) : 0;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (lu[k] == lv[k]) continue;
+        if (lv[k] == root)
+          ++into_root;
+        else
+          atomicAdd(&cnt[lv[k]], 1);
+      }
+    });
+  }
   into_root = __reduce_add_sync(FULL, into_root);
   if (into_root && lane_id() == 0) atomicAdd(&cnt[root], (int32_t)into_root);
 }
@@ -4089,6 +4166,7 @@ struct VdKahn {
   int32_t root_label;
   long long root_w;
   long long* vd;
+  const int32_t* long_rows;
 };
 
 __device__ __forceinline__ long long vd_weight(const VdKahn& K, int32_t L) {
@@ -4220,6 +4298,47 @@ __global__ void k_vd_kahn_level(VdKahn K, int64_t m, const int32_t* front, const
   VD_FOR_NODES(v) {
     const int32_t L = K.lab[v];
     if (L == (int32_t)v && K.sz[L] > 1 && K.rdy[L] == level) atomicMax(K.vd, vd_weight(K, L) + K.best[L]);
+  }
+  // The root's component was ready at this level or before (a value that this
+  // level's launch leaves as it is, or moves from -1 to level + 1): the nodes
+  // still waiting are outside it, and all their rows are short.
+  const int32_t root_rdy = *(volatile const int32_t*)&K.rdy[K.root_label];
+  if (!*K.long_rows && root_rdy >= 0 && root_rdy <= level) {
+    const int lane = lane_id();
+    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+    const int groups = n >= NODE_GROUPS * nthreads ? NODE_GROUPS : 1;
+    for (int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32 * groups; base < n;
+         base += nthreads * groups) {
+      uint32_t ready = 0;
+      for (int q = 0; q < groups; ++q) {
+        const int64_t y = base + 32 * q + lane;
+        int32_t L = K.root_label, a = 0, b = 0;
+        if (y < n) L = K.lab[y];
+        const bool waits = *(volatile const int32_t*)&K.cnt[L] > 0;
+        if (!__any_sync(FULL, waits)) continue;
+        if (waits && y < n) {
+          a = K.rrp[y];
+          b = K.rrp[y + 1];
+        }
+        const VdRow r = vd_rows(K.rci, a, b, L, [&](int32_t u, int32_t ly) {
+          const int32_t lu = K.lab[u];
+          return lu != ly && K.sz[lu] > 1 && K.rdy[lu] == level ? vd_weight(K, lu) + K.best[lu] : 0ll;
+        });
+        if (r.count) {
+          atomicMax(&K.best[L], r.most);
+          if (atomicSub(&K.cnt[L], r.count) == r.count) {
+            if (K.sz[L] == 1) {
+              ready |= 1u << q;  // a single-node component is its node
+            } else {
+              K.rdy[L] = level + 1;
+              slot[1] = 1;
+            }
+          }
+        }
+      }
+      warp_append_groups(ready, groups, base, next, &slot[0]);
+    }
+    return;
   }
   // Pulled along the in-arcs of the components still waiting: those are few
   // on power-law graphs (the ready giant component holds most arcs), and a
@@ -4985,7 +5104,7 @@ kadabra_status vd_condensation(kadabra_graph* g, LoadTrace& tr, const LoadScratc
     ~Free() { pool_free(p); }
   } guard{base};
   unsigned char* b = static_cast<unsigned char*>(base);
-  int32_t* flag = reinterpret_cast<int32_t*>(b);              // [0] a change, [1] an unlabelled node
+  int32_t* flag = reinterpret_cast<int32_t*>(b);              // [0] a change, [1] an unlabelled node, [2] a long row
   int32_t* slots = reinterpret_cast<int32_t*>(b + 64);        // 8 level slots of 2
   long long* vd = reinterpret_cast<long long*>(b + 128);
   int32_t* lab = reinterpret_cast<int32_t*>(b + 256);
@@ -4995,7 +5114,8 @@ kadabra_status vd_condensation(kadabra_graph* g, LoadTrace& tr, const LoadScratc
   int32_t* cnt = reinterpret_cast<int32_t*>(b + 256 + 4 * N4);
   int32_t* rdy = reinterpret_cast<int32_t*>(b + 256 + 5 * N4);
   long long* best = reinterpret_cast<long long*>(b + 256 + 6 * N4);
-  k_vd_label_init<<<bn, 256>>>(S.dist, db, n, S.best, lab);
+  KCK(cudaMemsetAsync(flag, 0, 3 * sizeof(int32_t)));
+  k_vd_label_init<<<bn, 256>>>(S.dist, db, n, S.best, lab, g->rp, rrp, flag + 2);
   KCK(cudaGetLastError());
   // repeats a kernel (4 queued rounds per read-back) until a round changes nothing
   auto until_stable = [&](auto&& round) -> kadabra_status {
@@ -5028,13 +5148,13 @@ kadabra_status vd_condensation(kadabra_graph* g, LoadTrace& tr, const LoadScratc
   KCK(cudaMemsetAsync(rdy, 0xFF, N4));
   KCK(cudaMemsetAsync(best, 0, N8));
   KCK(cudaMemsetAsync(b + 64, 0, 192));  // slots, vd
-  k_vd_sizes<<<bn, 256>>>(lab, n, sz);
-  k_vd_indeg<<<ba, 256>>>(g->rp, g->ci, n, m, lab, S.best, cnt);
+  k_vd_sizes<<<bn, 256>>>(lab, n, S.best, S.core, sz);
+  k_vd_indeg<<<ba, 256>>>(g->rp, g->ci, rrp, rci, n, m, lab, S.best, flag + 2, cnt);
   unsigned long long key = 0;
   if (cudaMemcpy(&key, S.best, sizeof(key), cudaMemcpyDeviceToHost) != cudaSuccess)
     return fail(KADABRA_ERR_CUDA, "vd bound");
   VdKahn K{g->rp, g->ci, rrp, rci, lab, sz, cnt, best, rdy, n, (int32_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull)),
-           root_w, vd};
+           root_w, vd, flag + 2};
   constexpr int SLOTS = 8, BATCH = 4;
   k_vd_kahn_init<<<bn, 256>>>(K, S.qa, slots + 2 * (SLOTS - 1));  // the slot level 0 reads
   KCK(cudaGetLastError());

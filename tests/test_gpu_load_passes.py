@@ -61,6 +61,31 @@ def test_components(kd, orc, gg):
     assert _vd(kd, und) == orc.vd_bound(und)
 
 
+@pytest.mark.parametrize("hub", [0, 1024, 1025])
+def test_outside_the_core(kd, orc, gg, hub):
+    """A large component, nodes before and behind it with rows of 0 to 40
+    arcs, a second component behind it that chains into more nodes, and a
+    node with `hub` in-arcs, whose row decides whether the passes over the
+    other components go by node or by arc."""
+    rng = np.random.default_rng(11)
+    core, out, src = 2500, 3000, 1500
+    e = [(i, (i + 1) % core) for i in range(core)] + [(0, i) for i in range(2, core)] + [(i, 0) for i in range(3, core)]
+    for i in range(out):  # behind the core: i % 41 in-arcs from it, some from the nodes before
+        y = core + i
+        e += [(int(u), y) for u in rng.choice(core, i % 41, replace=False)]
+        e += [(core + i - k, y) for k in (1, 7, 32) if i >= k and i % (k + 2) == 0]
+    base = core + out
+    e += [(base + i, (base + (i + 1) % 50)) for i in range(50)] + [(5, base), (base + 3, base + 50)]
+    e += [(base + 50 + i, base + 51 + i) for i in range(60)]
+    first = base + 111
+    for i in range(src):  # before it
+        e += [(first + i, int(u)) for u in rng.choice(core + out, i % 19, replace=False)]
+    n = first + src + 1
+    e += [(int(u), n - 1) for u in rng.choice(core, hub, replace=False)]
+    g = _directed(gg, n, e, f"core{hub}")
+    assert _vd(kd, g) == orc.vd_bound(g)
+
+
 @pytest.mark.parametrize("directed", [False, True])
 def test_changed_entry_is_refused(kd, gg, directed):
     rng = np.random.default_rng(3)
