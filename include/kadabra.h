@@ -93,7 +93,9 @@ typedef struct {
                               of table and warp tier; the choice is cached per graph
                               fingerprint), or one of the two values the library
                               offers (4: 4096-slot tables, lists of 3072 nodes; 5:
-                              the compact layout, lists of 2048 nodes; on GB300);
+                              the compact layout, lists of 2048 nodes, or on graphs
+                              of at most 16384 nodes the small one, 2048 slots and
+                              seven CTAs per SM; on GB300);
                               any other value is KADABRA_ERR_ARG.  Results do not
                               depend on it.  A batch run tunes it on its largest
                               graph; serving uses the default.                    */

@@ -110,8 +110,17 @@ namespace {
 // 65,536 samples with 8 warps, with 6, and in the default layout: Chung-Lu of
 // 10^5 nodes 2.07, 1.57, 1.73 ms, of 10^6 nodes 3.45, 2.97, 2.95 ms; 8,192 of
 // ER 2,000 nodes 266, 188, 214 us; 16,384 of BA 300,000 nodes 800, 656, 713 us.
+// The small tier-S layout, the compact one's place on graphs of few nodes: 4
+// warps, 2048 slots, seven CTAs per SM, so that a batch of 1,000 samples runs at
+// once and a sample's barriers join fewer warps.  Runs at K near 1,000 with the
+// compact layout and with it: ER of 2,000 nodes 1.02 -> 0.91 ms, of 8,000 1.14 ->
+// 1.01, of 32,000 1.28 -> 1.28; Chung-Lu of 4,000 nodes 0.98 -> 0.91, of 16,000
+// 1.24 -> 1.24; BA of 4,000 nodes 1.67 -> 1.51, of 16,000 1.60 -> 1.60; ER of 3.4 M
+// nodes 7.9 -> 8.4 ms, hence TINY_NODES.  Eight CTAs per SM, or 3 warps: the same.
 constexpr int NW_S = KD_NT / 32;
 constexpr int NW_CMP = 6;
+constexpr int NW_TINY = 4;
+constexpr int TINY_NODES = 16384;  // largest graph whose launches take it
 constexpr int NW_BIG = KD_NT_BIG / 32;
 constexpr int U = KD_U;            // independent items per thread per step (memory-level parallelism)
 // Tiers of per-sample tables.  A sample starts in a small shared-memory
@@ -2072,9 +2081,13 @@ struct SLayout {
 using FastLayout = SLayout<NW_S, FAST_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
 using CompactLayout = SLayout<NW_CMP, FAST_HLOG, KD_CMP_L8, 512, KD_CMP_FLOG, KD_CMP_MAXD, false>;
 using BigLayout = SLayout<NW_BIG, BIG_HLOG, 2 * KD_LOAD_QUARTERS, FRONTIER_SEG, FILTER_LOG, FAST_MAXD, true>;
+using TinyLayout = SLayout<NW_TINY, 11, 6, 512, 13, KD_CMP_MAXD, false>;
 // the tier-S layout a k_sample instance uses (SL)
 constexpr int SL_FAST = 0;
 constexpr int SL_COMPACT = 1;
+constexpr int SL_TINY = 2;
+template <int SL>
+using TierSLayout = std::conditional_t<SL == SL_FAST, FastLayout, std::conditional_t<SL == SL_TINY, TinyLayout, CompactLayout>>;
 
 template <class L>
 __device__ inline Tables smem_tables(unsigned char* smem) {
@@ -2107,6 +2120,7 @@ constexpr int TF_VEC = 16;  // pass 1 searches long rows (graphs beyond the L2)
 constexpr int TF_SEG64 = 32;  // shared-memory tiers scan frontiers in 64-node segments (tests)
 constexpr int TF_COMPACT = 64;  // tier S in the compact layout, whatever the launch's variant
 constexpr int TF_SCREEN = 128;  // k_screen first: tier S takes only the samples whose roots have arcs
+constexpr int TF_TINY = 256;  // the small layout where the launch's variant asks for the compact one
 
 // queue counters in SampleParams::ctr
 constexpr int Q_NEXT_A = 0;   // next sample index of the batch
@@ -2199,14 +2213,17 @@ __device__ void finish_sample(const SampleParams& P, Ctl<NW>& c, int64_t out_i) 
 // MODE 0: every sample of the batch, on tier S; overflow -> tier-B queue.
 // MODE 2: the tier-B queue, on tier B, then tier M; overflow -> tier-L queue.
 // MODE 1: the tier-L queue, on tier L.
-// SL: the tier-S layout of MODE 0; the compact one fits one more CTA per SM
-// and gives the same results (samples that outgrow it go on to tier B as
-// usual).  RG (the default layout only): pass 1 searches long rows (for
+// SL: the tier-S layout of MODE 0; the compact and the small one fit more CTAs
+// per SM and give the same results (samples that outgrow them go on to tier B
+// as usual).  RG (the default layout only): pass 1 searches long rows (for
 // graphs whose CSR exceeds L2); same results.
 template <int MODE, int SL = SL_FAST>
-constexpr int MODE_NW = MODE == 2 ? NW_BIG : SL == SL_COMPACT ? NW_CMP : NW_S;
+constexpr int MODE_NW = MODE == 2 ? NW_BIG : SL == SL_COMPACT ? NW_CMP : SL == SL_TINY ? NW_TINY : NW_S;
+template <int MODE, int SL>
+constexpr int MODE_CTAS =
+    MODE == 2 ? 1 : MODE == 1 ? 2 : SL == SL_FAST ? KD_MIN_BLOCKS : SL == SL_TINY ? 7 : KD_MIN_BLOCKS + 1;
 template <int MODE, int SL = SL_FAST, bool RG = false>
-__global__ void __launch_bounds__(32 * MODE_NW<MODE, SL>, MODE == 2 ? 1 : MODE == 1 ? 2 : SL == SL_FAST ? KD_MIN_BLOCKS : KD_MIN_BLOCKS + 1)
+__global__ void __launch_bounds__(32 * MODE_NW<MODE, SL>, MODE_CTAS<MODE, SL>)
     k_sample(SampleParams P) {
   static_assert(!RG || SL == SL_FAST, "the beyond-L2 scan has no compact-layout instance");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -2214,7 +2231,7 @@ __global__ void __launch_bounds__(32 * MODE_NW<MODE, SL>, MODE == 2 ? 1 : MODE =
   Ctl<NW>& c = *reinterpret_cast<Ctl<NW>*>(smem);
   Tables TS, TM;
   PiEntry* pi = P.pi_base + (size_t)blockIdx.x * PI_SEGS * P.pcap;
-  if (MODE == 0) TS = smem_tables<std::conditional_t<SL == SL_FAST, FastLayout, CompactLayout>>(smem);
+  if (MODE == 0) TS = smem_tables<TierSLayout<SL>>(smem);
   if (MODE == 2) {
     TS = smem_tables<BigLayout>(smem);
     TM = gm_tables(P.med_base + (size_t)blockIdx.x * P.med_stride, P.med_hlog, P.med_lcap, MED_MAXD);
@@ -2800,6 +2817,7 @@ size_t warp_tier_smem_bytes() { return sizeof(WSlot) * WT_WARPS; }
 
 size_t fast_smem_bytes() { return FastLayout::BYTES; }
 size_t compact_smem_bytes() { return CompactLayout::BYTES; }
+size_t tiny_smem_bytes() { return TinyLayout::BYTES; }
 size_t big_smem_bytes() { return BigLayout::BYTES; }
 
 // ============================================================== stop test
@@ -4445,8 +4463,8 @@ struct Workspace {
   int device = 0, num_sms = 0;
   int32_t max_n = 0;
   int64_t max_m = 0;
-  int grid_fast = 0, grid_big = 0, grid_gm = 0, grid_compact = 0, grid_warp = 0;
-  size_t smem_fast = 0, smem_big = 0, smem_compact = 0, smem_warp = 0;
+  int grid_fast = 0, grid_big = 0, grid_gm = 0, grid_compact = 0, grid_tiny = 0, grid_warp = 0;
+  size_t smem_fast = 0, smem_big = 0, smem_compact = 0, smem_tiny = 0, smem_warp = 0;
   unsigned long long* ctr = nullptr;
   int32_t* status = nullptr;
   unsigned long long* qb = nullptr;  // queue for tier B
@@ -4528,12 +4546,15 @@ constexpr uint32_t FLAG_VEC_AUTO = 1u << 31;
 constexpr uint32_t FLAG_SCREEN_AUTO = 1u << 30;
 constexpr double SCREEN_MIN = 0.25;
 constexpr uint64_t SCREEN_SAMPLES = 8192;
+// internal launch flag: no graph of the launch has more than TINY_NODES nodes
+constexpr uint32_t FLAG_TINY_AUTO = 1u << 29;
 // the flags a launch shared by several graphs takes from any of them (they
 // change no result; the tier-skipping flags stay per graph)
 constexpr uint32_t SHARED_LAUNCH_FLAGS = KADABRA_FLAG_WARP_TIER | KADABRA_FLAG_ASYNC_SCAN | FLAG_VEC_AUTO | FLAG_SCREEN_AUTO;
 
 uint32_t launch_flags(const kadabra_graph* g) {
-  return g->flags | (g->csr_beyond_l2 ? FLAG_VEC_AUTO : 0u) | (g->screened ? FLAG_SCREEN_AUTO : 0u);
+  return g->flags | (g->csr_beyond_l2 ? FLAG_VEC_AUTO : 0u) | (g->screened ? FLAG_SCREEN_AUTO : 0u) |
+         (g->n <= TINY_NODES ? FLAG_TINY_AUTO : 0u);
 }
 }  // namespace
 
@@ -4632,6 +4653,10 @@ kadabra_status ensure_ws(Workspace* w, uint64_t deferred_need, int njobs) {
     KCK(cudaFuncSetAttribute(k_sample<0, SL_COMPACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_compact));
     KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0, SL_COMPACT>, 32 * NW_CMP, w->smem_compact));
     w->grid_compact = w->num_sms * std::max(per_sm, 1);
+    w->smem_tiny = tiny_smem_bytes();
+    KCK(cudaFuncSetAttribute(k_sample<0, SL_TINY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_tiny));
+    KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<0, SL_TINY>, 32 * NW_TINY, w->smem_tiny));
+    w->grid_tiny = w->num_sms * std::max(per_sm, 1);
     w->smem_warp = warp_tier_smem_bytes();
     KCK(cudaFuncSetAttribute(k_sample_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->smem_warp));
     KCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample_warp, 32 * WT_WARPS, w->smem_warp));
@@ -4764,6 +4789,7 @@ SampleParams ws_params(const Workspace* w, uint32_t flags) {
   if (flags & KADABRA_FLAG_FRONTIER_SEGMENTS) P.tier_flags |= TF_SEG64;
   if (flags & KADABRA_FLAG_COMPACT_TABLES) P.tier_flags |= TF_COMPACT;
   if (flags & FLAG_SCREEN_AUTO) P.tier_flags |= TF_SCREEN;
+  if (flags & FLAG_TINY_AUTO) P.tier_flags |= TF_TINY;
   return P;
 }
 
@@ -4776,7 +4802,8 @@ SampleParams base_params(kadabra_graph* g) {
 // launches the main sampler grid, then the large-table pass and the
 // n-sized-table pass for the samples queued by the launch before (each exits
 // at once when its queue is empty)
-// variant bit 0: the compact tier-S layout with one more CTA per SM
+// variant bit 0: the compact tier-S layout with one more CTA per SM, or on
+// graphs of at most TINY_NODES nodes the small one
 // variant bit 1: tier W (one warp per sample) first; tier S takes only the
 // samples it queues
 kadabra_status launch_sampler_kernels(Workspace* w, SampleParams P, cudaStream_t st, int variant = 0) {
@@ -4792,7 +4819,12 @@ kadabra_status launch_sampler_kernels(Workspace* w, SampleParams P, cudaStream_t
     KCK(cudaGetLastError());
   }
   const bool rg = (P.tier_flags & TF_VEC) != 0;
-  if ((variant & 1) || ((P.tier_flags & TF_COMPACT) && !rg))  // the compact layout has no beyond-L2 variant
+  if ((variant & 1) && (P.tier_flags & TF_TINY) && !(P.tier_flags & TF_COMPACT)) {
+    // more CTAs share the candidate buffers; a sample beyond its part goes on to tier B
+    SampleParams T = P;
+    T.pcap = (int)((int64_t)FAST_PCAP * std::max(w->grid_fast, w->grid_compact) / w->grid_tiny);
+    k_sample<0, SL_TINY><<<w->grid_tiny, 32 * NW_TINY, w->smem_tiny, st>>>(T);
+  } else if ((variant & 1) || ((P.tier_flags & TF_COMPACT) && !rg))  // the compact layout has no beyond-L2 variant
     k_sample<0, SL_COMPACT><<<w->grid_compact, 32 * NW_CMP, w->smem_compact, st>>>(P);
   else if (rg)
     k_sample<0, SL_FAST, true><<<w->grid_fast, 32 * NW_S, w->smem_fast, st>>>(P);
@@ -5736,6 +5768,8 @@ kadabra_status run_graphs(Workspace* w, kadabra_graph* const* gs, int G, const d
   // any of them asks for it (it changes no result)
   uint32_t fl = G == 1 ? launch_flags(gs[0]) : 0;
   if (G > 1)
+    fl = FLAG_TINY_AUTO;
+    for (int i = 0; i < G; ++i) fl &= launch_flags(gs[i]);
     for (int i = 0; i < G; ++i) fl |= launch_flags(gs[i]) & SHARED_LAUNCH_FLAGS;
   auto launch_jobs = [&]() -> kadabra_status {
     uint64_t work = 0;

@@ -107,3 +107,28 @@ def test_screened_batch_run(kd, gg):
             assert np.array_equal(r.totals, one.totals) and (r.max_f, r.max_g) == (one.max_f, one.max_g)
     finally:
         B.free()
+
+
+def _chain(gg, width, layers=5):
+    e = [(a * width + i, (a + 1) * width + j) for a in range(layers - 1) for i in range(width) for j in range(width)]
+    return gg.from_edges(layers * width, e, name=f"chain{width}")
+
+
+@pytest.mark.parametrize("make", [
+    lambda gg: gg.erdos_renyi(16384, 8.0, 3, lcc=False), lambda gg: gg.erdos_renyi(16385, 8.0, 3, lcc=False),
+    lambda gg: gg.erdos_renyi(12000, 30.0, 5), lambda gg: _chain(gg, 11), lambda gg: _chain(gg, 12),
+    lambda gg: _chain(gg, 100), lambda gg: _chain(gg, 155), lambda gg: _chain(gg, 175),
+    lambda gg: gg.barabasi_albert(5000, 7, 2), lambda gg: gg.rmat(12, 8, 0.57, 0.19, 0.19, 2),
+], ids=["er16384", "er16385", "er12000", "chain11", "chain12", "chain100", "chain155", "chain175", "ba5000", "rmat12"])
+def test_small_layout(kd, gg, make):
+    """The layouts of ctas_per_sm 5, the small one up to 16,384 nodes, against
+    the default one: samples that outgrow 1,536 list nodes, and candidate sets
+    around 128 (one per thread) and beyond the small layout's share of the
+    buffers (about 23,000)."""
+    g = make(gg)
+    G = kd.kadabra_load_csr(g)
+    try:
+        a, b = (kd.kadabra_run(G, 0.02, 0.1, 0, 5, check_interval=1000, ctas_per_sm=c, warp_tier=-1) for c in (4, 5))
+    finally:
+        G.free()
+    assert a.tau == b.tau and np.array_equal(a.counts, b.counts) and np.array_equal(a.totals, b.totals)
