@@ -5149,9 +5149,10 @@ kadabra_status vd_condensation(kadabra_graph* g, LoadTrace& tr, const LoadScratc
   KCK(cudaMemsetAsync(flag, 0, 3 * sizeof(int32_t)));
   k_vd_label_init<<<bn, 256>>>(S.dist, db, n, S.best, lab, g->rp, rrp, flag + 2);
   KCK(cudaGetLastError());
-  // repeats a kernel (4 queued rounds per read-back) until a round changes nothing
+  // repeats a kernel (4 queued rounds per read-back) until a round changes
+  // nothing: at most n rounds change something, then one read-back more
   auto until_stable = [&](auto&& round) -> kadabra_status {
-    for (int64_t it = 0; it <= (int64_t)n; it += 4) {
+    for (int64_t it = 0; it < (int64_t)n + 4; it += 4) {
       KCK(cudaMemsetAsync(flag, 0, sizeof(int32_t)));
       for (int k = 0; k < 4; ++k) round();
       int32_t h = 0;
