@@ -3512,7 +3512,8 @@ __device__ __forceinline__ void for_each_arc(const int32_t* rp, const int32_t* c
   const int lane = lane_id();
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   // a graph with less than ARC_CHUNK arcs per warp is spread over all of them
-  const int64_t per = (m + nwarps - 1) / nwarps;
+  // (at least one window each, so a graph without arcs has no chunk)
+  const int64_t per = max((m + nwarps - 1) / nwarps, (int64_t)1);
   const int64_t chunk = per < ARC_CHUNK ? (per + 31) / 32 * 32 : ARC_CHUNK;
   const int64_t chunks = (m + chunk - 1) / chunk;
   for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < chunks; c += nwarps) {

@@ -44,3 +44,26 @@ def test_chains_of_few_nodes(kd, orc, gg, n):
         vd = G.vd
         G.free()
         assert vd == orc.vd_bound(g), e
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("n", [2, 33, 20000])
+def test_graph_without_arcs(kd, orc, gg, n, directed):
+    """No arcs at all: the arc passes have no chunk to take.  The bound, a run
+    and a batch equal the oracle's."""
+    g = gg.from_edges(n, [], directed=directed, name=f"edgeless{n}_{int(directed)}")
+    ref = orc.run(g, 0.05, 0.1, seed=3, K=500)
+    G = kd.kadabra_load_csr(g)
+    try:
+        assert G.vd == orc.vd_bound(g)
+        got = kd.kadabra_run(G, 0.05, 0.1, 0, 3, check_interval=500)
+    finally:
+        G.free()
+    B = kd.Batch([g, g])
+    try:
+        rb = B.run([0.05] * 2, [0.1] * 2, [3, 3], check_interval=500)
+    finally:
+        B.free()
+    for r in (got, *rb):
+        assert r.tau == ref.tau and r.C == ref.C and (r.max_f, r.max_g) == (ref.max_f, ref.max_g)
+        assert np.array_equal(r.counts, ref.counts)
