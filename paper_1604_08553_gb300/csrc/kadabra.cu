@@ -3506,7 +3506,8 @@ __device__ __forceinline__ int32_t warp_row_of_arc(const int32_t* rp, int32_t n,
 // ok[k] = there is one), with all lanes of the warp.  The lanes' rows come
 // from the starts of the next rows, 32 at a time, counted by a search over
 // the lanes' registers (several rounds only where rows are so short, or
-// empty, that more than 32 start in a window).
+// empty, that more than 32 start in a window).  Window ends are cut to the
+// chunk's arcs, below 2^31 - 1, the start that stands for "no more rows".
 template <int D, class F>
 __device__ __forceinline__ void for_each_arc(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m, F f) {
   const int lane = lane_id();
@@ -3531,16 +3532,17 @@ __device__ __forceinline__ void for_each_arc(const int32_t* rp, const int32_t* c
       }
 #pragma unroll
       for (int k = 0; k < D; ++k) {
-        const int64_t last = base + 32 * k + 31;
+        const int32_t last = (int32_t)min(base + 32 * k + 31, e1 - 1);
+        const int32_t at = (int32_t)min(e[k], (int64_t)last);
         u[k] = row;
         for (int32_t r = row;; r += 32) {
-          const int32_t st = r + 1 + lane < n ? __ldg(&rp[r + 1 + lane]) : 0x7FFFFFFF;  // no arc has this index
+          const int32_t st = r + 1 + lane < n ? __ldg(&rp[r + 1 + lane]) : 0x7FFFFFFF;  // above every arc's index
           if (!__any_sync(FULL, st <= last)) break;
-          int q = 0;  // how many of the 32 rows start at e or before
+          int q = 0;  // how many of the 32 rows start at the lane's arc or before
 #pragma unroll
           for (int h = 16; h > 0; h >>= 1)
-            if (__shfl_sync(FULL, st, q + h - 1) <= e[k]) q += h;
-          if (__shfl_sync(FULL, st, q) <= e[k]) ++q;
+            if (__shfl_sync(FULL, st, q + h - 1) <= at) q += h;
+          if (__shfl_sync(FULL, st, q) <= at) ++q;
           if (q > 0) u[k] = r + q;
           if (__shfl_sync(FULL, st, 31) > last) break;
         }
@@ -3783,8 +3785,8 @@ struct BfsItem {
 __device__ __forceinline__ void bfs_scan(const int32_t* tr, const int32_t* c, int32_t a, int32_t b, int32_t* next,
                                          int32_t* nnext, int32_t* dist, int32_t level, int32_t& arcs) {
   const int lane = lane_id();
-  for (int32_t base = a; base < b; base += 32) {  // bounds uniform in the warp
-    const int32_t e = base + lane;
+  for (int64_t base = a; base < b; base += 32) {  // bounds uniform in the warp
+    const int64_t e = base + lane;
     int32_t y = 0;
     bool mine = false;
     if (e < b) {
@@ -3899,7 +3901,7 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
     for (int32_t q = lane; q < k; q += 32) {
       if (at + q < items_cap) {
         const int32_t s = a + q * BFS_CHUNK;
-        items[at + q] = BfsItem{v, s, s + BFS_CHUNK < b ? s + BFS_CHUNK : b, 0};
+        items[at + q] = BfsItem{v, s, b - s > BFS_CHUNK ? s + BFS_CHUNK : b, 0};
       }
     }
     if (at + k > items_cap) bfs_scan(tr, tc, a + (items_cap > at ? items_cap - at : 0) * BFS_CHUNK, b, next, nnext,
@@ -4006,7 +4008,7 @@ __device__ __forceinline__ VdRow vd_rows(const int32_t* col, int32_t a, int32_t 
     const int32_t bj = __shfl_sync(FULL, b, j), kj = __shfl_sync(FULL, key, j);
     int32_t c = 0;
     long long most = 0;
-    for (int32_t e = __shfl_sync(FULL, a, j) + lane_id(); e < bj; e += 32) {
+    for (int64_t e = (int64_t)__shfl_sync(FULL, a, j) + lane_id(); e < bj; e += 32) {
       const long long w = p(__ldg(&col[e]), kj);
       c += w > 0;
       most = w > most ? w : most;
@@ -4231,8 +4233,8 @@ struct VdWarp {
 __device__ __forceinline__ void vd_kahn_row(const VdKahn& K, int32_t u, long long w, int32_t a, int32_t b,
                                             int32_t level, int32_t* next, int32_t* slot, VdWarp& W) {
   const int lane = lane_id();
-  for (int32_t base = a; base < b; base += 32) {
-    const int32_t e = base + lane;
+  for (int64_t base = a; base < b; base += 32) {
+    const int64_t e = base + lane;
     bool push = false;
     int32_t Ly = u;  // this lane's arc enters no other component unless set below
     if (e < b) Ly = K.lab[K.ci[e]];

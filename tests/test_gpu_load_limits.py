@@ -67,3 +67,116 @@ def test_graph_without_arcs(kd, orc, gg, n, directed):
     for r in (got, *rb):
         assert r.tau == ref.tau and r.C == ref.C and (r.max_f, r.max_g) == (ref.max_f, ref.max_g)
         assert np.array_equal(r.counts, ref.counts)
+
+
+def _clique_rows(c, groups, tail, device="cuda"):
+    """Columns of a clique's rows on ids [0, c), in order, with ids c, c + 1, ..
+    appended to the lower rows: groups is a list of (rows up to, extra ids)."""
+    import torch
+    total = sum((hi - lo) * (c - 1 + x) for (lo, hi, x) in _ranges(groups)) + tail
+    out = torch.empty(total, dtype=torch.int32, device=device)
+    t = torch.arange(c - 1, dtype=torch.int32, device=device)
+    at = 0
+    for lo, hi, x in _ranges(groups):
+        for a in range(lo, hi, 2000):
+            u = torch.arange(a, min(a + 2000, hi), dtype=torch.int32, device=device)[:, None]
+            m = t + (t >= u).to(torch.int32)
+            if x:
+                m = torch.cat([m, torch.arange(c, c + x, dtype=torch.int32, device=device).expand(len(u), x)], 1)
+            out[at:at + m.numel()] = m.reshape(-1)
+            at += m.numel()
+    return out, at
+
+
+def _ranges(groups):
+    lo = 0
+    for hi, x in groups:
+        yield lo, hi, x
+        lo = hi
+
+
+def _offsets(deg):
+    import torch
+    rp = np.concatenate([[0], np.cumsum(deg, dtype=np.int64)])
+    return torch.from_numpy(rp.astype(np.int32)).cuda(), int(rp[-1])
+
+
+# a clique of 46,000 nodes and 1,000 pendant nodes, pendant j joined to the
+# clique's nodes [0, 15,765) or, from the 824th on, [0, 15,764)
+CLIQUE, PENDANTS, JOINED, LONGER = 46000, 1000, 15764, 823
+
+
+@pytest.fixture(scope="module")
+def largest(kd):
+    """An undirected graph of 2^31 - 2 arcs on the device, the most there can be."""
+    import torch
+    groups = [(JOINED, PENDANTS), (JOINED + 1, LONGER), (CLIQUE, 0)]
+    q = np.full(PENDANTS, JOINED) + (np.arange(PENDANTS) < LONGER)
+    col, at = _clique_rows(CLIQUE, groups, int(q.sum()))
+    for k in q:
+        torch.arange(int(k), dtype=torch.int32, device="cuda", out=col[at:at + int(k)])
+        at += int(k)
+    deg = np.concatenate([np.full(hi - lo, CLIQUE - 1 + x) for lo, hi, x in _ranges(groups)] + [q])
+    rp, m = _offsets(deg)
+    assert m == at == col.numel() == 2 ** 31 - 2
+    G = kd.kadabra_load_csr_device(CLIQUE + PENDANTS, rp, col)
+    yield G, col
+    G.free()
+    del col, rp
+    kd.kadabra_release_cached()
+    torch.cuda.empty_cache()
+
+
+def test_most_arcs_undirected(kd, largest):
+    """Loads; node 0 is adjacent to all others, so the bound is 2 * 1 + 1.
+    With the last arc changed, an id out of range, it is refused."""
+    G, col = largest
+    assert G.vd == 3
+    kept = int(col[-1])
+    try:
+        col[-1] = CLIQUE + PENDANTS
+        with pytest.raises(kd.KadabraError) as e:
+            kd.kadabra_load_csr_device(CLIQUE + PENDANTS, G._keepalive[0], col)
+        assert e.value.status == kd.ERR_CSR
+        col[-1] = JOINED  # a node whose row does not hold the last pendant
+        with pytest.raises(kd.KadabraError) as e:
+            kd.kadabra_load_csr_device(CLIQUE + PENDANTS, G._keepalive[0], col)
+        assert e.value.status == kd.ERR_CSR
+    finally:
+        col[-1] = kept
+
+
+@pytest.mark.parametrize("sink", [False, True])
+def test_most_arcs_directed(kd, sink):
+    """2^31 - 1 arcs: a clique of both arcs and, at the end of the forward
+    rows, 41 nodes with arcs into it, or, at the end of the reverse rows, one
+    node with 41,707 arcs from it (whose row makes the condensation's passes go
+    by arc).  Two components one behind the other, weighing 3 and 1."""
+    import torch
+    c = 46341
+    if sink:
+        q = np.array([2 ** 31 - 1 - c * (c - 1)])
+        groups = [(int(q[0]), 1), (c, 0)]
+    else:
+        q = np.concatenate([np.full(40, 1020), [2 ** 31 - 1 - c * (c - 1) - 40 * 1020]])
+        groups = [(int(q[-1]), 41), (1020, 40), (c, 0)]
+    n = c + len(q)
+    plain, _ = _clique_rows(c, [(c, 0)], int(q.sum()))  # the clique, then the other nodes' rows
+    at = c * (c - 1)
+    for k in q:
+        torch.arange(int(k), dtype=torch.int32, device="cuda", out=plain[at:at + int(k)])
+        at += int(k)
+    joined, at2 = _clique_rows(c, groups, 0)
+    rp_plain, m = _offsets(np.concatenate([np.full(c, c - 1), q]))
+    rp_joined, m2 = _offsets(np.concatenate([np.full(hi - lo, c - 1 + x) for lo, hi, x in _ranges(groups)] +
+                                            [np.zeros(len(q), np.int64)]))
+    assert m == m2 == at == at2 == 2 ** 31 - 1
+    fwd, rev = ((rp_joined, joined), (rp_plain, plain)) if sink else ((rp_plain, plain), (rp_joined, joined))
+    G = kd.kadabra_load_csr_device(n, *fwd, True, *rev)
+    try:
+        assert G.vd == 4
+    finally:
+        G.free()
+        kd.kadabra_release_cached()
+        del plain, joined, fwd, rev
+        torch.cuda.empty_cache()
