@@ -633,7 +633,7 @@ __device__ __forceinline__ int frontier_next(const int2* pr, int a, int cnt, int
 __device__ __forceinline__ int lower_bound_row(const int32_t* col, int a, int b, int32_t y) {
 #pragma unroll 1
   while (a < b) {
-    const int mid = (a + b) >> 1;
+    const int mid = a + ((b - a) >> 1);  // a + b may pass 2^31
     if (__ldg(&col[mid]) < y)
       a = mid + 1;
     else
@@ -686,7 +686,7 @@ __device__ __forceinline__ void lower_bound_rows2(const int32_t* col, int& a0, i
   }
 #pragma unroll 1
   while (a0 < b0 || a1 < b1) {  // at most two more rounds
-    const int m0 = (a0 + b0) >> 1, m1 = (a1 + b1) >> 1;
+    const int m0 = a0 + ((b0 - a0) >> 1), m1 = a1 + ((b1 - a1) >> 1);
     const bool w0 = a0 < b0, w1 = a1 < b1;
     const int32_t u = w0 ? __ldg(&col[m0]) : 0, v = w1 ? __ldg(&col[m1]) : 0;
     if (w0) {
@@ -723,8 +723,7 @@ __device__ __forceinline__ int warp_lower_bound(const int32_t* col, int a, int b
     a = na;
     b = nb;
   }
-  const int e = a + lane;
-  const bool less = e < b && __ldg(&col[e]) < y;
+  const bool less = lane < b - a && __ldg(&col[a + lane]) < y;
   const unsigned m = __ballot_sync(FULL, less);
   return a + __popc(m);
 }

@@ -180,3 +180,30 @@ def test_most_arcs_directed(kd, sink):
         kd.kadabra_release_cached()
         del plain, joined, fwd, rev
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("flags", ["", "LARGE_SHARED_TABLES", "MEDIUM_TABLES", "GLOBAL_TABLES"])
+def test_rows_beyond_2_30_arcs(kd, largest, flags):
+    """Samples whose rows lie up to 2^31 into the column array: distances,
+    path counts and paths follow from the construction."""
+    G, _ = largest
+    count = 4000 if not flags else 600
+    G.set_flags(getattr(kd, "FLAG_" + flags) if flags else 0)
+    try:
+        got = kd.kadabra_sample_paths(G, 1, 0, 0, count, max_len=4)
+    finally:
+        G.set_flags(0)
+    assert not got.status.any()
+    width = JOINED + (np.arange(PENDANTS) < LONGER)  # clique nodes a pendant is joined to: [0, width)
+    seen = set()
+    for (s, t), path, length, dist, sigma in zip(got.st, got.paths, got.path_len, got.stat("dist"),
+                                                 got.stat("sigma_lo")):
+        w = [int(width[x - CLIQUE]) if x >= CLIQUE else CLIQUE for x in (s, t)]
+        pend = (s >= CLIQUE) + (t >= CLIQUE)
+        common = min(w)
+        near = pend == 0 or (pend == 1 and min(s, t) < common)
+        assert (dist, sigma) == ((1, 1) if near else (2, common)), (s, t)
+        assert length == dist + 1 and path[0] == s and path[length - 1] == t
+        assert near or 0 <= path[1] < common
+        seen.add((int(pend), bool(near)))
+    assert {(0, True), (1, True), (1, False)} <= seen
