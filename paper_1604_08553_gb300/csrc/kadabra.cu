@@ -775,15 +775,26 @@ __device__ __forceinline__ int warp_slice(int E) {
   return max(1, (int)(((unsigned)E + 32u * NW - 1u) / (32u * NW))) * 32;
 }
 
-// Frontier positions p[k] of the tails of arcs wb + 32 k + lane (k < D; those
-// below c1 matter), given row pcur with its start <= wb < the next row's
-// start.  Each lane takes one of the next 32 rows and sets a bit where it
+// The warp's slice [c0, c1) of the level's E arcs.  (E may be close to 2^31:
+// no sum of arc indices beyond it is taken as an int, and the scans below
+// count down the arcs left instead of comparing ends.)
+template <int NW>
+__device__ __forceinline__ void take_slice(int E, int& c0, int& c1) {
+  const unsigned per = (unsigned)warp_slice<NW>(E);
+  const unsigned a = min((unsigned)E, (unsigned)warp_id() * per);
+  c0 = (int)a;
+  c1 = (int)min((unsigned)E, a + per);
+}
+
+// Frontier positions p[k] of the tails of arcs wb + 32 k + lane (k < D; the
+// next `rem` of them matter), given row pcur with its start <= wb < the next
+// row's start.  Each lane takes one of the next 32 rows and sets a bit where it
 // starts; a lane's row is pcur plus the bits up to its arc.  That is one
 // shared load and a few warp reductions instead of a binary search per lane.
 // Rows without arcs share a start, and more than 32 rows may start in the
 // step: then the lanes search.
 template <int D>
-__device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcount, int wb, int c1, int (&p)[D]) {
+__device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcount, int wb, int rem, int (&p)[D]) {
   const int lane = lane_id();
   const int q = pcur + 1 + lane;
   const int st = T.pr[KIDX(min(q, fcount), T.frcap + 1, 7)].x - wb;  // at least 1
@@ -806,8 +817,7 @@ __device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcou
   } else {
 #pragma unroll 1
     for (int k = 0; k < D; ++k) {
-      const int e = wb + 32 * k + lane;
-      const int f = e < c1 ? frontier_next(T.pr, pcur, fcount, e) : pcur;
+      const int f = 32 * k + lane < rem ? frontier_next(T.pr, pcur, fcount, wb + 32 * k + lane) : pcur;
 #pragma unroll
       for (int j = 0; j < D; ++j)
         if (j == k) p[j] = f;
@@ -833,34 +843,35 @@ __device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcou
 template <bool PK, int D, int NW, class EM>
 __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount, int E, const int32_t* cols,
                                            int64_t ncols, EM emit) {
-  const int lane = lane_id(), wid = warp_id();
-  const int per = warp_slice<NW>(E);
-  const int c0 = min(E, wid * per), c1 = min(E, c0 + per);
+  const int lane = lane_id();
+  int c0, c1;
+  take_slice<NW>(E, c0, c1);
   if (c0 >= c1) return;
   int pcur = frontier_pos(T.pr, fcount, c0);  // warp-uniform
   int2 cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];  // {first arc index, row start}
   int nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;  // first arc index of the next row
 #pragma unroll 1
-  for (int wb = c0; wb < c1; wb += 32 * D) {
+  for (int rem = c1 - c0; rem > 0; rem -= 32 * D) {
+    const int wb = c1 - rem;
     if (nxt <= wb) {  // the next arc lies in a later row
       pcur = frontier_next(T.pr, pcur + 1, fcount, wb);
       cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];
       nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;
     }
     int a[D];  // the arcs' places in the column array
-    if (nxt >= min(c1, wb + 32 * D)) {  // one row
+    if (nxt - wb >= min(rem, 32 * D)) {  // one row
 #pragma unroll
       for (int k = 0; k < D; ++k) a[k] = cur.y + (wb - cur.x) + lane + 32 * k;
     } else {
       int p[D];
-      rows_of_step<D>(T, pcur, fcount, wb, c1, p);
+      rows_of_step<D>(T, pcur, fcount, wb, rem, p);
 #pragma unroll
       for (int k = 0; k < D; ++k) {
         const int2 q = T.pr[KIDX(p[k], T.frcap + 1, 7)];
         a[k] = q.y + (wb + 32 * k + lane - q.x);
       }
     }
-    const int left = c1 - wb - lane;  // the lane's arc k exists if left > 32 k
+    const int left = rem - lane;  // the lane's arc k exists if left > 32 k
     int y[D];
 #pragma unroll
     for (int k = 0; k < D; ++k)
@@ -908,18 +919,19 @@ __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount
 template <int NW, class F>
 __device__ __forceinline__ void scan_level(const Tables& T, int fcount, int E, const int32_t* cols, int64_t ncols,
                                            F f) {
-  const int lane = lane_id(), wid = warp_id();
-  const int per = warp_slice<NW>(E);
-  const int c0 = min(E, wid * per), c1 = min(E, c0 + per);
+  const int lane = lane_id();
+  int c0, c1;
+  take_slice<NW>(E, c0, c1);
   if (c0 >= c1) return;
   int pcur = frontier_pos(T.pr, fcount, c0);  // warp-uniform
   int2 cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];  // {first arc index, row start}
   int nxt = T.pr[KIDX(pcur + 1, T.frcap + 1, 7)].x;  // first arc index of the next row
-  // the window at wb: its lanes' frontier positions and heads (loads issued)
-  auto fetch = [&](int wb, bool& ok, int& p, int& y) {
+  // the window of the last `rem` arcs: its lanes' frontier positions and heads (loads issued)
+  auto fetch = [&](int rem, bool& ok, int& p, int& y) {
     ok = false;
     p = y = 0;
-    if (wb >= c1) return;
+    if (rem <= 0) return;
+    const int wb = c1 - rem;
     if (nxt <= wb) {  // the window starts in a later row
       pcur = frontier_next(T.pr, pcur + 1, fcount, wb);
       cur = T.pr[KIDX(pcur, T.frcap + 1, 7)];
@@ -927,22 +939,21 @@ __device__ __forceinline__ void scan_level(const Tables& T, int fcount, int E, c
     }
     int2 q = cur;
     p = pcur;
-    if (nxt < min(c1, wb + 32)) {
+    if (nxt - wb < min(rem, 32)) {
       int pk[1];
-      rows_of_step<1>(T, pcur, fcount, wb, c1, pk);
+      rows_of_step<1>(T, pcur, fcount, wb, rem, pk);
       p = pk[0];
       q = T.pr[KIDX(p, T.frcap + 1, 7)];
     }
-    const int e = wb + lane;
-    ok = e < c1;
-    if (ok) y = __ldg(&cols[KIDX((int64_t)q.y + (e - q.x), ncols, 8)]);
+    ok = lane < rem;
+    if (ok) y = __ldg(&cols[KIDX((int64_t)q.y + (wb - q.x) + lane, ncols, 8)]);
   };
   bool ok0 = false, ok1;
   int p0 = 0, p1, y0 = 0, y1;
 #pragma unroll 1
-  for (int wb = c0 - 32; wb < c1; wb += 32) {  // the first round only fetches
-    fetch(wb + 32, ok1, p1, y1);
-    if (wb >= c0) f(ok0, p0, y0);
+  for (int rem = c1 - c0 + 32; rem > 0; rem -= 32) {  // the first round only fetches
+    fetch(rem - 32, ok1, p1, y1);
+    if (rem <= c1 - c0) f(ok0, p0, y0);
     ok0 = ok1;
     p0 = p1;
     y0 = y1;
@@ -2514,8 +2525,8 @@ __device__ int run_sample_warp(const SampleParams& P, const Job& J, WSlot& S, ui
     n_edges += E;
     // pass 1: touch test against the other search
     npi = 0;
-    for (int base = 0; base < E; base += 32) {
-      const int e = base + lane;
+    for (int rem = E; rem > 0; rem -= 32) {
+      const int e = lane < rem ? E - rem + lane : E;
       bool touch = false;
       int x = 0, y = 0;
       unsigned long long wgt = 0;
@@ -2553,8 +2564,8 @@ __device__ int run_sample_warp(const SampleParams& P, const Job& J, WSlot& S, ui
     const int list_before = nlist;
     long long fresh = 0, hits = 0, cost = 0;
     bool cap = false;
-    for (int base = 0; base < E && !cap; base += 32) {
-      const int e = base + lane;
+    for (int rem = E; rem > 0 && !cap; rem -= 32) {
+      const int e = lane < rem ? E - rem + lane : E;
       bool ins = false, bad = false;
       uint32_t ipos = 0;
       int yy = 0, ydeg = 0;
