@@ -3516,15 +3516,16 @@ __device__ __forceinline__ int32_t warp_row_of_arc(const int32_t* rp, int32_t n,
 // ok[k] = there is one), with all lanes of the warp.  The lanes' rows come
 // from the starts of the next rows, 32 at a time, counted by a search over
 // the lanes' registers (several rounds only where rows are so short, or
-// empty, that more than 32 start in a window).  Window ends are cut to the
-// chunk's arcs, below 2^31 - 1, the start that stands for "no more rows".
+// empty, that more than 32 start in a window).  Starts count from the step's
+// first arc, since a window's end may lie behind arc 2^31 - 1, the largest
+// start and the one that stands for "no more rows".
 template <int D, class F>
 __device__ __forceinline__ void for_each_arc(const int32_t* rp, const int32_t* ci, int32_t n, int64_t m, F f) {
   const int lane = lane_id();
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  if (m <= 0) return;  // no chunk
   // a graph with less than ARC_CHUNK arcs per warp is spread over all of them
-  // (at least one window each, so a graph without arcs has no chunk)
-  const int64_t per = max((m + nwarps - 1) / nwarps, (int64_t)1);
+  const int64_t per = (m + nwarps - 1) / nwarps;
   const int64_t chunk = per < ARC_CHUNK ? (per + 31) / 32 * 32 : ARC_CHUNK;
   const int64_t chunks = (m + chunk - 1) / chunk;
   for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < chunks; c += nwarps) {
@@ -3542,13 +3543,12 @@ __device__ __forceinline__ void for_each_arc(const int32_t* rp, const int32_t* c
       }
 #pragma unroll
       for (int k = 0; k < D; ++k) {
-        const int32_t last = (int32_t)min(base + 32 * k + 31, e1 - 1);
-        const int32_t at = (int32_t)min(e[k], (int64_t)last);
+        const int32_t at = 32 * k + lane, last = 32 * k + 31;
         u[k] = row;
         for (int32_t r = row;; r += 32) {
-          const int32_t st = r + 1 + lane < n ? __ldg(&rp[r + 1 + lane]) : 0x7FFFFFFF;  // above every arc's index
+          const int32_t st = r + 1 + lane < n ? __ldg(&rp[r + 1 + lane]) - (int32_t)base : 0x7FFFFFFF;
           if (!__any_sync(FULL, st <= last)) break;
-          int q = 0;  // how many of the 32 rows start at the lane's arc or before
+          int q = 0;  // how many of the 32 rows start at e or before
 #pragma unroll
           for (int h = 16; h > 0; h >>= 1)
             if (__shfl_sync(FULL, st, q + h - 1) <= at) q += h;
