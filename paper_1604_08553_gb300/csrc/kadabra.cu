@@ -1593,6 +1593,13 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
       const int lf = (of ? LF_SIGMA : 0) | (cap ? LF_CAP : 0) | (sigma_of ? LF_TOUCH_SIGMA : 0);
       if (lf) atomicOr(&c.lvl_flags, lf);
       __syncthreads();
+      if (PK && (c.lvl_flags & LF_CAP)) {
+        // A packed sigma that ran out of its bits has carried into its entry's
+        // depth and side, so a one-pass level's touches may be false: the next
+        // tier takes the sample, touch or not.
+        if (tid == 0) c.flags |= F_CAP;
+        return;
+      }
       if (fused && c.npi > 0) {
         // the level touches: undo its insertions (slots that were empty
         // before it) and choose among its touch arcs, as after pass 1
