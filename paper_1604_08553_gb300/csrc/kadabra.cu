@@ -215,6 +215,7 @@ __device__ __forceinline__ uint64_t below128(uint4 b, uint64_t S) {
 // check records (site << 40 | index) in g_checked once, redirects the access
 // to index 0 (so nothing outside the arrays is touched), and the sample then
 // fails with KADABRA_ERR_INTERNAL, whose message names the site and index.
+// It also delays warps where several work at once between two barriers.
 // Without the flag the checks compile to nothing.
 #ifdef KADABRA_CHECKED
 __device__ unsigned long long g_checked;
@@ -224,8 +225,15 @@ __device__ __forceinline__ int64_t kchk(int64_t i, int64_t bound, int site) {
   return 0;
 }
 #define KIDX(i, bound, site) ((std::decay_t<decltype(i)>)kchk((int64_t)(i), (int64_t)(bound), (site)))
+// holds the warps for which `late` is true back by some microseconds, so that
+// a value they read without a barrier is seen to change under them
+#define KSTAGGER(late)             \
+  do {                             \
+    if (late) __nanosleep(20000u); \
+  } while (0)
 #else
 #define KIDX(i, bound, site) (i)
+#define KSTAGGER(late)
 #endif
 
 // ============================================================== tables
@@ -525,6 +533,7 @@ struct Ctl {
   uint4 draws[32];  // the sample's Philox blocks j = 0..31, drawn by warp 0 at its start
   int pick;
   int mode;       // backtracking: 0 = scan the row of x, 1 = scan the previous level
+  int cand[2];               // the chosen candidate edge: v on the s side, w on the t side
   int bt_x[2], bt_dx[2];     // backtracking walkers (0: v -> s, 1: w -> t): node, depth
   uint32_t bt_j[2];          //   and the next Philox block of each
   unsigned long long cur, k;  // the launch's running index, the sample's work index
@@ -1688,8 +1697,8 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
         const unsigned long long r = below128(c.draws[1], all);
         if (i < total && (tid & ((1 << sl) - 1)) == 0 && below <= r && r - below < mw) {
           c.pick = i;
-          c.bt_x[0] = side == 0 ? me.x : me.y;
-          c.bt_x[1] = side == 0 ? me.y : me.x;
+          c.cand[0] = c.bt_x[0] = side == 0 ? me.x : me.y;
+          c.cand[1] = c.bt_x[1] = side == 0 ? me.y : me.x;
           c.stat[KADABRA_STAT_SIGMA_LO] = (long long)(all & 0xFFFFFFFFull);
           c.stat[KADABRA_STAT_SIGMA_HI] = (long long)(all >> 32);
         }
@@ -1744,8 +1753,8 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
         c.pick = pick;
         if (pick >= 0) {
           const PiEntry e = T.pi[pick];
-          c.bt_x[0] = side == 0 ? e.x : e.y;
-          c.bt_x[1] = side == 0 ? e.y : e.x;
+          c.cand[0] = c.bt_x[0] = side == 0 ? e.x : e.y;
+          c.cand[1] = c.bt_x[1] = side == 0 ? e.y : e.x;
         }
       }
     }
@@ -1760,8 +1769,9 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
   // The candidate edge joins the two current frontiers, so v is at depth0
   // on the s side and w at depth1 on the t side.
   const bool want_path = P.paths != nullptr && out_i >= 0;
-  if (tid == NT - 1) {  // a warp that does not walk
-    const int cv = c.bt_x[0], cw = c.bt_x[1];
+  KSTAGGER(wid >= 2);
+  if (tid == NT - 1) {  // a warp that does not walk; the walkers change bt_x meanwhile
+    const int cv = c.cand[0], cw = c.cand[1];
     c.stat[KADABRA_STAT_DIST] = dv + 1 + dw;
     c.stat[KADABRA_STAT_PATH_NODES] = dv + dw + 2;
     if (want_path) {
