@@ -3804,8 +3804,34 @@ __global__ void k_bfs_root(const unsigned long long* best, int32_t* dist, int32_
 constexpr int BFS_CHUNK = 1024;
 
 struct BfsItem {
-  int32_t v, begin, end, pad;
+  int32_t v, begin, end;
+  int32_t look;  // bottom-up: 1, the arcs are searched for a node at the current level
 };
+
+// cuts arcs [a, b) of v's row, more than one chunk, into items (one warp);
+// returns the first arc that found no room, or b
+__device__ __forceinline__ int32_t bfs_cut(int32_t v, int32_t a, int32_t b, int32_t look, BfsItem* items,
+                                           int32_t* nitems, int32_t items_cap) {
+  const int lane = lane_id();
+  const int32_t k = (b - a + BFS_CHUNK - 1) / BFS_CHUNK;  // items of this row
+  int32_t at = 0;
+  if (lane == 0) at = atomicAdd(nitems, k);
+  at = __shfl_sync(FULL, at, 0);
+  for (int32_t q = lane; q < k; q += 32) {
+    if (at + q < items_cap) {
+      const int32_t s = a + q * BFS_CHUNK;
+      items[at + q] = BfsItem{v, s, b - s > BFS_CHUNK ? s + BFS_CHUNK : b, look};
+    }
+  }
+  return at + k > items_cap ? a + (items_cap > at ? items_cap - at : 0) * BFS_CHUNK : b;
+}
+
+// one of arcs [a, b) of row c is a node at `level` (one warp)
+__device__ __forceinline__ bool bfs_look(const int32_t* c, int64_t a, int32_t b, const int32_t* dist, int32_t level) {
+  for (; a < b; a += 32)
+    if (__any_sync(FULL, a + lane_id() < b && dist[c[a + lane_id()]] == level)) return true;
+  return false;
+}
 
 // scans arcs [a, b) of row c and appends the newly reached heads to next;
 // arcs: their rows' arcs, of this lane's heads
@@ -3867,14 +3893,19 @@ __device__ __forceinline__ void warp_append_groups(uint32_t bits, int groups, in
 // than m / BFS_BOTTOM_UP_ARCS arcs, is expanded bottom-up (Beamer et al.'s
 // direction-optimising BFS): every unvisited node looks in its row of the
 // opposite CSR (br, bc) for a node at the current level and stops at the
-// first, after m / (frontier arcs) looks or so.  Either direction yields the
-// same next level.  The arcs count for themselves: the neighbours of a
+// first, after m / (frontier arcs) looks or so.  A lane looks at BFS_LOOK arcs
+// of its node's row; the rest of a longer row, one the level may not reach at
+// all, goes to the whole warp, and beyond a chunk to k_bfs_items (an
+// undirected graph of 4.4 M nodes with a hub of 100,000 arcs out of reach on
+// two levels: load 18.98 -> 0.54 ms).  Either direction yields the same
+// next level.  The arcs count for themselves: the neighbours of a
 // power-law graph's largest hub are few, but hold most arcs (both BFS of
 // R-MAT scale 24: 6.7 -> 4.0 ms).  Whole loads with m, m/16, m/32 and m/64:
 // R-MAT scale 20 3.03, 2.17, 2.17, 2.17 ms, Chung-Lu of 10^6 nodes 0.82, 0.73,
 // 0.74, 0.74 ms, BA of 300,000 nodes 0.58, 0.59, 0.51, 0.51 ms.
 constexpr int BFS_BOTTOM_UP = 16;
 constexpr int BFS_BOTTOM_UP_ARCS = 32;
+constexpr int BFS_LOOK = 64;
 
 __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t* br, const int32_t* bc,
                             const int32_t* front, const int32_t* nfront_dev, int32_t* next, int32_t* nnext,
@@ -3893,17 +3924,24 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
       for (int q = 0; q < groups; ++q) {
         const int64_t v = base + 32 * q + lane;
         bool mine = false;
+        int32_t a = 0, b = 0;  // what is left of the row
         if (v < n && dist[v] < 0) {
-          for (int32_t e = br[v]; e < br[v + 1]; ++e)
-            if (dist[bc[e]] == level) {
-              mine = true;
-              break;
-            }
-          if (mine) {
-            dist[v] = level + 1;  // only this thread writes v's entry
-            own += tr[v + 1] - tr[v];
-            bits |= 1u << q;
-          }
+          a = br[v];
+          b = br[v + 1];
+          const int32_t stop = b - a > BFS_LOOK ? a + BFS_LOOK : b;
+          for (; a < stop && !mine; ++a) mine = dist[bc[a]] == level;
+        }
+        for (unsigned rows = __ballot_sync(FULL, !mine && a < b); rows; rows &= rows - 1) {
+          const int j = __ffs(rows) - 1;
+          int32_t aj = __shfl_sync(FULL, a, j);
+          const int32_t bj = __shfl_sync(FULL, b, j);
+          if (bj - aj > BFS_CHUNK) aj = bfs_cut((int32_t)(v - lane + j), aj, bj, 1, items, nitems, items_cap);
+          if (bfs_look(bc, aj, bj, dist, level) && lane == j) mine = true;
+        }
+        if (mine) {
+          dist[v] = level + 1;  // only this thread writes v's entry in this launch
+          own += tr[v + 1] - tr[v];
+          bits |= 1u << q;
         }
       }
       warp_append_groups(bits, groups, base, next, nnext);
@@ -3921,31 +3959,29 @@ __global__ void k_bfs_level(const int32_t* tr, const int32_t* tc, const int32_t*
       bfs_scan(tr, tc, a, b, next, nnext, dist, level, own);
       continue;
     }
-    const int32_t k = (b - a + BFS_CHUNK - 1) / BFS_CHUNK;  // items of this row
-    int32_t at = 0;
-    if (lane == 0) at = atomicAdd(nitems, k);
-    at = __shfl_sync(FULL, at, 0);
-    for (int32_t q = lane; q < k; q += 32) {
-      if (at + q < items_cap) {
-        const int32_t s = a + q * BFS_CHUNK;
-        items[at + q] = BfsItem{v, s, b - s > BFS_CHUNK ? s + BFS_CHUNK : b, 0};
-      }
-    }
-    if (at + k > items_cap) bfs_scan(tr, tc, a + (items_cap > at ? items_cap - at : 0) * BFS_CHUNK, b, next, nnext,
-                                     dist, level, own);  // items beyond the buffer: this warp scans them
+    // items beyond the buffer: this warp scans them
+    bfs_scan(tr, tc, bfs_cut(v, a, b, 0, items, nitems, items_cap), b, next, nnext, dist, level, own);
   }
   bfs_add_arcs(own, nnext);
 }
 
-__global__ void k_bfs_items(const int32_t* tr, const int32_t* tc, const BfsItem* items, const int32_t* nitems, int32_t items_cap,
-                            int32_t* next, int32_t* nnext, int32_t* dist, int32_t level) {
+__global__ void k_bfs_items(const int32_t* tr, const int32_t* tc, const int32_t* bc, const BfsItem* items,
+                            const int32_t* nitems, int32_t items_cap, int32_t* next, int32_t* nnext, int32_t* dist,
+                            int32_t level) {
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int32_t k = *nitems < items_cap ? *nitems : items_cap;
   int32_t own = 0;
   for (int64_t i = w0; i < k; i += nwarps) {
     const BfsItem it = items[i];
-    bfs_scan(tr, tc, it.begin, it.end, next, nnext, dist, level, own);
+    if (!it.look) {
+      bfs_scan(tr, tc, it.begin, it.end, next, nnext, dist, level, own);
+    } else if (__shfl_sync(FULL, *(volatile const int32_t*)&dist[it.v], 0) < 0 &&
+               bfs_look(bc, it.begin, it.end, dist, level) && lane_id() == 0 &&
+               atomicCAS(&dist[it.v], -1, level + 1) == -1) {  // not found by another of the row's items
+      next[atomicAdd(nnext, 1)] = it.v;
+      own += tr[it.v + 1] - tr[it.v];
+    }
   }
   bfs_add_arcs(own, nnext);
 }
@@ -5132,7 +5168,7 @@ kadabra_status vd_bfs(kadabra_graph* g, const LoadScratch& S, const int32_t* tr,
       const int32_t* prev = l == 0 ? nullptr : S.cnt + SLOT * ((l + SLOTS - 1) % SLOTS);
       k_bfs_level<<<8 * g->num_sms, 256>>>(tr, tc, br, bc, in_q, prev, out_q, c, dist, l, S.items, c + 1,
                                            S.items_cap, n, g->m);
-      k_bfs_items<<<8 * g->num_sms, 256>>>(tr, tc, S.items, c + 1, S.items_cap, out_q, c, dist, l);
+      k_bfs_items<<<8 * g->num_sms, 256>>>(tr, tc, bc, S.items, c + 1, S.items_cap, out_q, c, dist, l);
     }
     int32_t h[SLOT * SLOTS];
     if (cudaMemcpy(h, S.cnt, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess)
