@@ -433,7 +433,7 @@ struct SampleParams {
   Job job0;                         // the job, when the launch has only one
   const Job* jobs;                  // device array of njobs jobs, or null (then job0)
   int njobs;
-  uint64_t total_work;              // sum of the jobs' counts (with total_dev: what decides on k_screen)
+  uint64_t total_work;              // sum of the jobs' counts
   const unsigned long long* total_dev;  // if set: the sum, read from device memory at launch
   unsigned long long* ctr;          // queue counters, Q_*
   unsigned long long* qb;           // sample indices queued for tier B
@@ -4569,7 +4569,7 @@ struct kadabra_graph {
   int directed = 0;
   int32_t *rp = nullptr, *ci = nullptr, *rrp = nullptr, *rci = nullptr;
   int64_t vd = 0;
-  bool screened = false;       // enough samples end at a root without arcs: k_screen runs first
+  double idle = 0.0;           // share of the samples that end at a root without arcs
   bool csr_beyond_l2 = false;  // forward (+ reverse) CSR larger than the L2: long rows are searched
   int device = 0;
   int num_sms = 0;
@@ -4604,23 +4604,29 @@ namespace {
 // internal launch flag: the graph's CSR exceeds the L2, so pass 1 searches
 // its long rows (KADABRA_FLAG_ASYNC_SCAN asks for that explicitly)
 constexpr uint32_t FLAG_VEC_AUTO = 1u << 31;
-// internal launch flag: k_screen before tier S, for graphs on which at least
-// SCREEN_MIN of the samples end at a root without arcs, in launches of at
-// least SCREEN_SAMPLES samples.  It costs a launch (3 to 5 us); 1,000, 8,192,
-// 16,384 and 65,536 samples, without and with it: 109 and 114 us (R-MAT scale
-// 17), 445 and 436 (scale 20), 249 and 238 (scale 17), 1,092 and 996 (scale 20).
-constexpr uint32_t FLAG_SCREEN_AUTO = 1u << 30;
-constexpr double SCREEN_MIN = 0.25;
-constexpr uint64_t SCREEN_SAMPLES = 8192;
 // internal launch flag: no graph of the launch has more than TINY_NODES nodes
 constexpr uint32_t FLAG_TINY_AUTO = 1u << 29;
 // the flags a launch shared by several graphs takes from any of them (they
 // change no result; the tier-skipping flags stay per graph)
-constexpr uint32_t SHARED_LAUNCH_FLAGS = KADABRA_FLAG_WARP_TIER | KADABRA_FLAG_ASYNC_SCAN | FLAG_VEC_AUTO | FLAG_SCREEN_AUTO;
+constexpr uint32_t SHARED_LAUNCH_FLAGS = KADABRA_FLAG_WARP_TIER | KADABRA_FLAG_ASYNC_SCAN | FLAG_VEC_AUTO;
 
 uint32_t launch_flags(const kadabra_graph* g) {
-  return g->flags | (g->csr_beyond_l2 ? FLAG_VEC_AUTO : 0u) | (g->screened ? FLAG_SCREEN_AUTO : 0u) |
-         (g->n <= TINY_NODES ? FLAG_TINY_AUTO : 0u);
+  return g->flags | (g->csr_beyond_l2 ? FLAG_VEC_AUTO : 0u) | (g->n <= TINY_NODES ? FLAG_TINY_AUTO : 0u);
+}
+
+// k_screen before tier S, in launches of at least SCREEN_SAMPLES samples at
+// least SCREEN_MIN of which are expected to end at a root without arcs (over
+// all graphs of the launch).  It costs a launch (3 to 5 us) and a second draw
+// of the others; without and with it, in us: 1,000 samples 109 and 114 (R-MAT
+// scale 17); 8,192 445 and 436 (scale 20); 16,384 249 and 238 (scale 17);
+// 65,536 1,092 and 996 (scale 20).  With a quarter of the samples idle, random
+// directed graphs of mean degree 2, 8 and 16: 8,192 samples 773 and 766, 404
+// and 408, 206 and 207; 65,536 4,738 and 4,697, 2,751 and 2,700, 1,369 and
+// 1,325.
+constexpr double SCREEN_MIN = 0.25;
+constexpr uint64_t SCREEN_SAMPLES = 8192;
+void choose_screen(SampleParams& P, uint64_t samples, double idle_samples) {
+  if (samples >= SCREEN_SAMPLES && idle_samples >= SCREEN_MIN * (double)samples) P.tier_flags |= TF_SCREEN;
 }
 }  // namespace
 
@@ -4854,7 +4860,6 @@ SampleParams ws_params(const Workspace* w, uint32_t flags) {
   if (flags & (KADABRA_FLAG_ASYNC_SCAN | FLAG_VEC_AUTO)) P.tier_flags |= TF_VEC;
   if (flags & KADABRA_FLAG_FRONTIER_SEGMENTS) P.tier_flags |= TF_SEG64;
   if (flags & KADABRA_FLAG_COMPACT_TABLES) P.tier_flags |= TF_COMPACT;
-  if (flags & FLAG_SCREEN_AUTO) P.tier_flags |= TF_SCREEN;
   if (flags & FLAG_TINY_AUTO) P.tier_flags |= TF_TINY;
   return P;
 }
@@ -4879,7 +4884,7 @@ kadabra_status launch_sampler_kernels(Workspace* w, SampleParams P, cudaStream_t
     P.q0 = w->qs;  // tier W's overflow queue, tier S's input
     k_sample_warp<<<w->grid_warp, 32 * WT_WARPS, w->smem_warp, st>>>(P);
     KCK(cudaGetLastError());
-  } else if ((P.tier_flags & TF_SCREEN) && !(P.tier_flags & TF_SKIP_S) && P.total_work >= SCREEN_SAMPLES) {
+  } else if ((P.tier_flags & TF_SCREEN) && !(P.tier_flags & TF_SKIP_S)) {
     P.q0 = w->qs;
     k_screen<<<2 * w->num_sms, 256, 0, st>>>(P);
     KCK(cudaGetLastError());
@@ -5311,8 +5316,7 @@ kadabra_status compute_vd(kadabra_graph* g, LoadTrace& tr, const LoadScratch& S)
   if (cudaMemcpy(&core, S.core, sizeof(core), cudaMemcpyDeviceToHost) != cudaSuccess)
     return fail(KADABRA_ERR_CUDA, std::string("vd: ") + cudaGetErrorString(cudaGetLastError()));
   tr.mark("vd bfs");
-  const double idle = 1.0 - (1.0 - (double)core.idle[0] / n) * (1.0 - (double)core.idle[1] / n);
-  g->screened = idle >= SCREEN_MIN;
+  g->idle = 1.0 - (1.0 - (double)core.idle[0] / n) * (1.0 - (double)core.idle[1] / n);
   const long long root_w = (long long)core.e_out + core.e_in + 1;
   if (core.size == (unsigned long long)n) {
     g->vd = root_w;
@@ -5549,6 +5553,7 @@ kadabra_status tier_variant(kadabra_graph* g, Workspace* w, cudaStream_t st, int
   KTRY(ensure_ws(w, probe, 1));
   SampleParams P = ws_params(w, launch_flags(g));
   P.total_work = probe;
+  choose_screen(P, probe, g->idle * probe);
   std::memset(&P.job0, 0, sizeof(Job));
   P.job0.g = graph_dev(g);
   P.job0.seed = 0x5EEDu;
@@ -5686,13 +5691,19 @@ kadabra_status run_loop_graph(LoopCache& L, Workspace* w, cudaStream_t st, std::
   P.jobs = d_job;
   P.njobs = G;
   P.total_dev = &d_state->total_work;
-  // The launches read total_dev; the sum only decides whether k_screen runs.
-  // No more than that decision goes into the parameters, so that a run with
-  // another K (another lambda, if the library chooses K) finds the CUDA graph
-  // as it is: building it anew took 65 to 70 us of a 1.0 ms run on 2,000 nodes.
+  // The launches read total_dev; a round's samples only decide whether k_screen
+  // runs.  No more than that decision goes into the parameters, so that a run
+  // with another K (another lambda, if the library chooses K) finds the CUDA
+  // graph as it is: building it anew took 65 to 70 us of a 1.0 ms run on 2,000
+  // nodes.
   uint64_t round = 0;
-  for (const LoopRun& r : R) round += r.K;
-  P.total_work = round >= SCREEN_SAMPLES ? SCREEN_SAMPLES : 0;
+  double idle = 0.0;
+  for (const LoopRun& r : R) {
+    if (r.done) continue;
+    round += r.K;
+    idle += r.g->idle * (double)r.K;
+  }
+  choose_screen(P, round, idle);
   int64_t max_n = 1;
   for (const LoopRun& r : R) max_n = std::max<int64_t>(max_n, r.g->n);
   const int64_t want = (4 * (int64_t)w->num_sms + G - 1) / G;
@@ -5844,6 +5855,7 @@ kadabra_status run_graphs(Workspace* w, kadabra_graph* const* gs, int G, const d
     fl = FLAG_TINY_AUTO;
     for (int i = 0; i < G; ++i) fl &= launch_flags(gs[i]);
     for (int i = 0; i < G; ++i) fl |= launch_flags(gs[i]) & SHARED_LAUNCH_FLAGS;
+  double idle = 0.0;  // of the jobs' samples: expected to end at a root without arcs
   auto launch_jobs = [&]() -> kadabra_status {
     uint64_t work = 0;
     for (Job& j : jobs) {
@@ -5853,6 +5865,8 @@ kadabra_status run_graphs(Workspace* w, kadabra_graph* const* gs, int G, const d
     if (work == 0) return KADABRA_OK;
     SampleParams P = ws_params(w, fl);
     P.total_work = work;
+    choose_screen(P, work, idle);
+    idle = 0.0;
     if (jobs.size() == 1) {
       P.job0 = jobs[0];
     } else {
@@ -5873,6 +5887,7 @@ kadabra_status run_graphs(Workspace* w, kadabra_graph* const* gs, int G, const d
     j.count = count;
     j.counts = counts;
     j.totals = s.g->totals;
+    idle += s.g->idle * (double)count;
     return j;
   };
   // Warm-up of every graph in one launch (Alg. 2 lines 1-5).  The same
@@ -6288,6 +6303,7 @@ kadabra_status run_topk(kadabra_graph* g, double lambda, double delta, int32_t k
     RCK(cudaMemcpyAsync(w->d_jobs, jobs, sizeof(jobs), cudaMemcpyHostToDevice, st));
     SampleParams P = ws_params(w, launch_flags(g));
     P.total_work = 2 * alpha + B0;
+    choose_screen(P, P.total_work, g->idle * (double)P.total_work);
     P.jobs = w->d_jobs;
     P.njobs = 3;
     tr.mark("setup, tuning");
@@ -6413,6 +6429,7 @@ kadabra_status run_topk(kadabra_graph* g, double lambda, double delta, int32_t k
     if (tau > 0) {  // the first batch came with the warm-up
       SampleParams P = ws_params(w, launch_flags(g));
       P.total_work = B;
+      choose_screen(P, B, g->idle * (double)B);
       P.job0 = job(0, tau, B, g->counts);
       KTRY(launch_sampler(w, P, st, variant));
       tr.mark("main batch");
@@ -6851,22 +6868,27 @@ kadabra_status srv_round(kadabra_server* S, std::vector<SrvJob*>& act, std::vect
   for (SrvJob* J : act) nrun += (J->phase == 1 || J->phase == 2) ? 1 : 0;
   const uint64_t quota = std::max<uint64_t>(SRV_MIN_CHUNK, SRV_ROUND_SAMPLES / std::max<uint64_t>(nrun, 1));
   std::vector<SrvJob*> first;  // new jobs whose first main-loop chunk rides with their warm-up
+  double idle = 0.0;           // of the jobs' samples: expected to end at a root without arcs
+  auto add = [&](SrvJob* J, const Job& j) {
+    jobs.push_back(j);
+    idle += J->g->idle * (double)j.count;
+  };
   for (SrvJob* J : act) {
     if (J->phase == 1) {
-      if (J->k > 0) jobs.push_back(srv_job(J, 2, 0, J->alpha, J->count_pre));
-      jobs.push_back(srv_job(J, 1, 0, J->alpha, J->count0));
+      if (J->k > 0) add(J, srv_job(J, 2, 0, J->alpha, J->count_pre));
+      add(J, srv_job(J, 1, 0, J->alpha, J->count0));
       warm.push_back(J);
       // main-loop samples do not depend on computeDelta: the first batch (or
       // its first chunk) goes into the same launch
       J->B = std::min<uint64_t>(J->K, J->cap - J->tau);
       J->taken = 0;
       J->chunk = std::min<uint64_t>(J->B, quota);
-      jobs.push_back(srv_job(J, 0, J->tau, J->chunk, J->counts));
+      add(J, srv_job(J, 0, J->tau, J->chunk, J->counts));
       first.push_back(J);
     } else if (J->phase == 2) {
       if (J->taken == 0) J->B = std::min<uint64_t>(J->K, J->cap - J->tau);  // the next batch
       J->chunk = std::min<uint64_t>(J->B - J->taken, quota);
-      jobs.push_back(srv_job(J, 0, J->tau + J->taken, J->chunk, J->counts));
+      add(J, srv_job(J, 0, J->tau + J->taken, J->chunk, J->counts));
       main_j.push_back(J);
     }
   }
@@ -6882,6 +6904,7 @@ kadabra_status srv_round(kadabra_server* S, std::vector<SrvJob*>& act, std::vect
   for (SrvJob* J : act) fl |= launch_flags(J->g) & SHARED_LAUNCH_FLAGS;
   SampleParams P = ws_params(w, fl);
   P.total_work = work;
+  choose_screen(P, work, idle);
   if (jobs.size() == 1) {
     P.job0 = jobs[0];
   } else {
@@ -7434,6 +7457,7 @@ kadabra_status kadabra_sample_batch(kadabra_graph* g, uint64_t seed, uint32_t do
   P.job0.counts = d_counts;
   P.job0.totals = reinterpret_cast<long long*>(d_totals);
   P.total_work = count;
+  choose_screen(P, count, g->idle * (double)count);
   return launch_sampler(g->ws, P, as_stream(stream), tuned_variant(g, count));
 }
 
@@ -7543,6 +7567,7 @@ kadabra_status kadabra_sample_paths(kadabra_graph* g, uint64_t seed, uint32_t do
   P.job0.first_idx = first_idx;
   P.job0.count = count;
   P.total_work = count;
+  choose_screen(P, count, g->idle * (double)count);
   P.st_out = d_st;
   P.path_len = d_pl;
   P.paths = d_paths;

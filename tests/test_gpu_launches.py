@@ -50,3 +50,38 @@ print(json.dumps([count(lambda: run(0.01, 1000), *names), count(lambda: run(0.01
 """)
     assert first == [1, 1] and same == [0, 1]
     assert other == [0, 1] and chosen == [0, 1]
+
+
+def test_screening_goes_by_the_launch_s_samples():
+    """The screening kernel runs where a quarter of a launch's samples are
+    expected to end at a root without arcs: not in a batch or among served
+    jobs because one graph of many is of that kind."""
+    alone, few, mixed, most, served, served_mixed = _child("""
+rmat = [gg.rmat(12, 8, 0.57, 0.19, 0.19, s) for s in (3, 4, 5)]
+ba = [gg.barabasi_albert(20000, 5, s) for s in range(7)]
+names = ("k_screen", "k_sample<2")
+def batch(graphs, K):
+    B = kd.Batch(graphs)
+    run = lambda: B.run([0.01] * len(graphs), [0.1] * len(graphs), [1] * len(graphs), check_interval=K)
+    run()
+    c = count(run, *names)
+    B.free()
+    return c
+def serve(graphs):
+    G = [kd.kadabra_load_csr(g) for g in graphs]
+    def run():
+        ids = [kd.kadabra_submit(g, 0.01, 0.1, 0, 1, check_interval=16384) for g in G]
+        for i, g in zip(ids, G):
+            kd.kadabra_poll(i, g.n)
+    run()
+    c = count(run, *names)
+    kd.kadabra_serve_shutdown()
+    for g in G:
+        g.free()
+    return c
+print(json.dumps([batch(rmat, 16384), batch(rmat[:1], 1000), batch(rmat[:1] + ba, 8192), batch(rmat + ba[:1], 8192),
+                  serve(rmat), serve(rmat[:1] + ba)]))
+""")
+    assert alone[0] > 0 and most[0] > 0 and served[0] > 0
+    assert few[0] == 0 and mixed[0] == 0
+    assert served_mixed[0] <= served_mixed[1] // 2  # the last rounds may be the screened graph's job alone
