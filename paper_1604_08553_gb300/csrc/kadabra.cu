@@ -4592,8 +4592,9 @@ struct kadabra_graph {
   size_t tk_stage_cap = 0;           // entries
   struct TuneTable {  // autotuned setup by probe size class and allowed set (-1: not yet)
     int v[18][16];
+    uint32_t flags = 0;  // the launch flags of its probes; another set starts it anew
     TuneTable() { std::memset(v, 0xFF, sizeof(v)); }
-  } tier_choice;
+  } tier_choice, shared_choice;      // launches of its own; a batch's, tuned on this graph
   uint64_t fingerprint = 0;          // shape and sampled CSR entries (key of the autotuner's cache)
   // device-driven main loop of one-graph all-nodes runs (a CUDA graph), built on first use
   LoopCache loop;
@@ -5499,13 +5500,16 @@ namespace {
 // 65,536-sample batches as a loss (tails of a few samples per CTA), and one
 // of 16,384 picked either setup from run to run.
 constexpr uint64_t TUNE_PROBE = 65536;
-// process-wide: graphs with the same fingerprint, device and flags (a graph
-// loaded again) reuse the probe's choice; a collision could only cost speed
+// process-wide: graphs with the same fingerprint, device and launch flags (a
+// graph, or a batch, loaded again) reuse the probe's choice; a collision could
+// only cost speed
 std::mutex g_tune_mu;
 std::unordered_map<uint64_t, int> g_tune_cache;
 
+// flags, idle: the launches' flags and share of samples that end at a root
+// without arcs; shared: the launches are a batch's, g its largest graph.
 kadabra_status tier_variant(kadabra_graph* g, Workspace* w, cudaStream_t st, int32_t req_ctas, int32_t req_warp,
-                            uint64_t batch, int* variant) {
+                            uint64_t batch, uint32_t flags, double idle, bool shared, int* variant) {
   const uint64_t probe = std::max<uint64_t>(1, std::min<uint64_t>(batch, TUNE_PROBE));
   const int size_class = probe >= TUNE_PROBE ? 0 : 1 + ceil_log2(probe);  // <= 17
   const int per_default = w->grid_fast / w->num_sms, per_compact = w->grid_compact / w->num_sms;
@@ -5534,14 +5538,21 @@ kadabra_status tier_variant(kadabra_graph* g, Workspace* w, cudaStream_t st, int
     *variant = __builtin_ctz(allowed);
     return KADABRA_OK;
   }
-  int& choice = g->tier_choice.v[size_class][allowed];
+  kadabra_graph::TuneTable& table = shared ? g->shared_choice : g->tier_choice;
+  if (table.flags != flags) table = kadabra_graph::TuneTable();
+  table.flags = flags;
+  int& choice = table.v[size_class][allowed];
   if (choice >= 0) {
     *variant = choice;
     return KADABRA_OK;
   }
-  const uint64_t key = g->fingerprint ^ ((uint64_t)g->device << 56) ^ ((uint64_t)g->flags << 48) ^
-                       ((uint64_t)allowed << 40) ^ ((uint64_t)size_class << 32);
-  const bool cached = g->fingerprint != 0;  // graphs of a batch have none
+  // what else the probes' launches depend on
+  const bool screen = probe >= SCREEN_SAMPLES && idle >= SCREEN_MIN;
+  const uint64_t how = (flags & 127u) | ((uint64_t)(flags >> 29) << 7) | ((uint64_t)shared << 10) | ((uint64_t)screen << 11);
+  static_assert(KADABRA_FLAG_COMPACT_TABLES == 64 && FLAG_TINY_AUTO == 1u << 29, "the flags' bits in the key");
+  const uint64_t key = g->fingerprint ^ ((uint64_t)g->device << 56) ^ (how << 44) ^ ((uint64_t)allowed << 40) ^
+                       ((uint64_t)size_class << 32);
+  const bool cached = g->fingerprint != 0;
   if (cached) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
@@ -5551,9 +5562,9 @@ kadabra_status tier_variant(kadabra_graph* g, Workspace* w, cudaStream_t st, int
     }
   }
   KTRY(ensure_ws(w, probe, 1));
-  SampleParams P = ws_params(w, launch_flags(g));
+  SampleParams P = ws_params(w, flags);
   P.total_work = probe;
-  choose_screen(P, probe, g->idle * probe);
+  choose_screen(P, probe, idle * (double)probe);
   std::memset(&P.job0, 0, sizeof(Job));
   P.job0.g = graph_dev(g);
   P.job0.seed = 0x5EEDu;
@@ -5606,7 +5617,7 @@ kadabra_status tier_variant(kadabra_graph* g, Workspace* w, cudaStream_t st, int
 int tuned_variant(const kadabra_graph* g, uint64_t batch) {
   const uint64_t probe = std::max<uint64_t>(1, std::min<uint64_t>(batch, TUNE_PROBE));
   const int size_class = probe >= TUNE_PROBE ? 0 : 1 + ceil_log2(probe);
-  const int v = g->tier_choice.v[size_class][15];
+  const int v = g->tier_choice.flags == launch_flags(g) ? g->tier_choice.v[size_class][15] : -1;
   return v >= 0 ? v : 0;
 }
 
@@ -5828,15 +5839,27 @@ kadabra_status run_graphs(Workspace* w, kadabra_graph* const* gs, int G, const d
     cudaError_t e_ = (call);                                                              \
     if (e_ != cudaSuccess) return fail(KADABRA_ERR_CUDA, cudaGetErrorString(e_));         \
   } while (0)
+  // one graph: its flags.  Several share the launch: the small layout if every
+  // graph allows it, and what SHARED_LAUNCH_FLAGS has of any graph.
+  uint32_t fl = launch_flags(gs[0]);
+  if (G > 1) {
+    fl = FLAG_TINY_AUTO;
+    for (int i = 0; i < G; ++i) fl &= launch_flags(gs[i]);
+    for (int i = 0; i < G; ++i) fl |= launch_flags(gs[i]) & SHARED_LAUNCH_FLAGS;
+  }
   // The tier-S setup of the launches: autotuned on the graph (one-graph
-  // runs), or on the batch's largest graph, whose samples take most of each
-  // shared launch (it changes no result).
+  // runs), or with the shared flags on the batch's largest graph, whose
+  // samples take most of each shared launch (it changes no result).
   int variant = 0;
   {
     int big = 0;
-    for (int i = 1; i < G; ++i)
+    double idle_k = 0.0;
+    for (int i = 0; i < G; ++i) {
       if (gs[i]->m > gs[big]->m) big = i;
-    KTRY(tier_variant(gs[big], w, st, cfg.ctas_per_sm, cfg.warp_tier, std::min(S[big].K, S[big].cap), &variant));
+      idle_k += gs[i]->idle * (double)std::min(S[i].K, S[i].cap);
+    }
+    KTRY(tier_variant(gs[big], w, st, cfg.ctas_per_sm, cfg.warp_tier, std::min(S[big].K, S[big].cap), fl,
+                      idle_k / (double)sum_k, G > 1, &variant));
     for (int i = 0; i < G; ++i) {
       out[i].ctas_per_sm = variant_ctas_per_sm(w, variant);
       out[i].warp_tier = variant >> 1;
@@ -5848,13 +5871,6 @@ kadabra_status run_graphs(Workspace* w, kadabra_graph* const* gs, int G, const d
     RCK(cudaMemsetAsync(s.g->counts, 0, sizeof(uint32_t) * s.g->n, st));
   }
   std::vector<Job> jobs;
-  // one graph: its flags; several share the launch: only the warp tier, if
-  // any of them asks for it (it changes no result)
-  uint32_t fl = G == 1 ? launch_flags(gs[0]) : 0;
-  if (G > 1)
-    fl = FLAG_TINY_AUTO;
-    for (int i = 0; i < G; ++i) fl &= launch_flags(gs[i]);
-    for (int i = 0; i < G; ++i) fl |= launch_flags(gs[i]) & SHARED_LAUNCH_FLAGS;
   double idle = 0.0;  // of the jobs' samples: expected to end at a root without arcs
   auto launch_jobs = [&]() -> kadabra_status {
     uint64_t work = 0;
@@ -6277,7 +6293,7 @@ kadabra_status run_topk(kadabra_graph* g, double lambda, double delta, int32_t k
   RCK(cudaMemsetAsync(g->count0, 0, sizeof(uint32_t) * n, st));
   RCK(cudaMemsetAsync(g->counts, 0, sizeof(uint32_t) * n, st));
   int variant = 0;
-  KTRY(tier_variant(g, w, st, cfg.ctas_per_sm, cfg.warp_tier, K, &variant));
+  KTRY(tier_variant(g, w, st, cfg.ctas_per_sm, cfg.warp_tier, K, launch_flags(g), g->idle, false, &variant));
   r.ctas_per_sm = variant_ctas_per_sm(w, variant);
   r.warp_tier = variant >> 1;
   auto job = [&](uint32_t domain, uint64_t first, uint64_t count, uint32_t* counts) {
@@ -6900,7 +6916,7 @@ kadabra_status srv_round(kadabra_server* S, std::vector<SrvJob*>& act, std::vect
   }
   Workspace* w = S->ws.get();
   KTRY(ensure_ws(w, work, (int)jobs.size()));
-  uint32_t fl = 0;  // the warp tier, if any job's graph asks for it (it changes no result)
+  uint32_t fl = 0;  // the warp tier and the row searches, if any job's graph takes them (they change no result)
   for (SrvJob* J : act) fl |= launch_flags(J->g) & SHARED_LAUNCH_FLAGS;
   SampleParams P = ws_params(w, fl);
   P.total_work = work;

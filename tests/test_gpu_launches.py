@@ -85,3 +85,30 @@ print(json.dumps([batch(rmat, 16384), batch(rmat[:1], 1000), batch(rmat[:1] + ba
     assert alone[0] > 0 and most[0] > 0 and served[0] > 0
     assert few[0] == 0 and mixed[0] == 0
     assert served_mixed[0] <= served_mixed[1] // 2  # the last rounds may be the screened graph's job alone
+
+
+def test_batch_tunes_the_layout_it_runs():
+    """A batch's setup is timed with the launches the batch makes: the small
+    layout only if all its graphs are small, and whatever a run on the probed
+    graph alone has chosen before."""
+    small, large, alone, large_again = _child("""
+dense = gg.erdos_renyi(8000, 100.0, 1)   # the most arcs, few nodes
+wide = gg.erdos_renyi(20000, 8.0, 2)
+tiny, compact = "k_sample<0, 2", "k_sample<0, 1"
+def batch(graphs):
+    B = kd.Batch(graphs)
+    c = count(lambda: B.run([0.05] * len(graphs), [0.1] * len(graphs), [1] * len(graphs)), tiny, compact)
+    return B, c
+S, small = batch([dense, dense])
+L, large = batch([dense, wide])
+alone = count(lambda: kd.kadabra_run(L.views[0], 0.05, 0.1, 0, 1, check_interval=1024), tiny, compact)
+for B in (S, L):
+    B.free()
+L, again = batch([dense, wide])
+L.free()
+print(json.dumps([small, large, alone, again]))
+""")
+    assert small[0] > 0 and small[1] == 0
+    assert large[0] == 0 and large[1] > 0
+    assert alone[0] > 0 and alone[1] == 0
+    assert large_again[0] == 0 and large_again[1] <= large[1]  # tuned before
