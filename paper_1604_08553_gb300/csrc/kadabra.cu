@@ -1271,7 +1271,7 @@ KD_MEMB_ATTR void search_long_rows(const Tables& T, const Ctl<NW>& c, const int3
         py[h] = lpos_get<PK>(T, ob + yi);
         hy[h] = T.hkv[KIDX(py[h], T.hmask + 1u, 14)];
         y[h] = (int32_t)(hy[h] >> 32);
-        a[h] = T.lr->start[r[h]];
+        a[h] = T.lr->start[KIDX(r[h], LONG_CAP, 16)];
         e[h] = a[h] + T.lr->deg[r[h]];
       }
     }
@@ -1349,7 +1349,6 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
     // (shared-memory tiers, one segment), then to T.pi, at their running index.
     cand_at = (fcount + 2) & ~1;
     cand_cap = PK && nseg == 1 ? max(0, T.frcap + 1 - cand_at) / 2 : 0;
-    PiEntry* const cand = reinterpret_cast<PiEntry*>(T.pr + cand_at);
 
     // Degree prefix and row starts over frontier nodes [fb, fb + cnt) into
     // T.pr.  A frontier of more than T.frcap nodes is scanned in segments of
@@ -1364,7 +1363,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
       if (RG && row_is_long(deg, kl)) {
         const int q = atomicAdd(&c.nlong, 1);
         if (q < long_cap) {
-          T.lr->pos[q] = (uint16_t)seg_pos;
+          T.lr->pos[KIDX(q, LONG_CAP, 16)] = (uint16_t)seg_pos;
           T.lr->start[q] = rs;
           T.lr->deg[q] = deg;
           deg = 0;
@@ -1377,7 +1376,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
         if (wid == 0) {
           int deg = 0, rs = 0;
           if (lane < cnt) {
-            const int2 b = c.fr[side][lane];  // the rows' bounds, kept when the nodes were inserted
+            const int2 b = c.fr[side][KIDX(lane, 32, 17)];  // the rows' bounds, kept when the nodes were inserted
             rs = b.x;
             deg = take_long(b.y, kl, lane, rs);
           }
@@ -1438,10 +1437,10 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
         e.x = (int32_t)(hx >> 32);
         e.y = y;
         e.w = sx * sy;
-        if (at < cand_cap)
-          cand[at] = e;
+        if (at < cand_cap)  // entries cand_at + 2 at and the next one of T.pr
+          *reinterpret_cast<PiEntry*>(T.pr + (KIDX(cand_at + 2 * at + 1, T.frcap + 1, 18) - 1)) = e;
         else if (at < pi_cap)
-          T.pi[at] = e;
+          T.pi[KIDX(at, pi_cap, 15)] = e;
       }
     };
 
@@ -1562,7 +1561,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
                   if (!PK) T.lnode[at] = y;
                   lpos_set<PK>(T, at, pos);
                   cost += (unsigned)ydeg;
-                  if (at - list_before < 32) c.fr[side][at - list_before] = make_int2(ylo, ydeg);
+                  if (at - list_before < 32) c.fr[side][KIDX(at - list_before, 32, 17)] = make_int2(ylo, ydeg);
                   if (!PK && !ent_add<PK>(T, pos, add)) of = true;
                 }
               }
