@@ -5,8 +5,9 @@
 // via Random Approximation".  The method (Alg. 1) samples shortest paths
 // between uniform node pairs and stops once every node's estimate b~(v) is
 // within lambda with probability 1-delta:
-//   * k_sample      -- one sample per CTA of 256 threads (Sec. 4): (s,t)
-//                      draw, balanced bidirectional BFS with exact uint64
+//   * k_sample      -- one sample per CTA (Sec. 4; 128 to 1,024 threads by
+//                      tier and layout): (s,t) draw, balanced
+//                      bidirectional BFS with exact uint64
 //                      sigma, candidate-edge choice proportional to
 //                      sigma_sv*sigma_wt, backtracking to a uniform shortest
 //                      path, hit counters (Alg. 1).
@@ -28,7 +29,8 @@
 //   * Both searches' visited sets share one open-addressing hash table in
 //     shared memory, one packed 64-bit word per node (node | side | depth |
 //     sigma); level lists hold 16-bit hash positions (the node id is in the
-//     hash word).  Four CTAs of 256 threads fit per SM.
+//     hash word).  Four CTAs of 256 threads fit per SM in the default layout,
+//     five of 192 and seven of 128 in the smaller ones, one of 1,024 in tier B.
 //   * Every level runs pass 1 (touch test against the other search; most
 //     arcs lie in the touching level, which only reads the table, and a bit
 //     filter of the other side's frontier rejects most heads before the
@@ -43,10 +45,10 @@
 //     For graphs beyond the L2, pass 1 searches long rows instead.
 //     Candidate edges are chosen in (x, y) order without a sort (quadratic
 //     ranking or a weighted radix selection).
-//   * The kernel is short of issue slots and instruction cache, not of
+//   * The kernel is short of issue slots and instruction fetch, not of
 //     bandwidth: loops of the sampler are not unrolled unless it says so
-//     (130 KB of code against 72 KB; 128 KB of instruction cache per SM), and
-//     what one thread does while the others wait is kept short.
+//     (130 KB of code against 72 KB: the Chung-Lu graph's batch 4.50 -> 3.87
+//     ms), and what one thread does while the others wait is kept short.
 //   * A sample that outgrows its table moves on to bigger tables (tier B in
 //     shared memory, then global-memory tiers M and L) with identical
 //     results.
@@ -98,25 +100,21 @@ namespace {
 #ifndef KD_NT_BIG
 #define KD_NT_BIG 1024
 #endif
-// Warps per sampler CTA: tiers S and L, and tier B (with M), whose samples are
-// few and large, so that a sample's latency counts: 32 warps on one CTA per
-// SM with 16,384 slots.  Its launch per batch, against 8 warps on two CTAs
-// with 8,192 slots, 16 on two, and 24 on one CTA: ER 3.4 M nodes (1,100
-// samples) 0.83, 0.57, 0.26 -> 0.25 ms, Chung-Lu 10^6 nodes (65,536) 0.47,
-// 0.35, 0.19 -> 0.19 ms, R-MAT scale 24 (65,536) 2.28, 1.62, 1.30 -> 1.22 ms:
-// fewer samples go on to tier M, and a level's arcs take fewer steps.
-// The compact tier-S layout: 6 warps, which leaves five CTAs per SM 64 registers
-// a thread and so the fused pass; with 8 warps (48 registers) it spilled.
-// 65,536 samples with 8 warps, with 6, and in the default layout: Chung-Lu of
-// 10^5 nodes 2.07, 1.57, 1.73 ms, of 10^6 nodes 3.45, 2.97, 2.95 ms; 8,192 of
-// ER 2,000 nodes 266, 188, 214 us; 16,384 of BA 300,000 nodes 800, 656, 713 us.
-// The small tier-S layout, the compact one's place on graphs of few nodes: 4
-// warps, 2048 slots, seven CTAs per SM, so that a batch of 1,000 samples runs at
-// once and a sample's barriers join fewer warps.  Runs at K near 1,000 with the
-// compact layout and with it: ER of 2,000 nodes 1.02 -> 0.91 ms, of 8,000 1.14 ->
-// 1.01, of 32,000 1.28 -> 1.28; Chung-Lu of 4,000 nodes 0.98 -> 0.91, of 16,000
-// 1.24 -> 1.24; BA of 4,000 nodes 1.67 -> 1.51, of 16,000 1.60 -> 1.60; ER of 3.4 M
-// nodes 7.9 -> 8.4 ms, hence TINY_NODES.  Eight CTAs per SM, or 3 warps: the same.
+// Warps per sampler CTA.  Tiers S and L: 8.
+// Tier B (with M): 32 on one CTA per SM with 16,384 slots, since its samples are
+// few and large, so that a sample's latency counts.  Its launch per batch,
+// against 8 warps on two CTAs with 8,192 slots: ER 3.4 M nodes (1,100 samples)
+// 0.83 -> 0.25 ms, R-MAT scale 24 (65,536) 2.28 -> 1.22 ms.
+// The compact tier-S layout: 6, which leaves five CTAs per SM 64 registers a
+// thread; with 8 warps (48 registers) it spilled: 65,536 samples on the
+// Chung-Lu graph of 10^6 nodes 3.45 -> 2.97 ms.
+// The small tier-S layout, the compact one's place on graphs of few nodes: 4,
+// with 2048 slots and seven CTAs per SM, so that a batch of 1,000 samples runs
+// at once and a sample's barriers join fewer warps.  The line: runs at K near
+// 1,000 with the compact layout and with it, ER of 2,000 nodes 1.02 -> 0.91 ms,
+// of 8,000 1.14 -> 1.01, of 32,000 1.28 -> 1.28, of 3.4 M 7.9 -> 8.4.  On dense
+// graphs of 4,000 to 16,000 nodes (mean degree 40 to 800) the compact layout was
+// at most 2 % ahead of the better of the small and the default one.
 constexpr int NW_S = KD_NT / 32;
 constexpr int NW_CMP = 6;
 constexpr int NW_TINY = 4;
@@ -461,7 +459,6 @@ struct SampleParams {
   int gm_lcap;
 };
 
-// per-CTA control block in shared memory
 // Long rows of a level (the scan variant for graphs beyond the L2 only).
 // Every arc that can touch joins the two current frontiers, so a frontier
 // row x of deg arcs holds a touch arc for each node of the other frontier
@@ -506,6 +503,7 @@ struct LongRows {
   uint16_t pos[LONG_CAP];              // position in the frontier segment
 };
 
+// per-CTA control block in shared memory
 template <int NW>
 struct Ctl {
   Job job;        // the job of the current sample
@@ -847,8 +845,7 @@ __device__ __forceinline__ void rows_of_step(const Tables& T, int pcur, int fcou
 // one window at a time, took 23.2 k of 74 k cycles per sample on the Chung-Lu
 // graph of 10^6 nodes; this takes 16 k of 57 k.  Run twice, it adds 36 % to a
 // batch's instructions and 35 % to its time; without the branches around each
-// filter test a batch of 65,536 went 2.97 -> 2.85 ms.  Queueing the heads that
-// pass the filter and probing them 32 at a time changed nothing (2.96 -> 3.01).
+// filter test a batch of 65,536 went 2.97 -> 2.85 ms.
 template <bool PK, int D, int NW, class EM>
 __device__ __forceinline__ void touch_pass(const Tables& T, int side, int fcount, int E, const int32_t* cols,
                                            int64_t ncols, EM emit) {
@@ -2089,12 +2086,8 @@ struct SLayout {
 };
 // tier S at KD_MIN_BLOCKS CTAs per SM; tier S compact (one more CTA per SM:
 // half-full lists, 512-node segments, a 2^14-bit filter, 38 levels per
-// side; 5 x 45,408 B fit an SM's shared memory, 5 x 45,600 B did not);
-// tier B (four times the slots, one CTA per SM).  Tier B with frontier segments
-// of 2048 or 4096 nodes and a 2^16- or 2^17-bit filter: 2 to 5 % faster on the
-// ER graph of 3.4 M nodes, 8 % slower on the Chung-Lu graph, up to 30 % on
-// R-MAT scale 22.  Tier S with half-full lists: its own launch 4 to 30 % faster,
-// the batch 0 to 7 % slower, since more samples are begun twice.
+// side; 45,328 B, of which five fit an SM's shared memory up to 45,408 B);
+// tier B (four times the slots, one CTA per SM); the small layout.
 #ifndef KD_CMP_L8
 #define KD_CMP_L8 4
 #endif
