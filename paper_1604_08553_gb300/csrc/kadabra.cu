@@ -1598,10 +1598,11 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
       const int lf = (of ? LF_SIGMA : 0) | (cap ? LF_CAP : 0) | (sigma_of ? LF_TOUCH_SIGMA : 0);
       if (lf) atomicOr(&c.lvl_flags, lf);
       __syncthreads();
-      if (PK && (c.lvl_flags & LF_CAP)) {
-        // A packed sigma that ran out of its bits has carried into its entry's
-        // depth and side, so a one-pass level's touches may be false: the next
-        // tier takes the sample, touch or not.
+      if (PK && c.lvl_flags) {
+        // (Packed levels only run out of room.)  A sigma that ran out of its
+        // bits has carried into its entry's depth and side, so a one-pass
+        // level's touches may be false: the next tier takes the sample, touch
+        // or not.
         if (tid == 0) c.flags |= F_CAP;
         return;
       }
@@ -1623,7 +1624,7 @@ __device__ __forceinline__ void run_sample(const SampleParams& P, const Job& J, 
       if (tid == 0 && last >= 0) lvl_hi(T, last, last == 0 ? depth0 : depth1) = list_before;
       break;
     }
-    const int lf = c.lvl_flags, nl = c.nlist;
+    const int lf = PK ? 0 : c.lvl_flags, nl = c.nlist;
     if (lf) {
       if (tid == 0) c.flags |= ((lf & LF_SIGMA) ? F_SIGMA : 0) | ((lf & LF_CAP) ? F_CAP : 0);
       return;
