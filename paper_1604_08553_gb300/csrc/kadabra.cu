@@ -3604,7 +3604,7 @@ __global__ void __launch_bounds__(256) k_validate_arcs(const int32_t* rp, const 
 // not L2-resident cost HBM one sector each.  The mirror test of R-MAT scale 24
 // (263 M arcs): binary search 32 to 33 ms (one, two or four searches per lane
 // at once), binary over every 32nd entry first 15.6, this tree 9.6 ms (L1 at
-// 72 %, L2 61 %, issue 59 % on scale 22); with a last block of 16 or 32
+// 68 %, L2 62 %, issue 59 % on scale 22); with a last block of 16 or 32
 // entries (TREE_SHIFT 4, 5) 11.6, 14.0 ms.  Graphs within the L2 have no
 // tree: building it costs more than it saves (Chung-Lu 10^6 nodes 0.18 -> 0.23 ms).
 #ifndef KD_TREE_SHIFT
