@@ -34,7 +34,7 @@ count(lambda: torch.zeros(8, device="cuda") + 1, "x")  # the first profile of a 
 def _child(code):
     out = subprocess.run([sys.executable, "-c", PRELUDE + code, ROOT], capture_output=True, text=True, timeout=300)
     assert out.returncode == 0, out.stderr[-3000:]
-    return json.loads(out.stdout.strip().splitlines()[-1])
+    return json.loads([x for x in out.stdout.splitlines() if x.startswith("[")][-1])
 
 
 def test_loop_graph_serves_every_interval():
