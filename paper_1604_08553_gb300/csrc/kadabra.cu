@@ -145,6 +145,7 @@ constexpr int GM_MAXD = 65534;     // tier L, global memory, hash >= 2n slots, l
 constexpr int PI_SEGS = 16;        // a sample's candidate edges: PI_SEGS * pcap entries in global memory,
 constexpr int FAST_PCAP = 2048;    //   pcap in tiers S, B and M
 constexpr int QUAD_PICK_MAX = 256;  // global-memory tiers: candidate sets ranked quadratically up to this size
+constexpr size_t RADIX_HIST = 256 * (sizeof(unsigned long long) + sizeof(unsigned));  // larger sets: the selection's histogram
 constexpr unsigned long long EMPTY = ~0ull;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
@@ -2014,7 +2015,9 @@ __host__ __device__ inline size_t gm_layout(int hlog, int lcap, int maxd, size_t
                                             size_t* off_lpos, size_t* off_lvl) {
   size_t o = (2 * sizeof(unsigned long long)) << hlog;  // hkv, then hsig
   *off_pr = o;
-  o += sizeof(int2) * ((size_t)lcap + 1);
+  // the radix selection's histogram (RADIX_HIST) takes the frontier array, whatever the lists' capacity
+  const size_t frontier = sizeof(int2) * ((size_t)lcap + 1);
+  o += frontier > RADIX_HIST ? frontier : RADIX_HIST;
   *off_lnode = o;
   o += sizeof(int32_t) * (size_t)lcap;
   *off_lpos = o;
@@ -2082,7 +2085,7 @@ struct SLayout {
   static constexpr size_t BYTES = LONG + (LR ? sizeof(LongRows) : 0);
   static_assert(HLOG <= 16, "16-bit list positions");
   // the radix selection's histogram (256 u64 + 256 u32) in the frontier array
-  static_assert(sizeof(int2) * (FRCAP + 1) >= 256 * (sizeof(unsigned long long) + sizeof(unsigned)),
+  static_assert(sizeof(int2) * (FRCAP + 1) >= RADIX_HIST,
                 "frontier array holds the selection histogram");
 };
 // tier S at KD_MIN_BLOCKS CTAs per SM; tier S compact (one more CTA per SM:
